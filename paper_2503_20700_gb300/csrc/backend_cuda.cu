@@ -2,7 +2,8 @@
 //
 // Kernels:
 //   place_kernel        C += sum_s alpha_s op(S_s)            (HBM-bound block copies)
-//   gemm_f64_kernel     C += sum_s alpha_s op(A_s) op(B_s)    (FP64 reference path, DFMA)
+//   gemm_f64_kernel     C += sum_s alpha_s op(A_s) op(B_s)    (FP64 on the FMA pipe: small blocks)
+//   gemm_digits_kernel (gemm_digits.cu)                        (FP64 as exact bf16 digit products on tcgen05)
 //   gemm_tf32x3 (gemm_split.cu)                                (split-FP32 tensor-core path)
 //   dots/combine/axpby  Davidson vector algebra (FP64, deterministic two-stage reductions)
 //   jacobi_smem_kernel  parallel cyclic Jacobi eigensolver (FP64) of one matrix in shared memory, one CTA
@@ -21,6 +22,7 @@
 #include <vector>
 
 #include "backend.hpp"
+#include "gemm_digits.cuh"
 #include "gemm_split.cuh"
 #include "hpsi_fused.cuh"
 #include "hpsi_tc.cuh"
@@ -723,6 +725,7 @@ class CudaBackend : public Backend {
     if (dflag) cudaFreeAsync(dflag, st);
     if (htask) cudaFreeHost(htask);
     cudaStreamSynchronize(st);
+    if (dig_err) cudaFreeHost(dig_err);
     cudaStreamDestroy(st);
   }
   std::string name() const override { return "cuda"; }
@@ -840,6 +843,7 @@ class CudaBackend : public Backend {
     if (b) {
       CK(cudaMemcpyAsync(d, s, b, cudaMemcpyDeviceToHost, st));
       CK(cudaStreamSynchronize(st));
+      check_digits();
     }
   }
   void sync() override { CK(cudaStreamSynchronize(st)); }
@@ -852,6 +856,10 @@ class CudaBackend : public Backend {
     return dflag;
   }
   void check_device_flag() override {
+    if (dig_err) {
+      CK(cudaStreamSynchronize(st));
+      check_digits();
+    }
     if (!dflag) return;
     int h = 0;
     CK(cudaMemcpyAsync(&h, dflag, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -952,18 +960,29 @@ class CudaBackend : public Backend {
       if (rec) CK(cudaEventRecord(rec->b, st));
       return;
     }
+    std::vector<char> digits;
+    const bool any = choose_digits(groups, segs, digits);
     std::vector<GemmTile> tiles;
     for (size_t gi = 0; gi < groups.size(); ++gi) {
       auto& g = groups[gi];
+      if (any && digits[gi]) continue;
       for (int r = 0; r < g.m; r += kTM)
         for (int c = 0; c < g.n; c += kTN) tiles.push_back({(int)gi, r, c, 0});
+    }
+    if (any) {
+      if (rec) CK(cudaEventRecord(rec->a, st));
+      gemm_digits(groups, segs, digits);
+      if (tiles.empty()) {
+        if (rec) CK(cudaEventRecord(rec->b, st));
+        return;
+      }
     }
     std::vector<size_t> off;
     char* d = upload({{groups.data(), groups.size() * sizeof(GemmGroup)},
                       {segs.data(), segs.size() * sizeof(GemmSeg)},
                       {tiles.data(), tiles.size() * sizeof(GemmTile)}},
                      off);
-    if (rec) CK(cudaEventRecord(rec->a, st));
+    if (rec && !any) CK(cudaEventRecord(rec->a, st));
     // grid.x is limited to 2^31-1; task lists stay far below
     gemm_f64_kernel<<<(unsigned)tiles.size(), 256, 0, st>>>((const GemmGroup*)(d + off[0]),
                                                              (const GemmSeg*)(d + off[1]),
@@ -971,6 +990,114 @@ class CudaBackend : public Backend {
     ++launches;
     CK(cudaGetLastError());
     if (rec) CK(cudaEventRecord(rec->b, st));
+  }
+
+  // Which float64 groups go to the digit products (gemm_digits.cuh): those
+  // whose modelled tensor time is below their time on the FMA pipe, if that
+  // saves more than the two extra launches of the split (kDigLaunchClocks).
+  // The choice depends on the list's shapes only.
+  static constexpr double kDigLaunchClocks = 25000.0;
+  bool choose_digits(const std::vector<GemmGroup>& groups, const std::vector<GemmSeg>& segs,
+                     std::vector<char>& digits) const {
+    double df = 0.0, dd = 0.0, tf = 0.0, td = 0.0;
+    bool any = false;
+    digits.assign(groups.size(), 0);
+    for (size_t i = 0; i < groups.size(); ++i) {
+      const GemmGroup& g = groups[i];
+      if (g.m <= 0 || g.n <= 0 || g.seg_count <= 0) continue;
+      const DigCost c = dig_cost(g, segs.data());
+      if (c.digits >= c.fma) continue;
+      digits[i] = 1;
+      any = true;
+      df += c.fma;
+      dd += c.digits;
+      tf = std::max(tf, c.fma_tile);
+      td = std::max(td, c.digits_tile / dig_parts(g, segs.data()));
+    }
+    return any && std::max(dd / sms, td) + kDigLaunchClocks < std::max(df / sms, tf);
+  }
+  // Digit pool of one launch (bytes): groups are taken until their operands
+  // reach it (a single larger group still runs whole).  The pool is work
+  // space like the task lists: it is outside the context's budget, so under a
+  // budget it is kept to a sixteenth of it.
+  size_t dig_pool_cap() const {
+    const size_t cap = size_t(2) << 30;
+    return budget_ ? std::max<size_t>(size_t(16) << 20, std::min(cap, budget_ / 16)) : cap;
+  }
+  int* dig_err = nullptr;  // host-mapped: set by a digit launch whose wait ran out
+  void check_digits() {
+    if (dig_err && *(volatile int*)dig_err) {
+      *dig_err = 0;
+      throw std::runtime_error("timeout: a bounded wait in the digit GEMM ran out");
+    }
+  }
+  void gemm_digits(const std::vector<GemmGroup>& groups, const std::vector<GemmSeg>& segs,
+                   const std::vector<char>& digits) {
+    if (!dig_err) {
+      CK(cudaHostAlloc((void**)&dig_err, sizeof(int), cudaHostAllocMapped));
+      *dig_err = 0;
+    }
+    DigPlanner pl;
+    const size_t cap = dig_pool_cap();
+    for (size_t i = 0; i < groups.size(); ++i) {
+      if (!digits[i]) continue;
+      pl.add(groups[i], segs.data(), dig_parts(groups[i], segs.data()));
+      if (pl.pool_bytes() < cap) continue;
+      run_digits(pl.plan);
+      pl.clear();
+    }
+    run_digits(pl.plan);
+  }
+  void run_digits(DigPlan& p) {
+    if (p.tasks.empty()) return;
+    // longest tasks first, dealt round-robin over the persistent CTAs
+    std::vector<double> w(p.tasks.size());
+    std::vector<int> order(p.tasks.size());
+    for (size_t t = 0; t < p.tasks.size(); ++t) {
+      order[t] = (int)t;
+      for (int s = 0; s < p.tasks[t].seg_count; ++s)
+        w[t] += std::max(64, p.ops[p.segs[p.tasks[t].seg_begin + s].a].k);
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return w[a] > w[b]; });
+    std::vector<DigTask> tasks(p.tasks.size());
+    for (size_t t = 0; t < tasks.size(); ++t) tasks[t] = p.tasks[order[t]];
+    auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
+    const size_t ox = al(p.pool_bytes()), ok = ox + al(p.nexp * sizeof(int));
+    const size_t osp = ok + al(p.nkmax * sizeof(uint2)), osc = osp + al(p.ops.size() * sizeof(int));
+    char* ws = nullptr;
+    const size_t bytes = osc + (size_t)p.scratch * sizeof(double);
+    if (cudaMallocAsync((void**)&ws, bytes, st) != cudaSuccess) {
+      cudaGetLastError();
+      throw std::runtime_error("out of device memory (" + std::to_string(bytes) + " bytes)");
+    }
+    CK(cudaMemsetAsync(ws + ok, 0, osc - ok, st));
+    std::vector<size_t> off;
+    char* d = upload({{p.ops.data(), p.ops.size() * sizeof(DigOperand)},
+                      {p.splits.data(), p.splits.size() * sizeof(DigSplit)},
+                      {p.segs.data(), p.segs.size() * sizeof(DigSeg)},
+                      {tasks.data(), tasks.size() * sizeof(DigTask)},
+                      {p.reds.data(), p.reds.size() * sizeof(DigReduce)}},
+                     off);
+    DigLaunch L{};
+    L.ops = (const DigOperand*)(d + off[0]);
+    L.splits = (const DigSplit*)(d + off[1]);
+    L.segs = (const DigSeg*)(d + off[2]);
+    L.tasks = (const DigTask*)(d + off[3]);
+    L.reds = (const DigReduce*)(d + off[4]);
+    L.nsplits = (int)p.splits.size();
+    L.ntasks = (int)tasks.size();
+    L.nreds = (int)p.reds.size();
+    L.nops = (int)p.ops.size();
+    L.pool = (unsigned char*)ws;
+    L.exps = (int*)(ws + ox);
+    L.kmax = (uint2*)(ws + ok);
+    L.special = (int*)(ws + osp);
+    L.scratch = (double*)(ws + osc);
+    L.err = dig_err;
+    L.sms = sms;
+    dig_launch(L, st);
+    launches += 2 + (L.nreds > 0);
+    CK(cudaFreeAsync(ws, st));
   }
 
   void hpsi(const HpsiBlock* blocks, const HpsiItem* items, const HpsiTask* tasks, int ntasks,

@@ -1,0 +1,149 @@
+// Float64 grouped GEMM on the bf16 tensor cores by exact digit products (the
+// error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59
+// (2012) 95, with one exponent per operand row and balanced base-256 digits).
+//
+//   C += sum_s alpha_s op_s(A_s) op_s(B_s)
+//
+// Row i of op(A) (column j of op(B)) has one exponent e with |x| < 2^e; every
+// entry becomes the integer F = round(x 2^(62-e)), cut into eight balanced
+// digits of eight bits (bf16 holds them exactly).  The products of digits i
+// and j with i + j = d are summed by tcgen05.mma into one FP32 accumulator
+// per d; 256 terms of an accumulator stay below 2^24.3, so the sums are exact
+// (above d = 4 a worst case of aligned digits may round in the last place, at
+// 2^-52 of the row maxima's product).  The 36 products with d <= 7 are kept;
+// what is dropped is below 2^-62 of the product of the row maxima per term,
+// under the rounding of a float64 FMA chain.  The accumulators are combined
+// in integers, and each segment is added to the output tile in float64.
+//
+// Operands whose scaling makes that bound useless are not multiplied by
+// digits but by float64 FMAs in the same kernel: a segment with a non-finite
+// entry, with a row maximum outside 2^+-400, or graded along k, that is, whose
+// largest product |a_ik b_kj| is more than 2^8 below the product of the
+// largest entries of A and B, or is so after every row is divided by its
+// maximum.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <cstdint>
+#include <unordered_map>
+#include <vector>
+
+#include "backend.hpp"
+
+namespace dmrg {
+
+constexpr int kDigTileM = 128, kDigTileN = 64;  // output tile of a task
+constexpr int kDigSlices = 8;
+constexpr int kDigUnit = 256;  // bytes: 8 rows x 16 columns of one digit
+
+// One operand: rows x k, element (r, c) = trans ? src[c ld + r] : src[r ld + c].
+// Digit s of rows [8g, 8g+8) x columns [16kb, 16kb+16) is unit
+// unit + (kb * 8 + s) * groups + g of the pool: two 8-row x 16-byte core
+// matrices (the canonical no-swizzle K-major layout), k fast.
+struct DigOperand {
+  const double* src;
+  long long unit;  // first unit in the pool
+  int rows, k, ld, trans;
+  int groups;      // ceil(rows / 8)
+  int eoff;        // row exponents: exps[eoff + r]
+  int koff;        // column maxima: kmax[koff + c]
+  int pad;
+};
+
+struct DigSeg {
+  int a, b;  // operands
+  double alpha;
+};
+
+// rows of an operand split by one CTA
+struct DigSplit {
+  int op, r0;
+};
+
+// A tile of an output block and a range of its segments.  part >= 0: the
+// task stores its sum as a partial tile (128 x 64 doubles) of the scratch.
+struct DigTask {
+  double* C;
+  long long part;
+  int m, n, ldc, r0, c0;
+  int seg_begin, seg_count, pad;
+};
+
+struct DigReduce {
+  double* C;
+  long long part0;
+  int m, n, ldc, r0, c0, nparts;
+};
+
+// Host lists of one launch sequence (split, products, reduction).
+struct DigPlan {
+  std::vector<DigOperand> ops;
+  std::vector<DigSplit> splits;
+  std::vector<DigSeg> segs;
+  std::vector<DigTask> tasks;
+  std::vector<DigReduce> reds;
+  long long units = 0;    // of the digit pool
+  long long scratch = 0;  // doubles of partial tiles
+  int nexp = 0, nkmax = 0;
+  size_t pool_bytes() const { return (size_t)units * kDigUnit; }
+};
+
+// Modelled SM clocks of one group by digit products and by the float64 FMA
+// kernel (64 x 64 tiles, two FMAs a clock and SM), and of their longest tile.
+struct DigCost {
+  double digits, fma, digits_tile, fma_tile;
+};
+DigCost dig_cost(const GemmGroup& g, const GemmSeg* segs);
+
+// Adds group g (its operands, shared ones once, and its tasks) to the plan.
+// Groups are added whole, so a plan's numbers do not depend on where a list
+// of groups is cut into plans.
+class DigPlanner {
+ public:
+  DigPlan plan;
+  void add(const GemmGroup& g, const GemmSeg* segs, int parts);
+  void clear();
+  size_t pool_bytes() const { return plan.pool_bytes(); }
+
+ private:
+  struct Key {
+    const double* p;
+    int rows, k, ld, trans;
+    bool operator==(const Key& o) const {
+      return p == o.p && rows == o.rows && k == o.k && ld == o.ld && trans == o.trans;
+    }
+  };
+  struct Hash {
+    size_t operator()(const Key& x) const {
+      uint64_t h = (uint64_t)(uintptr_t)x.p;
+      for (uint64_t v : {(uint64_t)x.rows, (uint64_t)x.k, (uint64_t)x.ld, (uint64_t)x.trans})
+        h = (h ^ v) * 0x9E3779B97F4A7C15ull, h ^= h >> 29;
+      return (size_t)h;
+    }
+  };
+  std::unordered_map<Key, int, Hash> seen_;
+  int operand(const double* p, int rows, int k, int ld, int trans);
+};
+
+// Partial sums a group is cut into (1: none), from its own shape alone.
+int dig_parts(const GemmGroup& g, const GemmSeg* segs);
+
+struct DigLaunch {
+  const DigOperand* ops;
+  const DigSplit* splits;
+  const DigSeg* segs;
+  const DigTask* tasks;
+  const DigReduce* reds;
+  int nsplits, ntasks, nreds, nops;
+  unsigned char* pool;
+  double* scratch;
+  int* exps;           // nexp
+  uint2* kmax;         // nkmax, zero at launch; exponents of the columns' largest entries,
+                       // of the rows divided by their maxima (x) and as they are (y); 0: a zero column
+  int* special;        // nops, zero at launch
+  int* err;            // host-mapped flag, set when a bounded wait ran out
+  int sms;
+};
+void dig_launch(const DigLaunch& L, cudaStream_t st);
+
+}  // namespace dmrg
