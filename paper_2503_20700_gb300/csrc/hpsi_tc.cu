@@ -836,52 +836,86 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   cluster_sync();
 }
 
-// partial tiles are TM x TNMAX float pairs stored column by column (element
-// (r, c) at c * TM + r); CTA (tile, y) sums columns [32 y, 32 y + 32) of a
-// tile over its chunks in fixed order, thread t taking row t % 128 of every
-// second column
-__global__ void hpsi_tc_reduce(const HpsiBlock* __restrict__ blocks, const HpsiReduce* __restrict__ reds,
-                               const double* __restrict__ scratch, int tile_n) {
+// Partial tiles are TM x TNMAX float pairs stored column by column (element
+// (r, c) at c * TM + r); CTA (tile, y, z) sums rows [32 z, 32 z + 32) x columns
+// [32 y, 32 y + 32) of a tile over its chunks in fixed order and adds them to
+// sigma.  Bound by HBM for long lists of chunks, by the latency of its loads
+// for the tiles of a sweep: so a CTA is 32 x 32, a lane holds one row of four
+// columns (256 B per warp and load, 16 loads in flight), sigma is fetched
+// before the sums and written row by row through shared memory.  Measured,
+// per launch: the products of a D = 256 sweep 227 -> 116 us, of a D = 512 bond
+// 392 -> 101 us (a CTA of 128 rows that walked its 32 columns two at a time and
+// wrote sigma by columns before).
+constexpr int RED = 32;
+__global__ void __launch_bounds__(256) hpsi_tc_reduce(const HpsiBlock* __restrict__ blocks,
+                                                      const HpsiReduce* __restrict__ reds,
+                                                      const double* __restrict__ scratch, int tile_n) {
+  __shared__ double turn[RED][RED + 1];
   const HpsiReduce rd = reds[blockIdx.x];
   const HpsiBlock bk = blocks[rd.block];
-  const int nvalid = min(tile_n, bk.n - rd.c0);
-  const int r = threadIdx.x & (TM - 1), gr = rd.r0 + r;
-  if (gr >= bk.m) return;
-  const int cend = min(nvalid, (int)blockIdx.y * 32 + 32);
-  for (int c = blockIdx.y * 32 + (int)(threadIdx.x >> 7); c < cend; c += 2) {
-    const float2* part = reinterpret_cast<const float2*>(scratch + rd.part0) + (size_t)c * TM + r;
-    double acc = 0.0;
-    for (int p = 0; p < rd.nparts; ++p) {
-      const float2 v = part[(long long)p * TM * TNMAX];
-      acc += (double)v.x + (double)v.y;
-    }
-    bk.C[(size_t)gr * bk.ldc + rd.c0 + c] += acc;
+  const int c0 = (int)blockIdx.y * RED, r0 = (int)blockIdx.z * RED;
+  const int nc = min(RED, min(tile_n, bk.n - rd.c0) - c0), nr = min(RED, bk.m - rd.r0 - r0);
+  if (nc <= 0 || nr <= 0) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double* const out = bk.C + (size_t)(rd.r0 + r0) * bk.ldc + rd.c0 + c0 + lane;
+  double old[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    old[i] = (warp + 8 * i < nr && lane < nc) ? out[(size_t)(warp + 8 * i) * bk.ldc] : 0.0;
+  const float2* part = reinterpret_cast<const float2*>(scratch + rd.part0) + (size_t)(c0 + warp) * TM + r0 + lane;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+  for (int p = 0; p < rd.nparts; ++p, part += (size_t)TM * TNMAX) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (lane < nr && warp + 8 * i < nc) {
+        const float2 v = __ldg(part + 8 * i * TM);
+        acc[i] += (double)v.x + (double)v.y;
+      }
   }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) turn[warp + 8 * i][lane] = acc[i];
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if (warp + 8 * i < nr && lane < nc) out[(size_t)(warp + 8 * i) * bk.ldc] = old[i] + turn[lane][warp + 8 * i];
 }
 
-// unit pairs of job j: pair p = kblock * G + g holds hi (unit 2p) and lo
-// (unit 2p + 1) of rows [8g, 8g + 8) x cols [32 kblock, 32 kblock + 32)
-__global__ void split_kernel(const SplitJob* __restrict__ jobs, int n, float* __restrict__ pool) {
-  for (int j = blockIdx.x; j < n; j += gridDim.x) {
-    const SplitJob jb = jobs[j];
-    const int G = (jb.rows + 7) >> 3;
-    const size_t pairs = (size_t)G * ((jb.cols + 31) >> 5);
-    float* const base = pool + (size_t)jb.unit * kTcUnitFloats;
-    for (size_t e = threadIdx.x; e < pairs * kTcUnitFloats; e += blockDim.x) {
-      const size_t pr = e / kTcUnitFloats;
-      const int w = (int)(e % kTcUnitFloats);
-      const int kbk = (int)(pr / G), g = (int)(pr % G);
-      const int r = 8 * g + ((w >> 2) & 7);
-      const int k = 32 * kbk + 4 * (w >> 5) + (w & 3);
-      double v = 0.0;
+// Unit pairs of job j: pair p = kblock * G + g holds hi (unit 2p) and lo
+// (unit 2p + 1) of rows [8g, 8g + 8) x cols [32 kblock, 32 kblock + 32).
+// Bound by HBM (8 B read and written per element).  A warp takes a pair: its
+// eight loads per lane cover whole 32-byte sectors in either orientation, its
+// stores 128 bytes each.  The pairs of a job are dealt over gridDim.y CTAs: a
+// few large operands would otherwise sit on as many SMs (one CTA per job).
+// Measured: 1066 us of a contraction of some 60 operands of 280..600 with one
+// CTA per operand (the whole call 3.17 -> 2.20 ms, 0.1 ms of it the reduction);
+// the operands of a D = 256 sweep 63 -> 40 us per launch, of a D = 512 bond
+// 51 -> 29 us.
+__global__ void __launch_bounds__(256) split_kernel(const SplitJob* __restrict__ jobs, float* __restrict__ pool) {
+  const SplitJob jb = jobs[blockIdx.x];
+  const int G = (jb.rows + 7) >> 3;
+  const int pairs = G * ((jb.cols + 31) >> 5);
+  const int lane = threadIdx.x & 31;
+  float* const base = pool + (size_t)jb.unit * kTcUnitFloats + lane;
+  for (int pr = blockIdx.y * 8 + (threadIdx.x >> 5); pr < pairs; pr += 8 * gridDim.y) {
+    const int kbk = pr / G, g = pr - kbk * G;
+    const int r = 8 * g + (lane >> 2), k0 = 32 * kbk + (lane & 3);
+    double v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = k0 + 4 * i;
+      v[i] = 0.0;
       if (r < jb.rows && k < jb.cols) {
-        if (jb.src == nullptr) v = (r == k) ? 1.0 : 0.0;
-        else v = jb.trans ? jb.src[(size_t)k * jb.ld + r] : jb.src[(size_t)r * jb.ld + k];
+        if (jb.src == nullptr) v[i] = (r == k) ? 1.0 : 0.0;
+        else v[i] = __ldg(jb.trans ? jb.src + (size_t)k * jb.ld + r : jb.src + (size_t)r * jb.ld + k);
       }
-      const float h = __uint_as_float(tf32((float)v));
-      float* u = base + pr * 2 * kTcUnitFloats;
-      u[w] = h;
-      u[kTcUnitFloats + w] = __uint_as_float(tf32((float)(v - (double)h)));
+    }
+    float* const u = base + (size_t)pr * 2 * kTcUnitFloats;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float h = __uint_as_float(tf32((float)v[i]));
+      u[32 * i] = h;
+      u[kTcUnitFloats + 32 * i] = __uint_as_float(tf32((float)(v[i] - (double)h)));
     }
   }
 }
@@ -919,7 +953,10 @@ void make_map(CUtensorMap* m, const void* pool, size_t units, int rows) {
 
 void split_launch(const SplitJob* jobs, int n, float* pool, cudaStream_t st) {
   if (n <= 0) return;
-  split_kernel<<<std::min(n, 152 * 8), 256, 0, st>>>(jobs, n, pool);
+  // CTAs per operand: 64 for a few (the split of a 600 x 600 block is then
+  // three pairs a warp), one from 64 operands per SM on
+  const int per = std::max(1, std::min(64, 152 * 64 / n));
+  split_kernel<<<dim3(n, per), 256, 0, st>>>(jobs, pool);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: split launch: ") + cudaGetErrorString(e));
 }
@@ -987,7 +1024,7 @@ void hpsi_tc_launch(const TcLaunch& L, int* err, unsigned long long wait_ns, cud
     if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: hpsi tc launch: ") + cudaGetErrorString(e));
   }
   if (L.nreds > 0) {
-    hpsi_tc_reduce<<<dim3(L.nreds, (L.tile_n + 31) / 32), 256, 0, st>>>(L.blocks, L.reds, L.scratch, L.tile_n);
+    hpsi_tc_reduce<<<dim3(L.nreds, (L.tile_n + RED - 1) / RED, TM / RED), 256, 0, st>>>(L.blocks, L.reds, L.scratch, L.tile_n);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: hpsi tc reduce: ") + cudaGetErrorString(e));
   }
