@@ -756,7 +756,7 @@ dmrg_status dmrg_hpsi_contract(const double* A, int64_t a_len, const double* P, 
       reds = tp.reds;
       scr = tp.scratch;
     } else {
-      scr = dmrg::hpsi_plan_tasks(hb, pr, tasks, reds);
+      scr = dmrg::hpsi_plan_tasks(hb, hi, pr, tasks, reds);
     }
     auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
     size_t ob = 0, oi = al(hb.size() * sizeof(dmrg::HpsiBlock));
@@ -843,13 +843,16 @@ dmrg_status dmrg_hpsi_contract_noalloc(const double* dA, int64_t a_len, const do
     const dmrg::Precision pr = precision == DMRG_FP64 ? dmrg::Precision::FP64 : dmrg::Precision::SPLIT_TF32;
     std::vector<dmrg::HpsiTask> tasks;
     std::vector<dmrg::HpsiReduce> reds;
-    size_t scr = dmrg::hpsi_plan_tasks(hb, pr, tasks, reds);
+    size_t nominal = 0;
+    dmrg::hpsi_plan_tasks(hb, hi, pr, tasks, reds, &nominal);
     auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
     size_t ob = 0, oi = al(hb.size() * sizeof(dmrg::HpsiBlock));
     size_t ot = al(oi + hi.size() * sizeof(dmrg::HpsiItem));
     size_t orr = al(ot + tasks.size() * sizeof(dmrg::HpsiTask));
     size_t os = al(orr + reds.size() * sizeof(dmrg::HpsiReduce));
-    size_t need = os + scr * sizeof(double);
+    // what the 64 x 64 tile plan takes (either plan's lists and partial tiles
+    // fit into it), so the capacity is that of the task lists above it
+    size_t need = ot + nominal;
     if (need > dmrg::kNoAllocScratchBytes)
       return fail(nullptr, DMRG_EINVAL,
                   "request needs " + std::to_string(need) + " bytes of scratch; the allocation-free entry "

@@ -1716,7 +1716,7 @@ void Engine::plan_hpsi(Block& Le, Block& Re, HPsiPlan& plan) {
     last_tc_cand_ = plan.tc_cand;
     have_tc_plan_ = true;
   } else {
-    scr = hpsi_plan_tasks(blocks, plan.prec, tasks, reds);
+    scr = hpsi_plan_tasks(blocks, items, plan.prec, tasks, reds);
   }
   const double tp2 = now_s();
   stats_.t_plan_tasks += tp2 - tp1;

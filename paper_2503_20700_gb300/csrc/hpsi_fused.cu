@@ -1,8 +1,10 @@
 // Fused H_eff psi kernels (see hpsi_fused.cuh).
+#include <algorithm>
 #include <stdexcept>
 #include <string>
 
 #include "hpsi_fused.cuh"
+#include "hpsi_noalloc.hpp"
 #include "kattr.hpp"
 
 namespace dmrg {
@@ -230,124 +232,221 @@ __global__ void __launch_bounds__(256) hpsi_tf32x3_kernel(const HpsiBlock* __res
 }
 
 // ---------------------------------------------------------------- FP64 variant
-// 16 x 16 threads, each owning a 4 x 4 register tile of the 64 x 64 tile
-__global__ void __launch_bounds__(256) hpsi_f64_kernel(const HpsiBlock* __restrict__ blocks,
-                                                       const HpsiItem* __restrict__ items,
-                                                       const HpsiTask* __restrict__ tasks,
-                                                       double* __restrict__ scratch) {
+// Bound by the float64 pipe (two FMAs a clock and SM: one warp-wide FMA is 16
+// clocks of it), so what counts is that no FMA is spent on padding or done
+// twice; shared memory and issue slots have room to spare.  A task's tile is
+// mt x nt with nt all of a block's columns (up to 256: stage 1, X = alpha
+// op(A) P, is then computed once, not once per column tile) and mt x nt at
+// most kF64Out; its outputs are dealt to the threads one by one, 128 at a
+// time, and so are those of X, so a 20 x 20 block costs 512 FMAs a k instead
+// of a padded 4096.  The two shared-memory reads per FMA this takes (one
+// broadcast, one along the lanes) are a quarter of the FMA's own time.  128
+// threads and 52 KB: four CTAs an SM hide each other's loads.
+// Measured against 64 x 64 tiles padded to their size: 367 -> 59 us a product
+// of a 10-site D = 64 run (blocks of 5..40), 6.82 -> 3.20 ms a whole call with
+// sectors of 40..208.
+constexpr int kF64Threads = 128;
+constexpr int kF64Slots = 16;                       // outputs per thread
+constexpr int kF64Out = kF64Threads * kF64Slots;    // outputs of a tile
+constexpr int kF64Cols = 256;                       // columns of a tile
+constexpr int kF64Rows = 128;                       // rows of a tile
+constexpr int kF64Chunk = 128;                      // columns of psi per X chunk
+constexpr int F64_A = kF64Rows * (KS + 1), F64_P = KS * kF64Chunk, F64_B = kF64Cols * (KS + 1);
+constexpr int F64_STAGE = F64_A + F64_P > F64_B ? F64_A + F64_P : F64_B;
+constexpr int F64_X = kF64Out + kF64Rows;           // rows of odd length
+constexpr size_t kF64Smem = (size_t)(F64_STAGE + F64_X) * sizeof(double);
+
+// rows and columns of the tiles of an m x n block
+__host__ __device__ inline void f64_tile(int m, int n, int& mt, int& nt) {
+  const int ct = (n + kF64Cols - 1) / kF64Cols;
+  nt = (n + ct - 1) / ct;
+  mt = kF64Out / nt;
+  if (mt > kF64Rows) mt = kF64Rows;
+  if (mt > m) mt = m;
+  const int rt = (m + mt - 1) / mt;
+  mt = (m + rt - 1) / rt;
+}
+// e / d and e % d of e < 2048, 1 <= d <= 256: the rounding of 2^20 / d is worth
+// less than 2^-9 of a quotient, a remainder at least 2^-8
+__device__ __forceinline__ int div_tile(int e, unsigned inv) { return (int)(((unsigned)e * inv) >> 20); }
+__device__ __forceinline__ unsigned inv_tile(int d) { return (unsigned)(((1 << 20) + d - 1) / d); }
+
+// acc[i] += sum_k a[row_i][k] b, row_i and the column's address from off[i]
+// (row part | column part << 16); b moves by bstep per k
+template <int NS>
+__device__ __forceinline__ void f64_products(double (&acc)[kF64Slots], const int (&off)[kF64Slots], const double* a,
+                                             const double* b, int bstep, int kn) {
+  for (int k = 0; k < kn; ++k, ++a, b += bstep) {
+#pragma unroll
+    for (int i = 0; i < NS; ++i) acc[i] = fma(a[off[i] & 0xFFFF], b[off[i] >> 16], acc[i]);
+  }
+}
+__device__ __forceinline__ void f64_products(int ns, double (&acc)[kF64Slots], const int (&off)[kF64Slots],
+                                             const double* a, const double* b, int bstep, int kn) {
+  switch (ns) {
+#define F64_CASE(N) \
+  case N: f64_products<N>(acc, off, a, b, bstep, kn); break
+    F64_CASE(1); F64_CASE(2); F64_CASE(3); F64_CASE(4); F64_CASE(5); F64_CASE(6); F64_CASE(7); F64_CASE(8);
+    F64_CASE(9); F64_CASE(10); F64_CASE(11); F64_CASE(12); F64_CASE(13); F64_CASE(14); F64_CASE(15); F64_CASE(16);
+#undef F64_CASE
+  }
+}
+
+__global__ void __launch_bounds__(kF64Threads, 4) hpsi_f64_kernel(const HpsiBlock* __restrict__ blocks,
+                                                                  const HpsiItem* __restrict__ items,
+                                                                  const HpsiTask* __restrict__ tasks,
+                                                                  double* __restrict__ scratch) {
   extern __shared__ double smd[];
-  double* As = smd;                 // [KS][T+1]   (k-major)
-  double* Ps = As + KS * (T + 1);   // [KS][T+1]
-  double* Bs = Ps + KS * (T + 1);   // [KS][T+1]   (k-major, n fast)
-  double* Xs = Bs + KS * (T + 1);   // [T][T+1]    (m rows, k fast)
+  double* const As = smd;          // [row][KS + 1]
+  double* const Ps = smd + F64_A;  // [k][kc]
+  double* const Bs = smd;          // [column][KS + 1]; shares the buffer with A and P
+  double* const Xs = smd + F64_STAGE;  // [row][kc | 1]
   const HpsiTask tk = tasks[blockIdx.x];
   const HpsiBlock bk = blocks[tk.block];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double s[4][4];
+  const int tid = threadIdx.x;
+  int tm, tn;
+  f64_tile(bk.m, bk.n, tm, tn);
+  const int nt = min(tn, bk.n - tk.c0);
+  // r0 < 0: one task walks all row tiles
+  const int r_begin = max(tk.r0, 0), r_end = tk.r0 < 0 ? bk.m : min(bk.m, tk.r0 + tm);
+  for (int r0 = r_begin; r0 < r_end; r0 += tm) {
+    const int mt = min(tm, bk.m - r0);
+    const int outs = mt * nt, ns = (outs + kF64Threads - 1) / kF64Threads;
+    const unsigned inv_n = inv_tile(nt);
+    double s[kF64Slots];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < kF64Slots; ++i) s[i] = 0.0;
+    for (int ii = tk.it_begin; ii < tk.it_begin + tk.it_count; ++ii) {
+      const HpsiItem it = items[ii];
+      int jc_begin = 0, jc_end = it.kb;
+      if (it.B == nullptr) {  // identity on the right: only sigma's own columns
+        jc_begin = tk.c0;
+        jc_end = min(it.kb, tk.c0 + nt);
+      }
+      const int step = min(kF64Chunk, kF64Out / mt);
+      for (int jc = jc_begin; jc < jc_end; jc += step) {
+        const int kc = min(step, jc_end - jc), ldx = kc | 1;
+        const unsigned inv_c = inv_tile(kc);
+        if (it.A == nullptr) {
+          for (int e = tid; e < mt * kc; e += kF64Threads) {
+            const int r = div_tile(e, inv_c), c = e - r * kc;
+            Xs[r * ldx + c] = r0 + r < it.ka ? it.alpha * it.P[(size_t)(r0 + r) * it.ldp + jc + c] : 0.0;
+          }
+        } else {
+          double x[kF64Slots];
+          int off[kF64Slots];
+          const int xouts = mt * kc, xs = (xouts + kF64Threads - 1) / kF64Threads;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) s[i][j] = 0.0;
-  for (int ii = tk.it_begin; ii < tk.it_begin + tk.it_count; ++ii) {
-    const HpsiItem it = items[ii];
-    int jc_begin = 0, jc_end = it.kb;
-    if (it.B == nullptr) {
-      jc_begin = tk.c0;
-      jc_end = min(it.kb, tk.c0 + T);
+          for (int i = 0; i < kF64Slots; ++i) {
+            const int e = tid + i * kF64Threads;
+            const int r = e < xouts ? div_tile(e, inv_c) : 0, c = e < xouts ? e - r * kc : 0;
+            x[i] = 0.0;
+            off[i] = r * (KS + 1) | c << 16;
+          }
+          for (int k0 = 0; k0 < it.ka; k0 += KS) {
+            const int kn = min(KS, it.ka - k0);
+            if (it.transA) {
+              for (int e = tid; e < mt * kn; e += kF64Threads) {
+                const int k = e / mt, r = e - k * mt;
+                As[r * (KS + 1) + k] = it.alpha * __ldg(it.A + (size_t)(k0 + k) * it.lda + r0 + r);
+              }
+            } else {
+              for (int e = tid; e < mt * KS; e += kF64Threads) {
+                const int r = e / KS, k = e % KS;
+                if (k < kn) As[r * (KS + 1) + k] = it.alpha * __ldg(it.A + (size_t)(r0 + r) * it.lda + k0 + k);
+              }
+            }
+            for (int e = tid; e < kn * kc; e += kF64Threads) {
+              const int k = div_tile(e, inv_c), c = e - k * kc;
+              Ps[e] = __ldg(it.P + (size_t)(k0 + k) * it.ldp + jc + c);
+            }
+            __syncthreads();
+            f64_products(xs, x, off, As, Ps, kc, kn);
+            __syncthreads();
+          }
+#pragma unroll
+          for (int i = 0; i < kF64Slots; ++i) {
+            const int e = tid + i * kF64Threads;
+            if (e < xouts) {
+              const int r = div_tile(e, inv_c);
+              Xs[r * ldx + e - r * kc] = x[i];
+            }
+          }
+        }
+        if (it.B == nullptr) {
+          // sigma's columns [jc, jc + kc) += X
+          __syncthreads();
+          const int c_off = jc - tk.c0;
+#pragma unroll
+          for (int i = 0; i < kF64Slots; ++i) {
+            const int e = tid + i * kF64Threads;
+            if (e < outs) {
+              const int r = div_tile(e, inv_n), c = e - r * nt - c_off;
+              if (c >= 0 && c < kc) s[i] += Xs[r * ldx + c];
+            }
+          }
+          __syncthreads();
+          continue;
+        }
+        int off[kF64Slots];
+#pragma unroll
+        for (int i = 0; i < kF64Slots; ++i) {
+          const int e = tid + i * kF64Threads;
+          const int r = e < outs ? div_tile(e, inv_n) : 0, c = e < outs ? e - r * nt : 0;
+          off[i] = r * ldx | (c * (KS + 1)) << 16;
+        }
+        for (int k0 = 0; k0 < kc; k0 += KS) {
+          const int kn = min(KS, kc - k0);
+          if (it.transB) {
+            for (int e = tid; e < nt * kn; e += kF64Threads) {
+              const int k = e / nt, c = e - k * nt;
+              Bs[c * (KS + 1) + k] = __ldg(it.B + (size_t)(jc + k0 + k) * it.ldb + tk.c0 + c);
+            }
+          } else {
+            for (int e = tid; e < nt * KS; e += kF64Threads) {
+              const int c = e / KS, k = e % KS;
+              if (k < kn) Bs[c * (KS + 1) + k] = __ldg(it.B + (size_t)(tk.c0 + c) * it.ldb + jc + k0 + k);
+            }
+          }
+          __syncthreads();
+          f64_products(ns, s, off, Xs + k0, Bs, 1, kn);
+          __syncthreads();
+        }
+      }
     }
-    for (int jc = jc_begin; jc < jc_end; jc += T) {
-      double x[4][4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) x[i][j] = 0.0;
-      if (it.A == nullptr) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            int gr = tk.r0 + ty + 16 * i, gc = jc + tx + 16 * j;
-            x[i][j] = (gr < bk.m && gr < it.ka && gc < jc_end) ? it.alpha * it.P[(size_t)gr * it.ldp + gc] : 0.0;
-          }
+    for (int i = 0; i < kF64Slots; ++i) {
+      const int e = tid + i * kF64Threads;
+      if (e >= outs) continue;
+      if (tk.part >= 0) {
+        scratch[tk.part + e] = s[i];
       } else {
-        for (int k0 = 0; k0 < it.ka; k0 += KS) {
-          for (int e = threadIdx.x; e < T * KS; e += 256) {
-            int r, c;
-            if (!it.transA) { r = e / KS; c = e % KS; }
-            else { c = e / T; r = e % T; }
-            int gr = tk.r0 + r, gk = k0 + c;
-            As[c * (T + 1) + r] = (gr < bk.m && gk < it.ka) ? it.alpha * ldA(it, gr, gk) : 0.0;
-          }
-          for (int e = threadIdx.x; e < T * KS; e += 256) {
-            int kk = e / T, n = e % T;
-            int gk = k0 + kk, gn = jc + n;
-            Ps[kk * (T + 1) + n] = (gk < it.ka && gn < jc_end) ? it.P[(size_t)gk * it.ldp + gn] : 0.0;
-          }
-          __syncthreads();
-#pragma unroll
-          for (int kk = 0; kk < KS; ++kk) {
-            double a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk * (T + 1) + ty + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Ps[kk * (T + 1) + tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-              for (int j = 0; j < 4; ++j) x[i][j] = fma(a[i], b[j], x[i][j]);
-          }
-          __syncthreads();
-        }
-      }
-      if (it.B == nullptr) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) s[i][j] += x[i][j];
-        continue;
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) Xs[(ty + 16 * i) * (T + 1) + tx + 16 * j] = x[i][j];
-      __syncthreads();
-      for (int k0 = 0; k0 < T && jc + k0 < jc_end; k0 += KS) {
-        for (int e = threadIdx.x; e < T * KS; e += 256) {
-          int n, kk;
-          if (!it.transB) { n = e / KS; kk = e % KS; }
-          else { kk = e / T; n = e % T; }
-          int gn = tk.c0 + n, gk = jc + k0 + kk;
-          Bs[kk * (T + 1) + n] = (gn < bk.n && gk < jc_end) ? ldB(it, gn, gk) : 0.0;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < KS; ++kk) {
-          double a[4], b[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) a[i] = Xs[(ty + 16 * i) * (T + 1) + k0 + kk];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) b[j] = Bs[kk * (T + 1) + tx + 16 * j];
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) s[i][j] = fma(a[i], b[j], s[i][j]);
-        }
-        __syncthreads();
+        const int r = div_tile(e, inv_n);
+        bk.C[(size_t)(r0 + r) * bk.ldc + tk.c0 + e - r * nt] += s[i];
       }
     }
   }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int r = ty + 16 * i, c = tx + 16 * j;
-      if (tk.part >= 0) {
-        scratch[tk.part + r * T + c] = s[i][j];
-      } else {
-        int gr = tk.r0 + r, gc = tk.c0 + c;
-        if (gr < bk.m && gc < bk.n) bk.C[(size_t)gr * bk.ldc + gc] += s[i][j];
-      }
-    }
+}
+
+// C += the partial tiles of a sigma tile, in a fixed order: bound by the
+// latency of its loads, so a thread has one output and eight partials in flight
+__global__ void __launch_bounds__(128) hpsi_f64_reduce_kernel(const HpsiBlock* __restrict__ blocks,
+                                                              const HpsiReduce* __restrict__ reds,
+                                                              const double* __restrict__ scratch) {
+  const HpsiReduce rd = reds[blockIdx.x];
+  const HpsiBlock bk = blocks[rd.block];
+  int tm, tn;
+  f64_tile(bk.m, bk.n, tm, tn);
+  const int nt = min(tn, bk.n - rd.c0), outs = min(tm, bk.m - rd.r0) * nt;
+  const int e = blockIdx.y * 128 + threadIdx.x;
+  if (e >= outs) return;
+  double* const c = bk.C + (size_t)(rd.r0 + e / nt) * bk.ldc + rd.c0 + e % nt;
+  const double old = *c;
+  const double* p = scratch + rd.part0 + e;
+  double acc = 0.0;
+#pragma unroll 8
+  for (int i = 0; i < rd.nparts; ++i) acc += __ldg(p + (long long)i * outs);
+  *c = old + acc;
 }
 
 // sum the partial tiles of one sigma tile in a fixed order and add into C
@@ -367,20 +466,12 @@ __global__ void hpsi_reduce_kernel(const HpsiBlock* __restrict__ blocks, const H
 
 }  // namespace
 
-void hpsi_tile(Precision prec, int* tile_m, int* tile_n) {
-  (void)prec;
-  *tile_m = T;
-  *tile_n = T;
-}
+namespace {
 
-size_t hpsi_plan_tasks(const std::vector<HpsiBlock>& blocks, Precision prec, std::vector<HpsiTask>& tasks,
-                       std::vector<HpsiReduce>& reds) {
-  tasks.clear();
-  reds.clear();
-  int tm, tn;
-  hpsi_tile(prec, &tm, &tn);
+// tiles of 64 x 64 in item chunks of equal count
+size_t plan_square(const std::vector<HpsiBlock>& blocks, std::vector<HpsiTask>& tasks, std::vector<HpsiReduce>& reds) {
   long long tile_items = 0;
-  for (auto& b : blocks) tile_items += (long long)b.item_count * ((b.m + tm - 1) / tm) * ((b.n + tn - 1) / tn);
+  for (auto& b : blocks) tile_items += (long long)b.item_count * ((b.m + T - 1) / T) * ((b.n + T - 1) / T);
   const int max_items = (int)std::max<long long>(4, tile_items / (8 * 152) + 1);
   long long part = 0;
   for (size_t b = 0; b < blocks.size(); ++b) {
@@ -388,8 +479,8 @@ size_t hpsi_plan_tasks(const std::vector<HpsiBlock>& blocks, Precision prec, std
     if (bk.item_count == 0 || bk.m == 0 || bk.n == 0) continue;
     int nch = (bk.item_count + max_items - 1) / max_items;
     int per = (bk.item_count + nch - 1) / nch;
-    for (int r0 = 0; r0 < bk.m; r0 += tm)
-      for (int c0 = 0; c0 < bk.n; c0 += tn) {
+    for (int r0 = 0; r0 < bk.m; r0 += T)
+      for (int c0 = 0; c0 < bk.n; c0 += T) {
         if (nch == 1) {
           tasks.push_back({(int)b, r0, c0, bk.item_begin, bk.item_count, -1});
         } else {
@@ -398,12 +489,104 @@ size_t hpsi_plan_tasks(const std::vector<HpsiBlock>& blocks, Precision prec, std
             int i0 = bk.item_begin + c * per;
             int cnt = std::min(per, bk.item_begin + bk.item_count - i0);
             tasks.push_back({(int)b, r0, c0, i0, cnt, part});
-            part += (long long)tm * tn;
+            part += (long long)T * T;
           }
         }
       }
   }
   return (size_t)part;
+}
+
+// Clocks of an item on a tile: two FMAs a clock, and the latency of the loads
+// of its k-steps (about 1200 clocks each, shared by four CTAs an SM).
+double f64_item_cost(const HpsiItem& it, int mt, int nt) {
+  const double ka = it.A ? it.ka : 0.0, kb = it.kb;
+  double c = 0.5 * mt * (ka * (it.B ? kb : std::min<double>(kb, nt)) + (it.B ? kb * nt : 0.0));
+  return c + 300.0 * (1.0 + ka / KS * ((kb + kF64Chunk - 1) / kF64Chunk) + (it.B ? kb / KS : 0.0));
+}
+
+// Tiles of f64_tile, the items of a tile in chunks of about `target` clocks;
+// target < 0: one task per column tile, walking all rows and items.
+size_t plan_f64(const std::vector<HpsiBlock>& blocks, const std::vector<HpsiItem>& items, double target,
+                std::vector<HpsiTask>& tasks, std::vector<HpsiReduce>& reds) {
+  tasks.clear();
+  reds.clear();
+  long long part = 0;
+  std::vector<int> cut;
+  for (size_t b = 0; b < blocks.size(); ++b) {
+    const HpsiBlock& bk = blocks[b];
+    if (bk.item_count == 0 || bk.m == 0 || bk.n == 0) continue;
+    int mt, nt;
+    f64_tile(bk.m, bk.n, mt, nt);
+    const int first = bk.item_begin, last = first + bk.item_count;
+    if (target < 0) {
+      for (int c0 = 0; c0 < bk.n; c0 += nt) tasks.push_back({(int)b, -1, c0, first, bk.item_count, -1});
+      continue;
+    }
+    // cuts into chunks of equal cost, the same for every tile of the block
+    double total = 0.0;
+    for (int i = first; i < last; ++i) total += f64_item_cost(items[i], mt, nt);
+    const int nch = (int)std::max(1.0, std::min<double>(bk.item_count, total / target));
+    cut.assign(1, first);
+    double run = 0.0;
+    for (int i = first; i < last; ++i) {
+      run += f64_item_cost(items[i], mt, nt);
+      if (run >= total * cut.size() / nch && i + 1 < last && (int)cut.size() < nch) cut.push_back(i + 1);
+    }
+    cut.push_back(last);
+    const int n = (int)cut.size() - 1;
+    for (int r0 = 0; r0 < bk.m; r0 += mt)
+      for (int c0 = 0; c0 < bk.n; c0 += nt) {
+        const long long outs = (long long)std::min(mt, bk.m - r0) * std::min(nt, bk.n - c0);
+        if (n > 1) reds.push_back({(int)b, r0, c0, n, part});
+        for (int c = 0; c < n; ++c) {
+          tasks.push_back({(int)b, r0, c0, cut[c], cut[c + 1] - cut[c], n > 1 ? part : -1});
+          if (n > 1) part += outs;
+        }
+      }
+  }
+  return (size_t)part;
+}
+
+size_t plan_bytes(size_t part, const std::vector<HpsiTask>& tasks, const std::vector<HpsiReduce>& reds) {
+  return part * sizeof(double) + ((tasks.size() * sizeof(HpsiTask) + 255) & ~size_t(255)) +
+         ((reds.size() * sizeof(HpsiReduce) + 255) & ~size_t(255));
+}
+
+}  // namespace
+
+size_t hpsi_plan_tasks(const std::vector<HpsiBlock>& blocks, const std::vector<HpsiItem>& items, Precision prec,
+                       std::vector<HpsiTask>& tasks, std::vector<HpsiReduce>& reds, size_t* nominal_bytes) {
+  tasks.clear();
+  reds.clear();
+  const size_t square = plan_square(blocks, tasks, reds);
+  const size_t nominal = plan_bytes(square, tasks, reds);
+  if (nominal_bytes) *nominal_bytes = nominal;
+  if (prec != Precision::FP64) return square;
+  // Two waves of the CTAs that the SMs hold at once (152 x 4), no chunk below
+  // 8000 clocks (a tenth of which a partial tile's store and reduction cost).
+  // Lists and partial tiles take no more than those of the 64 x 64 plan would,
+  // or than 8 MB of what the allocation-free entry has: longer chunks, at last
+  // one task per column tile.
+  const size_t lists = (blocks.size() * sizeof(HpsiBlock) + 255) / 256 * 256 +
+                       (items.size() * sizeof(HpsiItem) + 255) / 256 * 256;
+  const size_t left = lists < kNoAllocScratchBytes ? kNoAllocScratchBytes - lists : 0;
+  const size_t limit = std::max(nominal, std::min(size_t(8) << 20, left));
+  double total = 0.0;
+  for (const HpsiBlock& bk : blocks) {
+    if (bk.item_count == 0 || bk.m == 0 || bk.n == 0) continue;
+    int mt, nt;
+    f64_tile(bk.m, bk.n, mt, nt);
+    double c = 0.0;
+    for (int i = bk.item_begin; i < bk.item_begin + bk.item_count; ++i) c += f64_item_cost(items[i], mt, nt);
+    total += c * ((bk.m + mt - 1) / mt) * ((bk.n + nt - 1) / nt);
+  }
+  double target = std::max(8000.0, total / (152 * 4 * 2));
+  for (int k = 0; k < 6; ++k, target *= 4.0) {
+    const size_t part = plan_f64(blocks, items, target, tasks, reds);
+    if (plan_bytes(part, tasks, reds) <= limit) return part;
+  }
+  return plan_f64(blocks, items, -1.0, tasks, reds);
 }
 
 void hpsi_launch(const HpsiBlock* blocks, const HpsiItem* items, const HpsiTask* tasks, int ntasks,
@@ -414,11 +597,10 @@ void hpsi_launch(const HpsiBlock* blocks, const HpsiItem* items, const HpsiTask*
     throw std::runtime_error("internal: the tcgen05 contraction runs on pre-split operands (hpsi_tc_launch)");
   if (ntasks > 0) {
     if (prec == Precision::FP64) {
-      size_t smem = (size_t)(3 * KS * (T + 1) + T * (T + 1)) * sizeof(double);
-      cudaError_t ea = ensure_smem_attr((const void*)hpsi_f64_kernel, (int)smem);
+      cudaError_t ea = ensure_smem_attr((const void*)hpsi_f64_kernel, (int)kF64Smem);
       if (ea != cudaSuccess)
         throw std::runtime_error(std::string("cuda: hpsi f64 attribute: ") + cudaGetErrorString(ea));
-      hpsi_f64_kernel<<<ntasks, 256, smem, st>>>(blocks, items, tasks, scratch);
+      hpsi_f64_kernel<<<ntasks, kF64Threads, kF64Smem, st>>>(blocks, items, tasks, scratch);
     } else {
       size_t smem = (size_t)SM_WORDS * sizeof(uint32_t);
       cudaError_t ea = ensure_smem_attr((const void*)hpsi_tf32x3_kernel, (int)smem);
@@ -430,7 +612,10 @@ void hpsi_launch(const HpsiBlock* blocks, const HpsiItem* items, const HpsiTask*
     if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: hpsi launch: ") + cudaGetErrorString(e));
   }
   if (nreds > 0) {
-    hpsi_reduce_kernel<<<nreds, 256, 0, st>>>(blocks, reds, scratch);
+    if (prec == Precision::FP64)
+      hpsi_f64_reduce_kernel<<<dim3(nreds, kF64Slots), 128, 0, st>>>(blocks, reds, scratch);
+    else
+      hpsi_reduce_kernel<<<nreds, 256, 0, st>>>(blocks, reds, scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: hpsi reduce: ") + cudaGetErrorString(e));
   }

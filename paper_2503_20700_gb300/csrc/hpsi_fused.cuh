@@ -38,26 +38,26 @@ struct HpsiBlock {
 };
 
 struct HpsiTask {
-  int block, r0, c0;
+  int block, r0, c0;  // r0 = -1 (FP64): all row tiles of the block
   int it_begin, it_count;
   long long part;  // offset (elements) of this task's partial tile in scratch, or -1: add into C
 };
 
 struct HpsiReduce {
   int block, r0, c0, nparts;
-  long long part0;  // first partial; the others follow at +tile_m*tile_n each
+  long long part0;  // first partial; the others follow, a tile each
 };
 
-// sigma tile owned by one CTA of the kernel used for `prec`: 64 x 64 (FP64 and
-// SPLIT_TF32 on mma.sync; the tcgen05 contraction plans its own 128 x 256
-// tiles in hpsi_tc_prepare).
-void hpsi_tile(Precision prec, int* tile_m, int* tile_n);
-
-// Builds the task list (tiles x item chunks) for the given blocks; returns the
-// scratch size (elements) the partial tiles need.  The item chunk length is
-// chosen so that one launch has several waves of CTAs on 152 SMs.
-size_t hpsi_plan_tasks(const std::vector<HpsiBlock>& blocks, Precision prec, std::vector<HpsiTask>& tasks,
-                       std::vector<HpsiReduce>& reds);
+// Builds the task list (tiles x item chunks) for the given blocks and items;
+// returns the scratch size (elements) the partial tiles need.  The chunk
+// length is chosen so that one launch has a few waves of CTAs on 152 SMs.
+// SPLIT_TF32 (mma.sync) has 64 x 64 tiles; FP64 has tiles that fit the blocks
+// and keeps its lists and partial tiles within what 64 x 64 tiles would take
+// (nominal_bytes: the bytes of those, for either precision); the tcgen05
+// contraction plans its own 128 x 256 tiles in hpsi_tc_prepare.
+size_t hpsi_plan_tasks(const std::vector<HpsiBlock>& blocks, const std::vector<HpsiItem>& items, Precision prec,
+                       std::vector<HpsiTask>& tasks, std::vector<HpsiReduce>& reds,
+                       size_t* nominal_bytes = nullptr);
 
 // Launches the fused kernel and the reduction (device pointers in the lists).
 // prec: FP64 or SPLIT_TF32 (err is unused by these kernels).

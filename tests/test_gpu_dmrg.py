@@ -334,6 +334,28 @@ def test_fused_hpsi_many_items_split_into_chunks(pkg):
         assert np.abs(C1[off:off + m * n].reshape(m, n) - ref).max() < 1e-11 * np.abs(ref).max()
 
 
+@pytest.mark.parametrize("m,n", [(1, 1), (1, 257), (300, 1), (128, 16), (129, 15), (8, 256), (9, 255), (45, 46),
+                                 (23, 512), (200, 208)])
+def test_fused_hpsi_f64_tile_edges(pkg, m, n):
+    """Float64 kernel at the edges of its tiles (2048 outputs, at most 128 rows
+    and 256 columns), of the 128-column chunks of psi and of its k-steps of
+    16, with identities on either side.  Tolerance: a chain of ka + kb FMAs
+    over ka kb products of unit normals, next to the largest result."""
+    rng = np.random.default_rng(1000 * m + n)
+    shapes = [(m, n, [(1, 1), (16, 128), (17, 129), (15, 300), (40, 3)])]
+    A, P, B, clen, blocks, items, refs = random_hpsi_problem(rng, 0, 0, 0, shapes=shapes)
+    x, y = rng.standard_normal((m, 33)), rng.standard_normal((29, n))      # psi of A = 1 and of B = 1
+    bt, al = rng.standard_normal((n, 33)), rng.standard_normal((m, 29))
+    items += [(0, P.size, B.size, 1, 33, 33, 0, 0, m, 33, 1, 0, 0.5),
+              (A.size, P.size + x.size, 0, 29, n, 1, 0, 0, 29, n, 0, 1, -2.0)]
+    blocks = [(0, m, n, n, 0, len(items))]
+    ref = refs[0][3] + 0.5 * x @ bt.T - 2.0 * al @ y
+    P, B, A = np.concatenate([P, x.ravel(), y.ravel()]), np.concatenate([B, bt.ravel()]), np.concatenate([A, al.ravel()])
+    C = np.zeros(clen)
+    pkg.ops.hpsi_contract(A, P, B, C, blocks, items, precision=0)
+    assert np.abs(C.reshape(m, n) - ref).max() < 1e-12 * max(1.0, np.abs(ref).max())
+
+
 def test_fused_hpsi_tcgen05_chunks_and_tails(pkg):
     """tcgen05 kernel (128 x 256 sigma tiles): blocks spanning several row and
     column tiles with ragged tails, hundreds of items split into chunks;
