@@ -6,11 +6,11 @@
 //   gemm_digits_kernel (gemm_digits.cu)                        (FP64 as exact bf16 digit products on tcgen05)
 //   gemm_tf32x3 (gemm_split.cu)                                (split-FP32 tensor-core path)
 //   dots/combine/axpby  Davidson vector algebra (FP64, deterministic two-stage reductions)
-//   jacobi_smem_kernel  parallel cyclic Jacobi eigensolver (FP64) of one matrix in shared memory, one CTA
-//   jacobi_coop_kernel  a batch of matrices on one CTA per SM, each on a group of CTAs sized to its work
+//   eigh.cu             batched FP64 eigensolver: Jacobi for small matrices, tridiagonalisation on groups of
+//                       CTAs and divide and conquer for larger ones
 // All kernels are bounded loops over their inputs; the one wait on other CTAs,
-// the group barrier of jacobi_coop_kernel, gives up after the backend's wait
-// bound (2 s by default) and sets the error flag.
+// the group barrier of the tridiagonalisation, gives up after the backend's
+// wait bound (2 s by default) and sets the error flag.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "backend.hpp"
+#include "eigh.cuh"
 #include "gemm_digits.cuh"
 #include "gemm_split.cuh"
 #include "hpsi_fused.cuh"
@@ -214,403 +215,6 @@ __global__ void precond_kernel(double* __restrict__ y, const double* __restrict_
   }
 }
 
-// ------------------------------------------------------------------ Jacobi
-// Parallel cyclic Jacobi (round-robin pairing) on a symmetric n x n matrix
-// (destroyed).  Eigenvalues descending in w, the eigenvectors as rows of V.
-// One round rotates n/2 disjoint pairs.  The matrix is updated as 2x2 blocks
-// (rows of pair i, columns of pair j) R_i X R_j^T for i <= j only, each
-// result stored at both symmetric positions: 2n^2 FP64 operations a round on
-// A instead of 4n^2, plus 2n^2 on the eigenvector rows p, q of V.  A pair is
-// skipped when its off-diagonal entry is negligible next to both diagonal
-// entries, or below 1e-16 ||A||_F: the rounding noise of a GEMM-formed
-// density matrix, whose (near) null space would otherwise keep rotating noise
-// for every sweep.  The iteration stops after a sweep without rotations, or
-// after kMaxSweeps sweeps.
-//
-// The work is FP64-bound (GB300 has few FP64 units per SM), so a batch of
-// matrices is spread over the SMs: one cooperative launch with one CTA per
-// SM, each matrix on a group of g CTAs sized to its share of the work (g = 1:
-// A and V in shared memory; g > 1: A and V in global memory, one group
-// barrier per round).
-constexpr int kMaxSweeps = 30;
-constexpr int kSmemN = kJacSmemN;  // largest matrix of the shared-memory path
-constexpr int kJacThreads = 512;  // threads of a batched-launch CTA
-
-__host__ __device__ constexpr size_t jacobi_smem_bytes(int n) {
-  return ((size_t)n * (n + 1) + (size_t)n * n + (size_t)((n + 1) & ~1)) * sizeof(double) +
-         (size_t)((n + 1) & ~1) * 2 * sizeof(int) + 64;
-}
-
-// pair i of a round, closed form of the round-robin schedule: (round, M) and
-// (round + i, round - i) mod M, M = np - 1
-__device__ __forceinline__ void jac_pair(int round, int i, int np, int& p, int& q) {
-  const int M = np - 1;
-  p = i == 0 ? round : (round + i) % M;
-  q = i == 0 ? M : (round - i + M) % M;
-  if (p > q) {
-    int t = p;
-    p = q;
-    q = t;
-  }
-}
-
-// (c, s) of the rotation that annihilates a_pq; false when the pair is skipped
-__device__ __forceinline__ bool jac_rotation(double apq, double app, double aqq, double floor_abs, double& c,
-                                             double& s) {
-  c = 1.0;
-  s = 0.0;
-  const double g = 100.0 * fabs(apq);
-  if (fabs(apq) <= floor_abs || (fabs(app) + g == fabs(app) && fabs(aqq) + g == fabs(aqq))) return false;
-  const double theta = (aqq - app) / (2.0 * apq);
-  const double t = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-  c = 1.0 / sqrt(t * t + 1.0);
-  s = t * c;
-  return true;
-}
-
-// block (i, j), i <= j < h, of linear index e in the row-major upper triangle;
-// row i starts at i h - i (i - 1) / 2
-__device__ __forceinline__ void tri_index(int e, int h, int& i, int& j) {
-  const float b = 2.0f * (float)h + 1.0f;
-  int r = (int)((b - sqrtf(fmaxf(b * b - 8.0f * (float)e, 0.0f))) * 0.5f);
-  r = max(0, min(r, h - 1));
-  while (r > 0 && r * h - r * (r - 1) / 2 > e) --r;
-  while (r + 1 < h && (r + 1) * h - (r + 1) * r / 2 <= e) ++r;
-  i = r;
-  j = r + (e - (r * h - r * (r - 1) / 2));
-}
-
-template <bool kGlobal>
-__device__ __forceinline__ double jac_ld(const double* p) {
-  if constexpr (kGlobal) return __ldcg(p);
-  else return *p;
-}
-
-struct JacRound {
-  const double* cs;
-  const double* sn;
-  const int* pp;
-  const int* qq;
-};
-
-// R_i X R_j^T on block (i, j), i <= j, stored at both symmetric positions
-template <bool kGlobal>
-__device__ __forceinline__ void jac_block(double* a, int lda, int n, int i, int j, const JacRound& R) {
-  const double ci = R.cs[i], si = R.sn[i], cj = R.cs[j], sj = R.sn[j];
-  if (si == 0.0 && sj == 0.0) return;
-  const int p = R.pp[i], q = R.qq[i], r = R.pp[j], t = R.qq[j];
-  const bool qv = q < n, tv = t < n;
-  const double x00 = jac_ld<kGlobal>(a + (size_t)p * lda + r);
-  const double x01 = tv ? jac_ld<kGlobal>(a + (size_t)p * lda + t) : 0.0;
-  const double x10 = qv ? jac_ld<kGlobal>(a + (size_t)q * lda + r) : 0.0;
-  const double x11 = (qv && tv) ? jac_ld<kGlobal>(a + (size_t)q * lda + t) : 0.0;
-  const double y00 = ci * x00 - si * x10, y01 = ci * x01 - si * x11;
-  const double y10 = si * x00 + ci * x10, y11 = si * x01 + ci * x11;
-  const double n00 = cj * y00 - sj * y01, n01 = sj * y00 + cj * y01;
-  if (i == j) {  // r = p, t = q: the diagonal block, (p, q) and (q, p) from one value
-    a[(size_t)p * lda + p] = n00;
-    if (qv) {
-      a[(size_t)p * lda + q] = n01;
-      a[(size_t)q * lda + p] = n01;
-      a[(size_t)q * lda + q] = sj * y10 + cj * y11;
-    }
-    return;
-  }
-  const double n10 = cj * y10 - sj * y11, n11 = sj * y10 + cj * y11;
-  a[(size_t)p * lda + r] = n00;
-  a[(size_t)r * lda + p] = n00;
-  if (tv) {
-    a[(size_t)p * lda + t] = n01;
-    a[(size_t)t * lda + p] = n01;
-  }
-  if (qv) {
-    a[(size_t)q * lda + r] = n10;
-    a[(size_t)r * lda + q] = n10;
-  }
-  if (qv && tv) {
-    a[(size_t)q * lda + t] = n11;
-    a[(size_t)t * lda + q] = n11;
-  }
-}
-
-// element k of the eigenvector rows p, q of pair i
-template <bool kGlobal>
-__device__ __forceinline__ void jac_vrot(double* v, int n, int i, int k, const JacRound& R) {
-  const double s = R.sn[i];
-  if (s == 0.0) return;
-  const double c = R.cs[i];
-  const int p = R.pp[i], q = R.qq[i];
-  const double vp = jac_ld<kGlobal>(v + (size_t)p * n + k), vq = jac_ld<kGlobal>(v + (size_t)q * n + k);
-  v[(size_t)p * n + k] = c * vp - s * vq;
-  v[(size_t)q * n + k] = s * vp + c * vq;
-}
-
-// rotation parameters of every pair of the round (threads < h); nrot counts
-// the rotations of the sweep
-template <bool kGlobal>
-__device__ __forceinline__ void jac_params(const double* a, int lda, int n, int np, int round, double floor_abs,
-                                           double* cs, double* sn, int* pp, int* qq, int* nrot) {
-  const int h = np / 2;
-  for (int i = threadIdx.x; i < h; i += blockDim.x) {
-    int p, q;
-    jac_pair(round, i, np, p, q);
-    pp[i] = p;
-    qq[i] = q;
-    double c = 1.0, s = 0.0;
-    if (q < n &&
-        jac_rotation(jac_ld<kGlobal>(a + (size_t)p * lda + q), jac_ld<kGlobal>(a + (size_t)p * lda + p),
-                     jac_ld<kGlobal>(a + (size_t)q * lda + q), floor_abs, c, s))
-      atomicAdd(nrot, 1);
-    cs[i] = c;
-    sn[i] = s;
-  }
-}
-
-// sum over the CTA (blockDim a power of two, red holds blockDim values)
-__device__ double jac_block_sum(double x, double* red) {
-  red[threadIdx.x] = x;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
-  }
-  const double r = red[0];
-  __syncthreads();
-  return r;
-}
-
-// rank of the diagonal entries, descending (NaN last, ties by index): perm[rank] = i
-template <bool kGlobal>
-__device__ void jac_order(const double* a, int lda, int n, int* perm) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    double di = jac_ld<kGlobal>(a + (size_t)i * lda + i);
-    if (!(di == di)) di = -INFINITY;
-    int rank = 0;
-    for (int j = 0; j < n; ++j) {
-      double dj = jac_ld<kGlobal>(a + (size_t)j * lda + j);
-      if (!(dj == dj)) dj = -INFINITY;
-      rank += (dj > di) || (dj == di && j < i);
-    }
-    perm[rank] = i;
-  }
-}
-
-// one matrix on one CTA, A (row stride n+1) and V in shared memory
-__device__ void jacobi_one(const EighTask& tk, double* sm, double* red, int* nrot) {
-  const int n = tk.n;
-  const int lda = n + 1;
-  const int np = (n + 1) & ~1, h = np / 2;
-  double* a = sm;                   // n x (n+1)
-  double* v = a + (size_t)n * lda;  // n x n, row p = eigenvector p
-  double* cs = v + (size_t)n * n;   // h
-  double* sn = cs + h;              // h
-  int* pp = (int*)(sn + h);
-  int* qq = pp + h;
-  int* perm = qq + h;  // np
-  const JacRound R{cs, sn, pp, qq};
-  double fro = 0.0;
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-    const int r = e / n, c = e % n;
-    const double x = tk.A[e];
-    a[r * lda + c] = x;
-    v[e] = (r == c) ? 1.0 : 0.0;
-    fro += x * x;
-  }
-  const double floor_abs = 1e-16 * sqrt(jac_block_sum(fro, red));
-  const int nb = h * (h + 1) / 2;
-  for (int sweep = 0; sweep < kMaxSweeps && n > 1; ++sweep) {
-    if (threadIdx.x == 0) *nrot = 0;
-    __syncthreads();
-    for (int round = 0; round < np - 1; ++round) {
-      jac_params<false>(a, lda, n, np, round, floor_abs, cs, sn, pp, qq, nrot);
-      __syncthreads();
-      for (int e = threadIdx.x; e < nb; e += blockDim.x) {
-        int i, j;
-        tri_index(e, h, i, j);
-        jac_block<false>(a, lda, n, i, j, R);
-      }
-      for (int e = threadIdx.x; e < h * n; e += blockDim.x) jac_vrot<false>(v, n, e / n, e % n, R);
-      __syncthreads();
-    }
-    if (*nrot == 0) break;
-    __syncthreads();
-  }
-  jac_order<false>(a, lda, n, perm);
-  __syncthreads();
-  for (int r = threadIdx.x; r < n; r += blockDim.x) tk.w[r] = a[perm[r] * lda + perm[r]];
-  // eigenvector rows in descending order, largest-magnitude component positive
-  for (int r = threadIdx.x; r < n; r += blockDim.x) {
-    const double* src = v + (size_t)perm[r] * n;
-    double best = 0.0;
-    int bi = 0;
-    for (int k = 0; k < n; ++k) {
-      double x = fabs(src[k]);
-      if (x > best + 1e-12) {
-        best = x;
-        bi = k;
-      }
-    }
-    const double sg = src[bi] < 0 ? -1.0 : 1.0;
-    for (int k = 0; k < n; ++k) tk.V[(size_t)r * n + k] = sg * src[k];
-  }
-}
-
-__global__ void __launch_bounds__(256) jacobi_smem_kernel(const EighTask* __restrict__ tasks) {
-  extern __shared__ double sm[];
-  __shared__ double red[256];
-  __shared__ int nrot;
-  jacobi_one(tasks[blockIdx.x], sm, red, &nrot);
-}
-
-// A matrix on a group of g CTAs: every CTA of the group computes the round's
-// rotation parameters from the same entries (identical values, so no
-// exchange is needed) and updates its own contiguous share of the triangle
-// blocks and of the eigenvector elements; one group barrier per round
-// publishes the updates.  The barrier's wait is bounded by the backend's
-// wait bound (wall clock) and sets the error flag on timeout; with a bound of
-// 0 a barrier not complete at its first probe gives up.
-struct CoopEigh {
-  EighTask t;
-  int g, cta0;
-  unsigned* bar;  // (arrivals, generation), zero at launch
-};
-
-__device__ __forceinline__ unsigned long long jac_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-
-__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
-  unsigned x;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(p) : "memory");
-  return x;
-}
-
-// returns false when the wait ran out
-__device__ bool group_sync(unsigned* bar, int g, unsigned& gen, int* ok_s, unsigned long long wait_ns) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned target = gen + 1;
-    if (atomicAdd(&bar[0], 1u) == (unsigned)g - 1) {
-      atomicExch(&bar[0], 0u);
-      __threadfence();
-      atomicExch(&bar[1], target);
-    } else {
-      const unsigned long long t0 = jac_ns();
-      const int spin = wait_ns > 0 ? 256 : 1;
-      for (int probe = 0; (int)(ld_acquire(&bar[1]) - target) < 0; ++probe) {
-        if (probe >= spin) {
-          if (jac_ns() - t0 >= wait_ns) {
-            *ok_s = 0;
-            break;
-          }
-          __nanosleep(32);
-        }
-      }
-    }
-    gen = target;
-    __threadfence();
-  }
-  __syncthreads();
-  return *ok_s != 0;
-}
-
-__device__ void jacobi_group(const CoopEigh& ct, int me, double* sm, double* red, int* nrot, int* ok_s,
-                             int* err, unsigned long long wait_ns) {
-  const int g = ct.g;
-  const int n = ct.t.n;
-  double* a = const_cast<double*>(ct.t.A);
-  double* v = ct.t.V;
-  const int np = (n + 1) & ~1, h = np / 2;
-  double* cs = sm;
-  double* sn = sm + h;
-  int* pp = (int*)(sm + np);
-  int* qq = pp + h;
-  int* perm = qq + h;
-  const JacRound R{cs, sn, pp, qq};
-  unsigned gen = 0;
-  if (threadIdx.x == 0) *ok_s = 1;
-  for (int r = me; r < n; r += g)
-    for (int k = threadIdx.x; k < n; k += blockDim.x) v[(size_t)r * n + k] = (r == k) ? 1.0 : 0.0;
-  double fro = 0.0;
-  for (size_t e = threadIdx.x; e < (size_t)n * n; e += blockDim.x) {
-    const double x = __ldcg(a + e);
-    fro += x * x;
-  }
-  const double floor_abs = 1e-16 * sqrt(jac_block_sum(fro, red));
-  // this CTA's shares: triangle blocks [b0, b1), eigenvector elements [v0, v1)
-  const long long nb = (long long)h * (h + 1) / 2, nv = (long long)h * n;
-  const int b0 = (int)(nb * me / g), b1 = (int)(nb * (me + 1) / g);
-  const int v0 = (int)(nv * me / g), v1 = (int)(nv * (me + 1) / g);
-  if (!group_sync(ct.bar, g, gen, ok_s, wait_ns)) goto fail;
-  for (int sweep = 0; sweep < kMaxSweeps && n > 1; ++sweep) {
-    if (threadIdx.x == 0) *nrot = 0;
-    __syncthreads();
-    for (int round = 0; round < np - 1; ++round) {
-      jac_params<true>(a, n, n, np, round, floor_abs, cs, sn, pp, qq, nrot);
-      __syncthreads();
-      for (int e = b0 + (int)threadIdx.x; e < b1; e += blockDim.x) {
-        int i, j;
-        tri_index(e, h, i, j);
-        jac_block<true>(a, n, n, i, j, R);
-      }
-      for (int e = v0 + (int)threadIdx.x; e < v1; e += blockDim.x) jac_vrot<true>(v, n, e / n, e % n, R);
-      if (!group_sync(ct.bar, g, gen, ok_s, wait_ns)) goto fail;
-    }
-    if (*nrot == 0) break;
-    __syncthreads();
-  }
-  if (me != 0) return;
-  // CTA 0: eigenvalues descending, rows of V permuted, largest component positive
-  jac_order<true>(a, n, n, perm);
-  __syncthreads();
-  for (int r = threadIdx.x; r < n; r += blockDim.x) ct.t.w[r] = __ldcg(a + (size_t)perm[r] * n + perm[r]);
-  __syncthreads();
-  for (size_t e = threadIdx.x; e < (size_t)n * n; e += blockDim.x) a[e] = __ldcg(v + e);
-  __syncthreads();
-  for (size_t e = threadIdx.x; e < (size_t)n * n; e += blockDim.x) {
-    const int r = (int)(e / n), k = (int)(e % n);
-    v[e] = a[(size_t)perm[r] * n + k];
-  }
-  __syncthreads();
-  for (int r = threadIdx.x; r < n; r += blockDim.x) {
-    double best = 0.0;
-    int bi = 0;
-    for (int k = 0; k < n; ++k) {
-      double x = fabs(v[(size_t)r * n + k]);
-      if (x > best + 1e-12) {
-        best = x;
-        bi = k;
-      }
-    }
-    if (v[(size_t)r * n + bi] < 0)
-      for (int k = 0; k < n; ++k) v[(size_t)r * n + k] = -v[(size_t)r * n + k];
-  }
-  return;
-fail:
-  if (threadIdx.x == 0) atomicExch(err, 1);
-}
-
-// The batched launch: CTA b belongs to the last task whose cta0 <= b.
-__global__ void __launch_bounds__(kJacThreads) jacobi_coop_kernel(const CoopEigh* __restrict__ tasks, int ntasks,
-                                                                  int* __restrict__ err,
-                                                                  unsigned long long wait_ns) {
-  int lo = 0, hi = ntasks - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) / 2;
-    if (tasks[mid].cta0 <= (int)blockIdx.x) lo = mid;
-    else hi = mid - 1;
-  }
-  const CoopEigh ct = tasks[lo];
-  extern __shared__ double sm[];
-  __shared__ double red[kJacThreads];
-  __shared__ int nrot, ok_s;
-  if (ct.g == 1) jacobi_one(ct.t, sm, red, &nrot);
-  else jacobi_group(ct, (int)blockIdx.x - ct.cta0, sm, red, &nrot, &ok_s, err, wait_ns);
-}
-
 // ------------------------------------------------------------------ backend
 class CudaBackend : public Backend {
  public:
@@ -635,8 +239,7 @@ class CudaBackend : public Backend {
   std::vector<Rec> recs;
   std::vector<cudaEvent_t> pool;
   // categories: 0 GEMMs, 1 H_eff psi (with its operand splits), 2 blocking
-  // placement, 3 eigensolver (shared-memory kernel), 4 eigensolver
-  // (cooperative kernel)
+  // placement, 3 eigensolver (small matrices only), 4 eigensolver
   static constexpr int kTags = 6;
   double acc_ms[kTags] = {0, 0, 0, 0, 0, 0}, acc_flops[kTags] = {0, 0, 0, 0, 0, 0};
   long acc_launch[kTags] = {0, 0, 0, 0, 0, 0};
@@ -1182,73 +785,179 @@ class CudaBackend : public Backend {
     ++launches;
     CK(cudaGetLastError());
   }
-  // One small matrix (the Davidson subspace problem): one CTA.  A batch (the
-  // density-matrix sectors of a decimation): cooperative launches of one CTA
-  // per SM (the shared memory of the n <= kSmemN path admits one CTA per SM),
-  // largest matrices first, group sizes from jac_assign_groups.
-  bool jac_init = false;
-  int jac_cap = 0;
+  // Matrices up to kEighSmall: one launch of the Jacobi kernel.  Larger ones:
+  // cooperative launches of the tridiagonalisation (largest matrices first,
+  // group sizes from jac_assign_groups), then the levels of merges with their
+  // products on the grouped GEMM, then the reflectors.  Work space (two more
+  // copies of the matrices) is kept to the digit pool's bound, the batch cut
+  // into parts of it; a larger single matrix runs whole.
+  int tri_cap = 0;
   void eigh(const std::vector<EighTask>& tasks) override {
     if (tasks.empty()) return;
-    const size_t smem = jacobi_smem_bytes(kSmemN);
-    if (!jac_init) {
-      CK(cudaFuncSetAttribute(jacobi_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      CK(cudaFuncSetAttribute(jacobi_coop_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      int per_sm = 0, sms = 0;
-      CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_coop_kernel, kJacThreads, smem));
-      CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-      jac_cap = per_sm * sms;
-      if (jac_cap < 2) throw std::runtime_error("cuda: eigensolver needs two co-resident CTAs");
-      jac_init = true;
-    }
-    if (tasks.size() == 1 && tasks[0].n <= kSmemN) {
-      std::vector<size_t> off;
-      char* d = upload({{tasks.data(), sizeof(EighTask)}}, off);
-      Rec* rec = nullptr;
-      if (profiling) {
-        recs.push_back(Rec{ev(), ev(), 0.0, 3});
-        rec = &recs.back();
-        CK(cudaEventRecord(rec->a, st));
-      }
-      jacobi_smem_kernel<<<1, 256, jacobi_smem_bytes(tasks[0].n), st>>>((const EighTask*)(d + off[0]));
-      if (rec) CK(cudaEventRecord(rec->b, st));
-      ++launches;
-      CK(cudaGetLastError());
-      return;
-    }
     std::vector<EighTask> order(tasks);
     std::stable_sort(order.begin(), order.end(), [](const EighTask& x, const EighTask& y) { return x.n > y.n; });
-    std::vector<int> n_desc;
-    for (auto& t : order) n_desc.push_back(t.n);
-    for (const JacBatch& jb : jac_plan_batches(n_desc, jac_cap)) {
-      std::vector<CoopEigh> ct;
-      int ctas = 0;
-      for (size_t k = jb.begin; k < jb.end; ++k) {
-        ct.push_back({order[k], jb.g[k - jb.begin], ctas, nullptr});
-        ctas += jb.g[k - jb.begin];
-      }
-      std::vector<unsigned> bars(2 * ct.size(), 0u);
+    while (!order.empty() && order.back().n <= 0) order.pop_back();
+    size_t big = 0;
+    while (big < order.size() && order[big].n > kEighSmall) ++big;
+    Rec* rec = nullptr;
+    if (profiling) {
+      recs.push_back(Rec{ev(), ev(), 0.0, big ? 4 : 3});
+      rec = &recs.back();
+      CK(cudaEventRecord(rec->a, st));
+    }
+    if (big < order.size()) {
       std::vector<size_t> off;
-      char* d = upload({{ct.data(), ct.size() * sizeof(CoopEigh)}, {bars.data(), bars.size() * sizeof(unsigned)}},
-                       off);
-      unsigned* dbar = (unsigned*)(d + off[1]);
-      for (size_t k = 0; k < ct.size(); ++k) ct[k].bar = dbar + 2 * k;
-      CK(cudaMemcpyAsync(d + off[0], ct.data(), ct.size() * sizeof(CoopEigh), cudaMemcpyHostToDevice, st));
-      const CoopEigh* dt = (const CoopEigh*)(d + off[0]);
-      int nt = (int)ct.size();
-      int* fl = flag();
-      unsigned long long wns = wait_ns_;
-      void* args[] = {(void*)&dt, (void*)&nt, (void*)&fl, (void*)&wns};
-      Rec* rec = nullptr;
-      if (profiling) {
-        recs.push_back(Rec{ev(), ev(), 0.0, 4});
-        rec = &recs.back();
-        CK(cudaEventRecord(rec->a, st));
-      }
-      CK(cudaLaunchCooperativeKernel((const void*)jacobi_coop_kernel, dim3(ctas), dim3(kJacThreads), args, smem, st));
-      if (rec) CK(cudaEventRecord(rec->b, st));
+      const int count = (int)(order.size() - big);
+      char* d = upload({{order.data() + big, count * sizeof(EighTask)}}, off);
+      eigh_small_launch((const EighTask*)(d + off[0]), count, st);
       ++launches;
     }
+    for (size_t i = 0; i < big;) {
+      size_t j = i, bytes = 0;
+      for (; j < big; ++j) {
+        bytes += 2 * (size_t)order[j].n * order[j].n * sizeof(double);
+        if (j > i && bytes > dig_pool_cap()) break;
+      }
+      eigh_large(std::vector<EighTask>(order.begin() + i, order.begin() + j));
+      i = j;
+    }
+    if (rec) CK(cudaEventRecord(rec->b, st));
+    if (recs.size() > 4096) drain();
+  }
+  void eigh_large(const std::vector<EighTask>& t) {
+    if (tri_cap == 0) {
+      tri_cap = tridiag_max_ctas(sms);
+      if (tri_cap < 2) throw std::runtime_error("cuda: eigensolver needs two co-resident CTAs");
+    }
+    std::vector<int> sizes;
+    size_t sum = 0, sq = 0;
+    for (auto& x : t) {
+      sizes.push_back(x.n);
+      sum += x.n;
+      sq += (size_t)x.n * x.n;
+    }
+    if (sum > (size_t)INT32_MAX) throw std::runtime_error("eigensolver: batch beyond 2^31 rows");
+    const DcPlan plan = dc_plan(sizes);
+    const std::vector<JacBatch> batches = jac_plan_batches(sizes, tri_cap);
+    std::vector<DcNode> nodes = plan.leaves;
+    std::vector<size_t> first;
+    for (auto& level : plan.merges) {
+      first.push_back(nodes.size());
+      nodes.insert(nodes.end(), level.begin(), level.end());
+    }
+    // one allocation: matrices, descriptors, flat arrays
+    size_t at = 0;
+    auto take = [&](size_t bytes) {
+      const size_t o = at;
+      at += (bytes + 255) & ~size_t(255);
+      return o;
+    };
+    const size_t oB0 = take(sq * 8), oB1 = take(sq * 8), oX = take(4 * sum * 8);
+    size_t oD[11];
+    for (auto& o : oD) o = take(sum * 8);
+    const size_t oI = take(3 * sum * 4), oC = take(2 * sum * 4), oR = take(sum * sizeof(DcRot));
+    const size_t oW = take(tridiag_wide(sizes[0], (int)sum, tri_cap) * 8);
+    const size_t obar = take(t.size() * sizeof(unsigned)), osc = take(t.size() * 8);
+    const size_t om = take(t.size() * sizeof(DcMatrix)), on = take(nodes.size() * sizeof(DcNode));
+    char* ws = nullptr;
+    if (cudaMallocAsync((void**)&ws, at, st) != cudaSuccess) {
+      cudaGetLastError();
+      throw std::runtime_error("out of device memory (" + std::to_string(at) + " bytes)");
+    }
+    struct Free {
+      char* p;
+      cudaStream_t s;
+      ~Free() { cudaFreeAsync(p, s); }
+    } release{ws, st};
+    auto dbl = [&](size_t o) { return (double*)(ws + o); };
+    DcArrays ar{};
+    ar.d = dbl(oD[0]);
+    ar.e = dbl(oD[1]);
+    ar.tau = dbl(oD[2]);
+    ar.val = dbl(oD[3]);
+    ar.dl = dbl(oD[4]);
+    ar.zl = dbl(oD[5]);
+    ar.mu = dbl(oD[6]);
+    ar.zhat = dbl(oD[7]);
+    ar.ninv = dbl(oD[8]);
+    ar.rho = dbl(oD[9]);
+    ar.org = (int*)(ws + oI);
+    ar.pos = ar.org + sum;
+    ar.inv = ar.pos + sum;
+    ar.count = (int*)(ws + oC);
+    ar.rot = (DcRot*)(ws + oR);
+    ar.scale = dbl(osc);
+    ar.wide = dbl(oW);
+    std::vector<DcMatrix> mats;
+    std::vector<int> ctas;
+    size_t sqo = 0;
+    int off = 0;
+    for (const JacBatch& b : batches) {
+      int c = 0;
+      for (size_t k = b.begin; k < b.end; ++k) {
+        const int n = t[k].n, g = b.g[k - b.begin];
+        DcMatrix m{};
+        m.A = const_cast<double*>(t[k].A);
+        m.w = t[k].w;
+        m.V = t[k].V;
+        m.B[0] = dbl(oB0) + sqo;
+        m.B[1] = dbl(oB1) + sqo;
+        m.xch = dbl(oX) + 4 * (size_t)off;
+        m.bar = (unsigned*)(ws + obar) + k;
+        m.n = n;
+        m.off = off;
+        m.g = g;
+        m.cta0 = c;
+        m.rows_in_smem = tridiag_rows_fit(n, g);
+        m.levels = dc_levels(n);
+        mats.push_back(m);
+        c += g;
+        off += n;
+        sqo += (size_t)n * n;
+      }
+      ctas.push_back(c);
+    }
+    std::vector<size_t> uo;
+    char* d = upload({{mats.data(), mats.size() * sizeof(DcMatrix)}, {nodes.data(), nodes.size() * sizeof(DcNode)}}, uo);
+    CK(cudaMemcpyAsync(ws + om, d + uo[0], mats.size() * sizeof(DcMatrix), cudaMemcpyDeviceToDevice, st));
+    CK(cudaMemcpyAsync(ws + on, d + uo[1], nodes.size() * sizeof(DcNode), cudaMemcpyDeviceToDevice, st));
+    CK(cudaMemsetAsync(ws + obar, 0, t.size() * sizeof(unsigned), st));
+    const DcMatrix* dm = (const DcMatrix*)(ws + om);
+    const DcNode* dn = (const DcNode*)(ws + on);
+    for (size_t b = 0; b < batches.size(); ++b)
+      tridiag_launch(dm, (int)batches[b].begin, (int)(batches[b].end - batches[b].begin), ctas[b], ar, flag(),
+                     wait_ns_, st);
+    dc_leaves_launch(dm, dn, (int)plan.leaves.size(), ar, st);
+    launches += (long)batches.size() + 1;
+    for (size_t l = 0; l < plan.merges.size(); ++l) {
+      const auto& level = plan.merges[l];
+      int largest = 0, positions = 0;
+      size_t prefix = 0;
+      std::vector<GemmGroup> groups;
+      std::vector<GemmSeg> segs;
+      for (const DcNode& nd : level) {
+        const DcMatrix& m = mats[nd.mat];
+        const int N = nd.n1 + nd.n2, n = m.n;
+        largest = std::max(largest, N);
+        positions += N;
+        prefix = std::max(prefix, (size_t)(m.B[0] - mats[0].B[0]) + (size_t)n * n);
+        const size_t o = (size_t)nd.lo * n + nd.lo, o2 = o + (size_t)nd.n1 * n + nd.n1;
+        double* out = m.B[(l + 1) & 1] + o;
+        const double* in = m.B[l & 1];
+        // rows of the merged vectors: U^T (the children's vectors)
+        groups.push_back({out, N, nd.n1, n, (int)segs.size(), 1});
+        segs.push_back({m.V + o, in + o, nd.n1, n, n, 1, 0, 1.0});
+        groups.push_back({out + nd.n1, N, nd.n2, n, (int)segs.size(), 1});
+        segs.push_back({m.V + o + (size_t)nd.n1 * n, in + o2, nd.n2, n, n, 1, 0, 1.0});
+      }
+      dc_merge_launch(dm, dn + first[l], (int)level.size(), positions, largest, (int)l, ar, st);
+      CK(cudaMemsetAsync(mats[0].B[(l + 1) & 1], 0, prefix * sizeof(double), st));
+      gemm_impl(groups, segs, Precision::FP64, nullptr);
+      launches += 6;
+    }
+    dc_back_launch(dm, (int)mats.size(), (int)sum, sizes[0], ar, st);
+    ++launches;
+    CK(cudaGetLastError());
   }
 };
 

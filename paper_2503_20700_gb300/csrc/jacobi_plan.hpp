@@ -1,6 +1,6 @@
-// Host planning of the batched Jacobi eigensolver (the density-matrix
-// sectors of a decimation): which matrices share a cooperative launch of one
-// CTA per SM, and how many CTAs each matrix gets.
+// Host planning of the batched tridiagonalisation (the density-matrix sectors
+// of a decimation): which matrices share a cooperative launch of one CTA per
+// SM, and how many CTAs each matrix gets.
 #pragma once
 #include <algorithm>
 #include <stdexcept>
@@ -8,15 +8,17 @@
 
 namespace dmrg {
 
-constexpr int kJacSmemN = 112;  // largest matrix of the one-CTA shared-memory path
+constexpr int kJacSmemN = 112;  // largest matrix that may stay on one CTA
 
-// Modelled time of an n x n matrix on g CTAs, in SM clocks (FP64 rate of 2
-// operations a clock; a group barrier about 6000 clocks): the group sizes of
-// a batch minimise the slowest matrix.
+// Modelled time of an n x n matrix on g CTAs, in SM clocks: n steps of three
+// float64 FMAs per entry of the trailing matrix (n^2 / 3 entries on average,
+// two FMAs a clock), what every CTA repeats (about 4500 clocks) and, in a
+// group, a barrier (about 4000); the group sizes of a batch minimise the
+// slowest matrix.
 inline double jac_cost(int n, int g) {
-  const double rounds = std::max(1, ((n + 1) & ~1) - 1);
-  const double ops = 2.0 * (double)n * n;  // clocks of the FP64 work of a round on one SM
-  return rounds * (g == 1 ? ops + 1000.0 : 1.15 * ops / g + 6000.0);
+  const double steps = std::max(1, n - 1);
+  const double fma = 0.5 * (double)n * n;
+  return steps * (g == 1 ? fma + 4500.0 : fma / g + 8500.0);
 }
 
 // g[k] of batch tasks (descending n) start at their minimum; spare CTAs go to
@@ -26,7 +28,7 @@ inline void jac_assign_groups(const std::vector<int>& n, std::vector<int>& g, in
     size_t k = 0;
     for (size_t i = 1; i < n.size(); ++i)
       if (jac_cost(n[i], g[i]) > jac_cost(n[k], g[k])) k = i;
-    const int gmax = std::max(2, std::min(32, ((n[k] + 1) & ~1) / 2));
+    const int gmax = std::max(2, std::min(std::max(32, n[k] / 16), ((n[k] + 1) & ~1) / 2));
     int ng = g[k] + 1;
     while (ng <= gmax && ng - g[k] <= spare && jac_cost(n[k], ng) >= jac_cost(n[k], g[k])) ++ng;
     if (ng > gmax || ng - g[k] > spare) break;
