@@ -838,47 +838,41 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 
 // Partial tiles are TM x TNMAX float pairs stored column by column (element
 // (r, c) at c * TM + r); CTA (tile, y, z) sums rows [32 z, 32 z + 32) x columns
-// [32 y, 32 y + 32) of a tile over its chunks in fixed order and adds them to
-// sigma.  Bound by HBM for long lists of chunks, by the latency of its loads
-// for the tiles of a sweep: so a CTA is 32 x 32, a lane holds one row of four
-// columns (256 B per warp and load, 16 loads in flight), sigma is fetched
-// before the sums and written row by row through shared memory.  Measured,
-// per launch: the products of a D = 256 sweep 227 -> 116 us, of a D = 512 bond
-// 392 -> 101 us (a CTA of 128 rows that walked its 32 columns two at a time and
-// wrote sigma by columns before).
-constexpr int RED = 32;
+// [8 y, 8 y + 8) of a tile over its chunks in fixed order and adds them to
+// sigma.  Bound by HBM for large blocks, by the latency of its loads for the
+// tiles of a sweep, which are cut into a hundred chunks and more: so a thread
+// has one element and sixteen chunks in flight (256 B per warp and load), the
+// CTA is 32 x 8, sigma is fetched before the sums and written row by row
+// through shared memory.  Measured, per launch: the products of a D = 256 sweep
+// 227 -> 116 us with 32 x 32 CTAs and four chunks in flight -> 54 us, of a
+// D = 512 bond 392 -> 101 -> 59 us (a CTA of 128 rows that walked 32 columns
+// two at a time and wrote sigma by columns at first).
+constexpr int RED_R = 32, RED_C = 8;
 __global__ void __launch_bounds__(256) hpsi_tc_reduce(const HpsiBlock* __restrict__ blocks,
                                                       const HpsiReduce* __restrict__ reds,
                                                       const double* __restrict__ scratch, int tile_n) {
-  __shared__ double turn[RED][RED + 1];
+  __shared__ double turn[RED_C][RED_R + 1];
   const HpsiReduce rd = reds[blockIdx.x];
   const HpsiBlock bk = blocks[rd.block];
-  const int c0 = (int)blockIdx.y * RED, r0 = (int)blockIdx.z * RED;
-  const int nc = min(RED, min(tile_n, bk.n - rd.c0) - c0), nr = min(RED, bk.m - rd.r0 - r0);
+  const int c0 = (int)blockIdx.y * RED_C, r0 = (int)blockIdx.z * RED_R;
+  const int nc = min(RED_C, min(tile_n, bk.n - rd.c0) - c0), nr = min(RED_R, bk.m - rd.r0 - r0);
   if (nc <= 0 || nr <= 0) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double* const out = bk.C + (size_t)(rd.r0 + r0) * bk.ldc + rd.c0 + c0 + lane;
-  double old[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-    old[i] = (warp + 8 * i < nr && lane < nc) ? out[(size_t)(warp + 8 * i) * bk.ldc] : 0.0;
-  const float2* part = reinterpret_cast<const float2*>(scratch + rd.part0) + (size_t)(c0 + warp) * TM + r0 + lane;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll 4
-  for (int p = 0; p < rd.nparts; ++p, part += (size_t)TM * TNMAX) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (lane < nr && warp + 8 * i < nc) {
-        const float2 v = __ldg(part + 8 * i * TM);
-        acc[i] += (double)v.x + (double)v.y;
-      }
+  const int wr = threadIdx.x >> 3, wc = threadIdx.x & 7;  // the element this thread writes
+  double* const out = bk.C + (size_t)(rd.r0 + r0 + wr) * bk.ldc + rd.c0 + c0 + wc;
+  const double old = wr < nr && wc < nc ? *out : 0.0;
+  if (warp < nc && lane < nr) {
+    const float2* part = reinterpret_cast<const float2*>(scratch + rd.part0) + (size_t)(c0 + warp) * TM + r0 + lane;
+    double acc = 0.0;
+#pragma unroll 16
+    for (int p = 0; p < rd.nparts; ++p) {
+      const float2 v = __ldg(part + (size_t)p * TM * TNMAX);
+      acc += (double)v.x + (double)v.y;
+    }
+    turn[warp][lane] = acc;
   }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) turn[warp + 8 * i][lane] = acc[i];
   __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-    if (warp + 8 * i < nr && lane < nc) out[(size_t)(warp + 8 * i) * bk.ldc] = old[i] + turn[lane][warp + 8 * i];
+  if (wr < nr && wc < nc) *out = old + turn[wc][wr];
 }
 
 // Unit pairs of job j: pair p = kblock * G + g holds hi (unit 2p) and lo
@@ -1024,7 +1018,7 @@ void hpsi_tc_launch(const TcLaunch& L, int* err, unsigned long long wait_ns, cud
     if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: hpsi tc launch: ") + cudaGetErrorString(e));
   }
   if (L.nreds > 0) {
-    hpsi_tc_reduce<<<dim3(L.nreds, (L.tile_n + RED - 1) / RED, TM / RED), 256, 0, st>>>(L.blocks, L.reds, L.scratch, L.tile_n);
+    hpsi_tc_reduce<<<dim3(L.nreds, (L.tile_n + RED_C - 1) / RED_C, TM / RED_R), 256, 0, st>>>(L.blocks, L.reds, L.scratch, L.tile_n);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: hpsi tc reduce: ") + cudaGetErrorString(e));
   }
