@@ -139,7 +139,18 @@ class Backend {
   virtual void axpby(double* y, double a, const double* x, double b, size_t len) = 0;
   // y[t] = x[t] / (d[t] - e) with a guarded denominator (Davidson preconditioner)
   virtual void precondition(double* y, const double* x, const double* d, double e, size_t len) = 0;
-  // Symmetric eigendecompositions (FP64, one CTA per matrix).
+  // Steps of a Davidson iteration on m rows of V and HV (length and stride len).
+  // x = sum_i c[i] V_i (c on the host), r = sum_i c[i] HV_i - e x and, with t,
+  // t = r / (d - e) with a guarded denominator (r without d); returns |r|^2.
+  virtual double dav_residual(double* x, double* r, double* t, const double* d, const double* V, const double* HV,
+                              int m, size_t len, const double* c, double e) = 0;
+  // t = V_m orthogonalised twice against the rows before it and normalised
+  // (zero if less than 1e-14 is left), also into `in`
+  virtual void dav_orthonormalise(double* V, int m, size_t len, double* in) = 0;
+  // hv = y and out[i] = V_i . y, i < m (host); returns the norm that the last
+  // dav_orthonormalise found.  Synchronises the stream.
+  virtual double dav_project(const double* V, int m, size_t len, const double* y, double* hv, double* out) = 0;
+  // Symmetric eigendecompositions (FP64).
   virtual void eigh(const std::vector<EighTask>& tasks) = 0;
 
   // Counters (for the FLOP/byte accounting of the benchmark).
@@ -154,9 +165,15 @@ class Backend {
   size_t window_peak = 0;  // high-water mark since the caller last reset it
   // Device-side interval on the backend stream (CUDA events): mark_begin()
   // then mark_end() returns the elapsed milliseconds (synchronising the
-  // stream).  Two independent slots (0, 1) so that intervals can nest.
+  // stream).  Independent slots (0, 1, 2) so that intervals can nest; mark_stop
+  // ends the interval without waiting, mark_ms reads it.
   virtual void mark_begin(int slot = 0) = 0;
-  virtual double mark_end(int slot = 0) = 0;
+  virtual void mark_stop(int slot) = 0;
+  virtual double mark_ms(int slot) = 0;
+  double mark_end(int slot = 0) {
+    mark_stop(slot);
+    return mark_ms(slot);
+  }
   virtual void set_profile(bool on) = 0;
 
  protected:

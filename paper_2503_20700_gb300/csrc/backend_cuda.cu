@@ -5,7 +5,8 @@
 //   gemm_f64_kernel     C += sum_s alpha_s op(A_s) op(B_s)    (FP64 on the FMA pipe: small blocks)
 //   gemm_digits_kernel (gemm_digits.cu)                        (FP64 as exact bf16 digit products on tcgen05)
 //   gemm_tf32x3 (gemm_split.cu)                                (split-FP32 tensor-core path)
-//   dots/combine/axpby  Davidson vector algebra (FP64, deterministic two-stage reductions)
+//   dots/combine/axpby  vector algebra (FP64, deterministic two-stage reductions); davidson.cu has the
+//                       fused steps of an iteration
 //   eigh.cu             batched FP64 eigensolver: Jacobi for small matrices, tridiagonalisation on groups of
 //                       CTAs and divide and conquer for larger ones
 // All kernels are bounded loops over their inputs; the one wait on other CTAs,
@@ -22,6 +23,7 @@
 #include <vector>
 
 #include "backend.hpp"
+#include "davidson.cuh"
 #include "eigh.cuh"
 #include "gemm_digits.cuh"
 #include "gemm_split.cuh"
@@ -267,18 +269,22 @@ class CudaBackend : public Backend {
     }
     recs.clear();
   }
-  cudaEvent_t mb_[2] = {nullptr, nullptr}, me_[2] = {nullptr, nullptr};
+  static constexpr int kSlots = 3;
+  cudaEvent_t mb_[kSlots] = {}, me_[kSlots] = {};
   void mark_begin(int slot) override {
-    if (slot < 0 || slot > 1) throw std::logic_error("internal: event slot out of range");
+    if (slot < 0 || slot >= kSlots) throw std::logic_error("internal: event slot out of range");
     if (!mb_[slot]) {
       CK(cudaEventCreate(&mb_[slot]));
       CK(cudaEventCreate(&me_[slot]));
     }
     CK(cudaEventRecord(mb_[slot], st));
   }
-  double mark_end(int slot) override {
-    if (slot < 0 || slot > 1 || !mb_[slot]) throw std::logic_error("internal: event slot not started");
+  void mark_stop(int slot) override {
+    if (slot < 0 || slot >= kSlots || !mb_[slot]) throw std::logic_error("internal: event slot not started");
     CK(cudaEventRecord(me_[slot], st));
+  }
+  double mark_ms(int slot) override {
+    if (slot < 0 || slot >= kSlots || !mb_[slot]) throw std::logic_error("internal: event slot not started");
     CK(cudaEventSynchronize(me_[slot]));
     float ms = 0.f;
     CK(cudaEventElapsedTime(&ms, mb_[slot], me_[slot]));
@@ -318,17 +324,19 @@ class CudaBackend : public Backend {
     }
     for (auto& r : recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
     for (auto e : pool) cudaEventDestroy(e);
-    for (int k = 0; k < 2; ++k)
+    for (int k = 0; k < kSlots; ++k)
       if (mb_[k]) {
         cudaEventDestroy(mb_[k]);
         cudaEventDestroy(me_[k]);
       }
     if (dtask) cudaFreeAsync(dtask, st);
     if (part) cudaFreeAsync(part, st);
+    if (dav_dev) cudaFreeAsync(dav_dev, st);
     if (dflag) cudaFreeAsync(dflag, st);
     if (htask) cudaFreeHost(htask);
     cudaStreamSynchronize(st);
     if (dig_err) cudaFreeHost(dig_err);
+    if (dav_host) cudaFreeHost(dav_host);
     cudaStreamDestroy(st);
   }
   std::string name() const override { return "cuda"; }
@@ -784,6 +792,60 @@ class CudaBackend : public Backend {
     precond_kernel<<<nb, 256, 0, st>>>(y, x, d, e, len);
     ++launches;
     CK(cudaGetLastError());
+  }
+  // Davidson: partials, counters and coefficients on the device, results in
+  // mapped host memory ([0] |r|^2, [1] the norm, [2 ...] the projections)
+  double* dav_dev = nullptr;
+  double* dav_host = nullptr;
+  int dav_rows = 0;
+  DavWork dav_work(int m) {
+    if (m > dav_rows) {
+      CK(cudaStreamSynchronize(st));
+      if (dav_dev) CK(cudaFreeAsync(dav_dev, st));
+      if (dav_host) CK(cudaFreeHost(dav_host));
+      dav_dev = dav_host = nullptr;
+      dav_rows = 0;
+      const int rows = std::max(m, 32);
+      // per row: partials, a counter, two coefficients; and |t|^2
+      const size_t n = (size_t)rows * (kDavParts + 3) + 1;
+      CK(cudaMallocAsync((void**)&dav_dev, n * sizeof(double), st));
+      CK(cudaMemsetAsync(dav_dev, 0, n * sizeof(double), st));
+      CK(cudaHostAlloc((void**)&dav_host, (size_t)(rows + 2) * sizeof(double), cudaHostAllocMapped));
+      dav_rows = rows;
+    }
+    return DavWork{dav_dev, (unsigned*)(dav_dev + (size_t)dav_rows * kDavParts), dav_host};
+  }
+  double* dav_coefs() { return dav_dev + (size_t)dav_rows * (kDavParts + 1); }
+  double dav_residual(double* x, double* r, double* t, const double* d, const double* V, const double* HV, int m,
+                      size_t len, const double* c, double e) override {
+    const DavWork w = dav_work(m + 1);
+    if (m > kDavCoefs) {
+      CK(cudaMemcpyAsync(dav_coefs(), c, m * sizeof(double), cudaMemcpyHostToDevice, st));
+      c = dav_coefs();
+    }
+    dav_ritz_launch(x, r, t, d, V, HV, m, len, c, e, w, w.host, st);
+    ++launches;
+    CK(cudaStreamSynchronize(st));
+    return ((volatile double*)w.host)[0];
+  }
+  void dav_orthonormalise(double* V, int m, size_t len, double* in) override {
+    const DavWork w = dav_work(m + 1);
+    double *t = V + (size_t)m * len, *c = dav_coefs(), *norm2 = c + 2 * (size_t)dav_rows;
+    for (int pass = 0; pass < 2; ++pass) {
+      dav_dots_launch(V, m, len, t, nullptr, w, c, st);
+      dav_subtract_launch(t, V, m, len, c, w, pass ? norm2 : nullptr, st);
+    }
+    dav_normalise_launch(t, in, len, norm2, w.host + 1, st);
+    launches += 5;
+  }
+  double dav_project(const double* V, int m, size_t len, const double* y, double* hv, double* out) override {
+    const DavWork w = dav_work(m + 1);
+    dav_dots_launch(V, m, len, y, hv, w, w.host + 2, st);
+    ++launches;
+    CK(cudaStreamSynchronize(st));
+    check_digits();
+    for (int i = 0; i < m; ++i) out[i] = ((volatile double*)w.host)[2 + i];
+    return ((volatile double*)w.host)[1];
   }
   // Matrices up to kEighSmall: one launch of the Jacobi kernel.  Larger ones:
   // cooperative launches of the tridiagonalisation (largest matrices first,

@@ -1,5 +1,6 @@
 // Host planner of the spin-adapted two-site DMRG (see dmrg.hpp).
 #include "dmrg.hpp"
+#include "small_eigh.hpp"
 #include "hpsi_fused.cuh"
 #include "hpsi_tc.cuh"
 #include "host_pool.hpp"
@@ -1917,13 +1918,8 @@ double Engine::davidson(HPsiPlan& plan, double* psi, int* iters) {
   const int M = std::max(4, opt_.max_space);
   double* V = (double*)be_->alloc((size_t)M * len * sizeof(double));
   double* HV = (double*)be_->alloc((size_t)M * len * sizeof(double));
-  double* dv = (double*)be_->alloc((size_t)(M * M + 4 * M + 8) * sizeof(double));
-  double* dA = dv;
-  double* dw = dv + M * M;
-  double* dZ = dw + M;        // reused for coefficient vectors (M)
-  double* dc = dZ + M;
-  double* dEv = (double*)be_->alloc((size_t)M * M * sizeof(double));
-  std::vector<double> A((size_t)M * M, 0.0), w(M), Z((size_t)M * M), c(M), tmpv(M);
+  double* dZ = (double*)be_->alloc((size_t)M * sizeof(double));  // coefficients of a restart
+  std::vector<double> A((size_t)M * M, 0.0), w(M), Z((size_t)M * M), tmpv(M);
   // guess: provided psi (if nonzero) else a deterministic pseudo-random vector
   {
     std::vector<double> h(len);
@@ -1941,27 +1937,23 @@ double Engine::davidson(HPsiPlan& plan, double* psi, int* iters) {
     for (double& x : h) x /= nrm;
     be_->copy_h2d(V, h.data(), len * sizeof(double));
   }
-  auto dot_host = [&](const double* a, const double* b) {
-    be_->dots(a, 1, len, len, b, dc);
-    double r;
-    be_->copy_d2h(&r, dc, sizeof(double));
-    return r;
-  };
+  // sigma of the vector in plan.in; tmpv = V . sigma over i + 1 rows and
+  // sigma into HV_i.  Returns the norm left by the last orthonormalisation.
   auto apply = [&](int i) {
-    be_->copy_d2d(plan.in, V + (size_t)i * len, len * sizeof(double));
-    auto t0 = std::chrono::steady_clock::now();
-    if (call_ms_) be_->mark_begin();
+    be_->mark_begin(2);
     apply_hpsi(plan);
-    if (call_ms_) call_ms_->push_back(be_->mark_end());
-    be_->sync();
+    be_->mark_stop(2);
+    const double tn = be_->dav_project(V, i + 1, len, plan.out, HV + (size_t)i * len, tmpv.data());
     if (plan.prec == Precision::TC_TF32X3) be_->check_device_flag();
-    auto t1 = std::chrono::steady_clock::now();
-    stats_.hpsi_seconds += std::chrono::duration<double>(t1 - t0).count();
+    const double ms = be_->mark_ms(2);
+    if (call_ms_) call_ms_->push_back(ms);
+    stats_.hpsi_seconds += 1e-3 * ms;
     stats_.hpsi_flops += plan.flops;
     stats_.hpsi_calls += 1;
-    be_->copy_d2d(HV + (size_t)i * len, plan.out, len * sizeof(double));
+    return tn;
   };
   int m = 1;
+  be_->copy_d2d(plan.in, V, len * sizeof(double));
   apply(0);
   double e = 0.0;
   double* x = psi;  // result vector
@@ -1972,26 +1964,17 @@ double Engine::davidson(HPsiPlan& plan, double* psi, int* iters) {
   double last_res = 1e300, last_tol = 0.0;
   for (it = 1; it <= opt_.max_davidson_iter; ++it) {
     // projected matrix: row/col m-1
-    be_->dots(V, m, len, len, HV + (size_t)(m - 1) * len, dc);
-    be_->copy_d2h(tmpv.data(), dc, m * sizeof(double));
     for (int i = 0; i < m; ++i) A[(size_t)i * M + (m - 1)] = A[(size_t)(m - 1) * M + i] = tmpv[i];
-    // small eigenproblem on the device
     std::vector<double> Am((size_t)m * m);
     for (int i = 0; i < m; ++i)
       for (int j = 0; j < m; ++j) Am[(size_t)i * m + j] = 0.5 * (A[(size_t)i * M + j] + A[(size_t)j * M + i]);
-    be_->copy_h2d(dA, Am.data(), Am.size() * sizeof(double));
-    be_->eigh({EighTask{dA, dw, dEv, m}});
-    be_->copy_d2h(w.data(), dw, m * sizeof(double));
-    be_->copy_d2h(Z.data(), dEv, (size_t)m * m * sizeof(double));
-    // lowest eigenpair = last row (eigenvalues descending)
-    e = w[m - 1];
-    last_gap_ = m >= 2 ? w[m - 2] - w[m - 1] : 0.0;
-    for (int i = 0; i < m; ++i) c[i] = Z[(size_t)(m - 1) * m + i];
-    be_->copy_h2d(dZ, c.data(), m * sizeof(double));
-    be_->combine(x, 0.0, V, m, len, len, dZ);
-    be_->combine(r, 0.0, HV, m, len, len, dZ);
-    be_->axpby(r, 1.0, x, -e, len);
-    double rn = std::sqrt(std::max(0.0, dot_host(r, r)));
+    small_eigh(m, Am.data(), w.data(), Z.data());
+    e = w[0];
+    last_gap_ = m >= 2 ? w[1] - w[0] : 0.0;
+    // the Ritz vector, its residual and (unless a restart moves the rows) the
+    // preconditioned residual as the next row
+    const double rn = std::sqrt(std::max(0.0, be_->dav_residual(x, r, m < M ? V + (size_t)m * len : nullptr, plan.diag,
+                                                                V, HV, m, len, Z.data(), e)));
     if (opt_.verbose > 1) std::fprintf(stderr, "  davidson it %d m %d E %.12f res %.3e\n", it, m, e, rn);
     // With split-precision H_eff psi the residual has a noise floor of about
     // 1e-7 |E| (TF32 pairs keep ~22 bits, FP32 accumulation): converge to
@@ -2012,8 +1995,8 @@ double Engine::davidson(HPsiPlan& plan, double* psi, int* iters) {
       // restart with the lowest two Ritz vectors
       std::vector<double> c2((size_t)2 * m);
       for (int i = 0; i < m; ++i) {
-        c2[i] = Z[(size_t)(m - 1) * m + i];
-        c2[m + i] = Z[(size_t)(m - 2) * m + i];
+        c2[i] = Z[i];
+        c2[m + i] = Z[m + i];
       }
       double* nV = (double*)be_->alloc((size_t)2 * len * sizeof(double));
       double* nH = (double*)be_->alloc((size_t)2 * len * sizeof(double));
@@ -2027,25 +2010,16 @@ double Engine::davidson(HPsiPlan& plan, double* psi, int* iters) {
       be_->free(nV);
       be_->free(nH);
       std::fill(A.begin(), A.end(), 0.0);
-      A[0] = w[m - 1];
-      A[(size_t)1 * M + 1] = w[m - 2];
+      A[0] = w[0];
+      A[(size_t)1 * M + 1] = w[1];
       m = 2;
+      if (plan.diag) be_->precondition(V + (size_t)m * len, r, plan.diag, e, len);
+      else be_->copy_d2d(V + (size_t)m * len, r, len * sizeof(double));
     }
-    // new direction t = (D - E)^-1 r, orthogonalised twice against V
-    double* t = V + (size_t)m * len;
-    if (plan.diag) be_->precondition(t, r, plan.diag, e, len);
-    else be_->copy_d2d(t, r, len * sizeof(double));
-    for (int pass = 0; pass < 2; ++pass) {
-      be_->dots(V, m, len, len, t, dc);
-      be_->copy_d2h(tmpv.data(), dc, m * sizeof(double));
-      for (int i = 0; i < m; ++i) tmpv[i] = -tmpv[i];
-      be_->copy_h2d(dZ, tmpv.data(), m * sizeof(double));
-      be_->combine(t, 1.0, V, m, len, len, dZ);
-    }
-    double tn = std::sqrt(std::max(0.0, dot_host(t, t)));
-    if (tn < 1e-14) break;
-    be_->axpby(t, 0.0, t, 1.0 / tn, len);
-    apply(m);
+    // new direction t = (D - E)^-1 r, orthogonalised twice against V; nothing
+    // left of it: the space is exhausted (its product is one of zeros)
+    be_->dav_orthonormalise(V, m, len, plan.in);
+    if (apply(m) < 1e-14) break;
     ++m;
   }
   if (iters) *iters = it;
@@ -2053,8 +2027,7 @@ double Engine::davidson(HPsiPlan& plan, double* psi, int* iters) {
   be_->sync();
   be_->free(V);
   be_->free(HV);
-  be_->free(dv);
-  be_->free(dEv);
+  be_->free(dZ);
   return e;
 }
 
