@@ -106,6 +106,8 @@ class Backend {
   virtual void memset0(void* p, size_t bytes) = 0;
   virtual void copy_d2d(void* dst, const void* src, size_t bytes) = 0;
   virtual void copy_h2d(void* dst, const void* src, size_t bytes) = 0;
+  // without a wait: src stays as it is until the stream is synchronised
+  virtual void copy_h2d_later(void* dst, const void* src, size_t bytes) = 0;
   virtual void copy_d2h(void* dst, const void* src, size_t bytes) = 0;
   virtual void sync() = 0;
   // Reads and clears the device error flag that bounded waits in kernels set;

@@ -18,6 +18,8 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <stdexcept>
 #include <string>
 #include <vector>
@@ -217,6 +219,73 @@ __global__ void precond_kernel(double* __restrict__ y, const double* __restrict_
   }
 }
 
+// ------------------------------------------------------------------ pinned memory
+// Page-locked blocks that outlive a backend: the host entries make one backend
+// per call, and allocating and freeing its staging memory took 0.3 to 0.4 ms
+// of each.  A block belongs to one backend between get and put (which comes
+// after the backend's stream is idle); at most kPinnedKept bytes wait for the
+// next one, more is freed.  Portable and mapped, so any device may use it.
+class PinnedPool {
+ public:
+  static PinnedPool& get() {
+    static PinnedPool* p = new PinnedPool;  // never destroyed: the driver may be gone before it
+    return *p;
+  }
+  void* take(size_t bytes, size_t* capacity) {
+    {
+      std::lock_guard<std::mutex> lock(mu_);
+      auto it = free_.lower_bound(bytes);
+      if (it != free_.end() && it->first <= 16 * std::max(bytes, kSmallest)) {
+        void* p = it->second;
+        *capacity = it->first;
+        kept_ -= it->first;
+        free_.erase(it);
+        return p;
+      }
+    }
+    size_t cap = kSmallest;
+    while (cap < bytes) cap *= 2;
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, cap, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+      cudaGetLastError();
+      throw std::runtime_error("out of pinned host memory (" + std::to_string(cap) + " bytes)");
+    }
+    *capacity = cap;
+    return p;
+  }
+  void put(void* p, size_t capacity) {
+    if (!p) return;
+    {
+      std::lock_guard<std::mutex> lock(mu_);
+      if (kept_ + capacity <= kPinnedKept) {
+        free_.emplace(capacity, p);
+        kept_ += capacity;
+        return;
+      }
+    }
+    cudaFreeHost(p);
+  }
+
+ private:
+  static constexpr size_t kSmallest = 4096, kPinnedKept = size_t(64) << 20;
+  std::mutex mu_;
+  std::multimap<size_t, void*> free_;
+  size_t kept_ = 0;
+};
+
+// Device memory in total: a constant of the device (asking for it takes 20 us)
+static size_t total_memory(int dev) {
+  static std::mutex mu;
+  static std::map<int, size_t> known;
+  std::lock_guard<std::mutex> lock(mu);
+  auto it = known.find(dev);
+  if (it != known.end()) return it->second;
+  size_t fr = 0, total = 0;
+  CK(cudaMemGetInfo(&fr, &total));
+  known[dev] = total;
+  return total;
+}
+
 // ------------------------------------------------------------------ backend
 class CudaBackend : public Backend {
  public:
@@ -224,11 +293,10 @@ class CudaBackend : public Backend {
   cudaStream_t st = nullptr;
   size_t used = 0;
   std::vector<std::pair<void*, size_t>> live;
-  // staging for task lists
-  void* dtask = nullptr;
-  size_t dtask_cap = 0;
-  void* htask = nullptr;
-  size_t htask_cap = 0;
+  // staging for task lists: a ring of pinned memory and its device copy
+  char* dtask = nullptr;
+  char* htask = nullptr;
+  size_t task_cap = 0, task_pos = 0;
   double* part = nullptr;
   size_t part_cap = 0;
   // profiling
@@ -310,8 +378,7 @@ class CudaBackend : public Backend {
     CK(cudaDeviceGetDefaultMemPool(&pool, dev));
     uint64_t thr = UINT64_MAX;
     CK(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr));
-    size_t fr = 0;
-    CK(cudaMemGetInfo(&fr, &total_mem));
+    total_mem = total_memory(dev);
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   }
   int sms = 152;
@@ -333,10 +400,10 @@ class CudaBackend : public Backend {
     if (part) cudaFreeAsync(part, st);
     if (dav_dev) cudaFreeAsync(dav_dev, st);
     if (dflag) cudaFreeAsync(dflag, st);
-    if (htask) cudaFreeHost(htask);
     cudaStreamSynchronize(st);
-    if (dig_err) cudaFreeHost(dig_err);
-    if (dav_host) cudaFreeHost(dav_host);
+    PinnedPool::get().put(htask, task_cap);
+    PinnedPool::get().put(dig_err, dig_err_cap);
+    PinnedPool::get().put(dav_host, dav_host_cap);
     cudaStreamDestroy(st);
   }
   std::string name() const override { return "cuda"; }
@@ -450,6 +517,9 @@ class CudaBackend : public Backend {
       CK(cudaStreamSynchronize(st));
     }
   }
+  void copy_h2d_later(void* d, const void* s, size_t b) override {
+    if (b) CK(cudaMemcpyAsync(d, s, b, cudaMemcpyHostToDevice, st));
+  }
   void copy_d2h(void* d, const void* s, size_t b) override {
     if (b) {
       CK(cudaMemcpyAsync(d, s, b, cudaMemcpyDeviceToHost, st));
@@ -490,24 +560,31 @@ class CudaBackend : public Backend {
       offs.push_back(tot);
       tot += (p.second + 255) & ~size_t(255);
     }
-    if (tot > htask_cap) {
+    if (tot > task_cap) {
       CK(cudaStreamSynchronize(st));
-      if (htask) CK(cudaFreeHost(htask));
-      htask_cap = std::max(tot, htask_cap * 2);
-      CK(cudaMallocHost(&htask, htask_cap));
-    }
-    if (tot > dtask_cap) {
+      PinnedPool::get().put(htask, task_cap);
+      htask = nullptr;
+      const size_t want = std::max(std::max(tot, 2 * task_cap), kTaskRing);
+      task_cap = task_pos = 0;
+      size_t cap = 0;
+      htask = (char*)PinnedPool::get().take(want, &cap);
       if (dtask) CK(cudaFreeAsync(dtask, st));
-      dtask_cap = std::max(tot, dtask_cap * 2);
-      CK(cudaMallocAsync(&dtask, dtask_cap, st));
+      dtask = nullptr;
+      CK(cudaMallocAsync((void**)&dtask, cap, st));
+      task_cap = cap;
     }
-    // the pinned staging buffer may still be in use by a previous copy
-    CK(cudaStreamSynchronize(st));
-    for (size_t i = 0; i < parts.size(); ++i)
-      std::memcpy((char*)htask + offs[i], parts[i].first, parts[i].second);
-    CK(cudaMemcpyAsync(dtask, htask, tot, cudaMemcpyHostToDevice, st));
-    return (char*)dtask;
+    if (task_pos + tot > task_cap) {
+      // around the ring: what was uploaded before has been used
+      CK(cudaStreamSynchronize(st));
+      task_pos = 0;
+    }
+    char *h = htask + task_pos, *d = dtask + task_pos;
+    task_pos += tot;
+    for (size_t i = 0; i < parts.size(); ++i) std::memcpy(h + offs[i], parts[i].first, parts[i].second);
+    CK(cudaMemcpyAsync(d, h, tot, cudaMemcpyHostToDevice, st));
+    return d;
   }
+  static constexpr size_t kTaskRing = size_t(4) << 20;  // some hundred lists between two waits
 
   void place(const std::vector<PlaceGroup>& groups, const std::vector<PlaceSeg>& segs) override {
     std::vector<PlaceTile> tiles;
@@ -635,6 +712,7 @@ class CudaBackend : public Backend {
     const size_t cap = size_t(2) << 30;
     return budget_ ? std::max<size_t>(size_t(16) << 20, std::min(cap, budget_ / 16)) : cap;
   }
+  size_t dig_err_cap = 0;
   int* dig_err = nullptr;  // host-mapped: set by a digit launch whose wait ran out
   void check_digits() {
     if (dig_err && *(volatile int*)dig_err) {
@@ -645,7 +723,7 @@ class CudaBackend : public Backend {
   void gemm_digits(const std::vector<GemmGroup>& groups, const std::vector<GemmSeg>& segs,
                    const std::vector<char>& digits) {
     if (!dig_err) {
-      CK(cudaHostAlloc((void**)&dig_err, sizeof(int), cudaHostAllocMapped));
+      dig_err = (int*)PinnedPool::get().take(sizeof(int), &dig_err_cap);
       *dig_err = 0;
     }
     DigPlanner pl;
@@ -797,12 +875,13 @@ class CudaBackend : public Backend {
   // mapped host memory ([0] |r|^2, [1] the norm, [2 ...] the projections)
   double* dav_dev = nullptr;
   double* dav_host = nullptr;
+  size_t dav_host_cap = 0;
   int dav_rows = 0;
   DavWork dav_work(int m) {
     if (m > dav_rows) {
       CK(cudaStreamSynchronize(st));
       if (dav_dev) CK(cudaFreeAsync(dav_dev, st));
-      if (dav_host) CK(cudaFreeHost(dav_host));
+      PinnedPool::get().put(dav_host, dav_host_cap);
       dav_dev = dav_host = nullptr;
       dav_rows = 0;
       const int rows = std::max(m, 32);
@@ -810,7 +889,7 @@ class CudaBackend : public Backend {
       const size_t n = (size_t)rows * (kDavParts + 3) + 1;
       CK(cudaMallocAsync((void**)&dav_dev, n * sizeof(double), st));
       CK(cudaMemsetAsync(dav_dev, 0, n * sizeof(double), st));
-      CK(cudaHostAlloc((void**)&dav_host, (size_t)(rows + 2) * sizeof(double), cudaHostAllocMapped));
+      dav_host = (double*)PinnedPool::get().take((size_t)(rows + 2) * sizeof(double), &dav_host_cap);
       dav_rows = rows;
     }
     return DavWork{dav_dev, (unsigned*)(dav_dev + (size_t)dav_rows * kDavParts), dav_host};

@@ -632,9 +632,9 @@ dmrg_status dmrg_grouped_gemm(const double* A, int64_t a_len, const double* B, i
     double* dA = (double*)be->alloc(std::max<int64_t>(a_len, 1) * sizeof(double));
     double* dB = (double*)be->alloc(std::max<int64_t>(b_len, 1) * sizeof(double));
     double* dC = (double*)be->alloc(std::max<int64_t>(c_len, 1) * sizeof(double));
-    be->copy_h2d(dA, A, a_len * sizeof(double));
-    be->copy_h2d(dB, B, b_len * sizeof(double));
-    be->copy_h2d(dC, C, c_len * sizeof(double));
+    be->copy_h2d_later(dA, A, a_len * sizeof(double));
+    be->copy_h2d_later(dB, B, b_len * sizeof(double));
+    be->copy_h2d_later(dC, C, c_len * sizeof(double));
     std::vector<dmrg::GemmGroup> gg(n_groups);
     std::vector<dmrg::GemmSeg> ss(n_segs);
     for (int g = 0; g < n_groups; ++g)
@@ -719,13 +719,14 @@ dmrg_status dmrg_hpsi_contract(const double* A, int64_t a_len, const double* P, 
   if (const char* m = check_hpsi(a_len, p_len, b_len, c_len, blocks, n_blocks, items, n_items))
     return fail(nullptr, DMRG_EINVAL, m);
   std::string err;
+  std::vector<char> lists;  // outlives the backend's stream
   std::unique_ptr<dmrg::Backend> be(dmrg::make_cuda_backend(device, &err));
   if (be) be->set_wait_ns(g_kernel_wait_ns.load());
   if (!be) return fail(nullptr, DMRG_ECUDA, err);
   try {
     auto up = [&](const double* h, int64_t n) {
       double* d = (double*)be->alloc(std::max<int64_t>(n, 1) * sizeof(double));
-      be->copy_h2d(d, h, n * sizeof(double));
+      be->copy_h2d_later(d, h, n * sizeof(double));
       return d;
     };
     double* dA = up(A, a_len);
@@ -736,7 +737,6 @@ dmrg_status dmrg_hpsi_contract(const double* A, int64_t a_len, const double* P, 
     std::vector<dmrg::HpsiItem> hi;
     double fl = 0.0;
     to_device_lists(blocks, n_blocks, items, n_items, dA, dP, dB, dC, hb, hi, &fl);
-    be->sync();
     be->set_profile(true);
     const dmrg::Precision pr = precision == DMRG_FP64           ? dmrg::Precision::FP64
                                : precision == DMRG_SPLIT_HPSI_TC ? dmrg::Precision::TC_TF32X3
@@ -768,20 +768,24 @@ dmrg_status dmrg_hpsi_contract(const double* A, int64_t a_len, const double* P, 
     size_t oct = al(oco + tp.cta_off.size() * sizeof(int));
     size_t os = al(oct + tp.cta_task.size() * sizeof(dmrg::TcSlot));
     char* d = (char*)be->alloc(os + scr * sizeof(double) + 256);
-    if (!hb.empty()) be->copy_h2d(d + ob, hb.data(), hb.size() * sizeof(dmrg::HpsiBlock));
-    if (!hi.empty()) be->copy_h2d(d + oi, hi.data(), hi.size() * sizeof(dmrg::HpsiItem));
-    if (!tp.items.empty()) be->copy_h2d(d + oc, tp.items.data(), tp.items.size() * sizeof(dmrg::TcItem));
-    if (!tasks.empty()) be->copy_h2d(d + ot, tasks.data(), tasks.size() * sizeof(dmrg::HpsiTask));
-    if (!reds.empty()) be->copy_h2d(d + orr, reds.data(), reds.size() * sizeof(dmrg::HpsiReduce));
+    // all lists in one copy
+    std::vector<dmrg::SplitJob> jobs = tp.op_jobs;
+    jobs.insert(jobs.end(), tp.psi_jobs.begin(), tp.psi_jobs.end());
+    lists.resize(os);
+    auto put = [&](size_t at, const auto& v) {
+      if (!v.empty()) std::memcpy(lists.data() + at, v.data(), v.size() * sizeof(v[0]));
+    };
+    put(ob, hb);
+    put(oi, hi);
+    put(oc, tp.items);
+    put(ot, tasks);
+    put(orr, reds);
+    put(oj, jobs);
+    put(oco, tp.cta_off);
+    put(oct, tp.cta_task);
+    be->copy_h2d_later(d, lists.data(), os);
     if (tc) {
-      std::vector<dmrg::SplitJob> jobs = tp.op_jobs;
-      jobs.insert(jobs.end(), tp.psi_jobs.begin(), tp.psi_jobs.end());
-      if (!jobs.empty()) {
-        be->copy_h2d(d + oj, jobs.data(), jobs.size() * sizeof(dmrg::SplitJob));
-        be->split((const dmrg::SplitJob*)(d + oj), (int)jobs.size(), (float*)pool);
-      }
-      if (!tp.cta_off.empty()) be->copy_h2d(d + oco, tp.cta_off.data(), tp.cta_off.size() * sizeof(int));
-      if (!tp.cta_task.empty()) be->copy_h2d(d + oct, tp.cta_task.data(), tp.cta_task.size() * sizeof(dmrg::TcSlot));
+      if (!jobs.empty()) be->split((const dmrg::SplitJob*)(d + oj), (int)jobs.size(), (float*)pool);
       dmrg::TcLaunch L;
       L.blocks = (const dmrg::HpsiBlock*)(d + ob);
       L.items = (const dmrg::TcItem*)(d + oc);
@@ -864,13 +868,16 @@ dmrg_status dmrg_hpsi_contract_noalloc(const double* dA, int64_t a_len, const do
     if (e != cudaSuccess) return fail(nullptr, DMRG_ECUDA, std::string("cuda: ") + cudaGetErrorString(e));
     cudaStream_t st = (cudaStream_t)stream;
     char* d = (char*)base;
+    // all lists in one copy (pageable: staged before the call returns)
+    std::vector<char> lists(os);
     auto put = [&](size_t off, const void* h, size_t bytes) {
-      if (bytes && e == cudaSuccess) e = cudaMemcpyAsync(d + off, h, bytes, cudaMemcpyHostToDevice, st);
+      if (bytes) std::memcpy(lists.data() + off, h, bytes);
     };
     put(ob, hb.data(), hb.size() * sizeof(dmrg::HpsiBlock));
     put(oi, hi.data(), hi.size() * sizeof(dmrg::HpsiItem));
     put(ot, tasks.data(), tasks.size() * sizeof(dmrg::HpsiTask));
     put(orr, reds.data(), reds.size() * sizeof(dmrg::HpsiReduce));
+    if (os && e == cudaSuccess) e = cudaMemcpyAsync(d, lists.data(), os, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
       dmrg::hpsi_launch((const dmrg::HpsiBlock*)(d + ob), (const dmrg::HpsiItem*)(d + oi),
                         (const dmrg::HpsiTask*)(d + ot), (int)tasks.size(),
@@ -902,7 +909,7 @@ dmrg_status dmrg_eigh_batched(const double* mats, const int* n, int count, doubl
     double* dA = (double*)be->alloc(std::max<size_t>(tot, 1) * sizeof(double));
     double* dV = (double*)be->alloc(std::max<size_t>(tot, 1) * sizeof(double));
     double* dw = (double*)be->alloc(std::max<size_t>(wt, 1) * sizeof(double));
-    be->copy_h2d(dA, mats, tot * sizeof(double));
+    be->copy_h2d_later(dA, mats, tot * sizeof(double));
     std::vector<dmrg::EighTask> t;
     size_t o = 0, ow = 0;
     for (int i = 0; i < count; ++i) {

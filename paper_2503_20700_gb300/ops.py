@@ -5,6 +5,7 @@ Argument marshalling only; the computation runs in the library's kernels.
 from __future__ import annotations
 
 import ctypes
+import struct
 
 import numpy as np
 
@@ -34,6 +35,28 @@ class HpsiBlock(ctypes.Structure):
 
 
 _lib = None
+
+def _packer(kind):
+    fmt = "@" + "".join({ctypes.c_int64: "q", ctypes.c_int: "i", ctypes.c_double: "d"}[t] for _, t in kind._fields_)
+    return struct.Struct(fmt + "x" * (ctypes.sizeof(kind) - struct.calcsize(fmt)))
+
+
+# the same layouts for struct, which fills a list of some hundred rows in a
+# fifth of the time that as many ctypes constructors take
+_PACK = {k: _packer(k) for k in (GemmSeg, GemmGroup, HpsiItem, HpsiBlock)}
+
+
+def _rows(kind, rows):
+    """ctypes array of `kind` (at least one element) from a list of tuples."""
+    out = (kind * max(1, len(rows)))()
+    pack = _PACK[kind].pack
+    try:
+        data = b"".join([pack(*r) for r in rows])
+        ctypes.memmove(out, data, len(data))
+    except struct.error:  # shorter rows, values out of range: as ctypes takes them
+        for i, r in enumerate(rows):
+            out[i] = kind(*r)
+    return out
 
 
 def bind(lib):
@@ -80,8 +103,7 @@ def grouped_gemm(A, B, C, groups, segs, precision=0, device=0):
     A = np.ascontiguousarray(A, dtype=np.float64)
     B = np.ascontiguousarray(B, dtype=np.float64)
     assert C.dtype == np.float64 and C.flags.c_contiguous
-    ga = (GemmGroup * max(1, len(groups)))(*[GemmGroup(*g) for g in groups])
-    sa = (GemmSeg * max(1, len(segs)))(*[GemmSeg(*s) for s in segs])
+    ga, sa = _rows(GemmGroup, groups), _rows(GemmSeg, segs)
     st = lib.dmrg_grouped_gemm(_dp(A), A.size, _dp(B), B.size, _dp(C), C.size, ga, len(groups),
                                sa, len(segs), precision, device)
     if st != 0:
@@ -98,8 +120,7 @@ def hpsi_contract_noalloc(dA, a_len, dP, p_len, dB, b_len, dC, c_len, blocks, it
     device must not overlap (they share one static scratch)."""
     from . import load, DmrgError
     lib = load()
-    ba = (HpsiBlock * max(1, len(blocks)))(*[HpsiBlock(*b) for b in blocks])
-    ia = (HpsiItem * max(1, len(items)))(*[HpsiItem(*i) for i in items])
+    ba, ia = _rows(HpsiBlock, blocks), _rows(HpsiItem, items)
     st = lib.dmrg_hpsi_contract_noalloc(dA, a_len, dP, p_len, dB, b_len, dC, c_len, ba, len(blocks), ia,
                                         len(items), precision, device, stream or None)
     if st != 0:
@@ -128,8 +149,7 @@ def hpsi_contract(A, P, B, C, blocks, items, precision=0, device=0):
     P = np.ascontiguousarray(P, dtype=np.float64)
     B = np.ascontiguousarray(B, dtype=np.float64)
     assert C.dtype == np.float64 and C.flags.c_contiguous
-    ba = (HpsiBlock * max(1, len(blocks)))(*[HpsiBlock(*b) for b in blocks])
-    ia = (HpsiItem * max(1, len(items)))(*[HpsiItem(*i) for i in items])
+    ba, ia = _rows(HpsiBlock, blocks), _rows(HpsiItem, items)
     st = lib.dmrg_hpsi_contract(_dp(A), A.size, _dp(P), P.size, _dp(B), B.size, _dp(C), C.size,
                                 ba, len(blocks), ia, len(items), precision, device)
     if st != 0:
@@ -144,16 +164,17 @@ def eigh_batched(mats, device=0):
     from . import load, DmrgError
     lib = load()
     ns = np.array([m.shape[0] for m in mats], dtype=np.int32)
-    flat = np.concatenate([np.ascontiguousarray(m, dtype=np.float64).ravel() for m in mats])
-    w = np.zeros(int(ns.sum()))
-    v = np.zeros_like(flat)
+    flat = np.concatenate([m.ravel() if type(m) is np.ndarray and m.dtype == np.float64 else
+                           np.ascontiguousarray(m, dtype=np.float64).ravel() for m in mats])
+    w = np.empty(int(ns.sum()))
+    v = np.empty_like(flat)
     st = lib.dmrg_eigh_batched(_dp(flat), ns.ctypes.data_as(ctypes.POINTER(ctypes.c_int)),
                                len(mats), _dp(w), _dp(v), device)
     if st != 0:
         raise DmrgError(st, lib.dmrg_last_error(None).decode())
     out, o, ow = [], 0, 0
-    for n in ns:
-        out.append((w[ow:ow + n].copy(), v[o:o + n * n].reshape(n, n).copy()))
+    for n in ns.tolist():  # disjoint parts of the two results
+        out.append((w[ow:ow + n], v[o:o + n * n].reshape(n, n)))
         o += n * n
         ow += n
     return out
@@ -225,7 +246,7 @@ def rotation_backward(K, G, device=0):
 def transform(R, h, L, device=0):
     """(R^T h R, R^T L^k R) on the device."""
     R, h, L = _c(R), _c(h), _c(L)
-    ho, Lo = np.zeros_like(h), np.zeros_like(L)
+    ho, Lo = np.empty_like(h), np.empty_like(L)  # written whole; zeroing first took most of a call
     _call("casscf_transform", _dp(R), _dp(h), _dp(L), L.shape[0], h.shape[0], _dp(ho), _dp(Lo), device)
     return ho, Lo
 
