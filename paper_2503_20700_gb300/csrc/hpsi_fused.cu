@@ -241,12 +241,14 @@ __global__ void __launch_bounds__(256) hpsi_tf32x3_kernel(const HpsiBlock* __res
 // time, and so are those of X, so a 20 x 20 block costs 512 FMAs a k instead
 // of a padded 4096.  The two shared-memory reads per FMA this takes (one
 // broadcast, one along the lanes) are a quarter of the FMA's own time.  128
-// threads and 52 KB: four CTAs an SM hide each other's loads.
-// Measured against 64 x 64 tiles padded to their size: 367 -> 59 us a product
-// of a 10-site D = 64 run (blocks of 5..40), 6.82 -> 3.20 ms a whole call with
-// sectors of 40..208.
+// threads and 44 KB: five CTAs an SM hide each other's loads.  1024 outputs
+// rather than 2048: the rows of a large block make twice the tasks, whose last
+// wave is then short.
+// Measured against 64 x 64 tiles padded to their size: 367 -> 21 us a product
+// of a 10-site D = 64 run (blocks of 5..40), 6.2 -> 1.69 ms with sectors of
+// 40..208 (0.96 TFLOP/s, three quarters of the pipe).
 constexpr int kF64Threads = 128;
-constexpr int kF64Slots = 16;                       // outputs per thread
+constexpr int kF64Slots = 8;                        // outputs per thread
 constexpr int kF64Out = kF64Threads * kF64Slots;    // outputs of a tile
 constexpr int kF64Cols = 256;                       // columns of a tile
 constexpr int kF64Rows = 128;                       // rows of a tile
@@ -287,12 +289,11 @@ __device__ __forceinline__ void f64_products(int ns, double (&acc)[kF64Slots], c
 #define F64_CASE(N) \
   case N: f64_products<N>(acc, off, a, b, bstep, kn); break
     F64_CASE(1); F64_CASE(2); F64_CASE(3); F64_CASE(4); F64_CASE(5); F64_CASE(6); F64_CASE(7); F64_CASE(8);
-    F64_CASE(9); F64_CASE(10); F64_CASE(11); F64_CASE(12); F64_CASE(13); F64_CASE(14); F64_CASE(15); F64_CASE(16);
 #undef F64_CASE
   }
 }
 
-__global__ void __launch_bounds__(kF64Threads, 4) hpsi_f64_kernel(const HpsiBlock* __restrict__ blocks,
+__global__ void __launch_bounds__(kF64Threads, 5) hpsi_f64_kernel(const HpsiBlock* __restrict__ blocks,
                                                                   const HpsiItem* __restrict__ items,
                                                                   const HpsiTask* __restrict__ tasks,
                                                                   double* __restrict__ scratch) {
@@ -316,8 +317,10 @@ __global__ void __launch_bounds__(kF64Threads, 4) hpsi_f64_kernel(const HpsiBloc
     double s[kF64Slots];
 #pragma unroll
     for (int i = 0; i < kF64Slots; ++i) s[i] = 0.0;
+    HpsiItem next = items[tk.it_begin];
     for (int ii = tk.it_begin; ii < tk.it_begin + tk.it_count; ++ii) {
-      const HpsiItem it = items[ii];
+      const HpsiItem it = next;
+      if (ii + 1 < tk.it_begin + tk.it_count) next = items[ii + 1];
       int jc_begin = 0, jc_end = it.kb;
       if (it.B == nullptr) {  // identity on the right: only sigma's own columns
         jc_begin = tk.c0;
@@ -429,7 +432,7 @@ __global__ void __launch_bounds__(kF64Threads, 4) hpsi_f64_kernel(const HpsiBloc
 }
 
 // C += the partial tiles of a sigma tile, in a fixed order: bound by the
-// latency of its loads, so a thread has one output and eight partials in flight
+// latency of its loads, so a thread has one output and sixteen partials in flight
 __global__ void __launch_bounds__(128) hpsi_f64_reduce_kernel(const HpsiBlock* __restrict__ blocks,
                                                               const HpsiReduce* __restrict__ reds,
                                                               const double* __restrict__ scratch) {
@@ -444,7 +447,7 @@ __global__ void __launch_bounds__(128) hpsi_f64_reduce_kernel(const HpsiBlock* _
   const double old = *c;
   const double* p = scratch + rd.part0 + e;
   double acc = 0.0;
-#pragma unroll 8
+#pragma unroll 16
   for (int i = 0; i < rd.nparts; ++i) acc += __ldg(p + (long long)i * outs);
   *c = old + acc;
 }
@@ -468,11 +471,18 @@ __global__ void hpsi_reduce_kernel(const HpsiBlock* __restrict__ blocks, const H
 
 namespace {
 
-// tiles of 64 x 64 in item chunks of equal count
-size_t plan_square(const std::vector<HpsiBlock>& blocks, std::vector<HpsiTask>& tasks, std::vector<HpsiReduce>& reds) {
+size_t plan_bytes(size_t part, size_t tasks, size_t reds);
+
+// items per chunk of tiles of 64 x 64, and the chunks of a block
+int square_items(const std::vector<HpsiBlock>& blocks) {
   long long tile_items = 0;
   for (auto& b : blocks) tile_items += (long long)b.item_count * ((b.m + T - 1) / T) * ((b.n + T - 1) / T);
-  const int max_items = (int)std::max<long long>(4, tile_items / (8 * 152) + 1);
+  return (int)std::max<long long>(4, tile_items / (8 * 152) + 1);
+}
+
+// tiles of 64 x 64 in item chunks of equal count
+size_t plan_square(const std::vector<HpsiBlock>& blocks, std::vector<HpsiTask>& tasks, std::vector<HpsiReduce>& reds) {
+  const int max_items = square_items(blocks);
   long long part = 0;
   for (size_t b = 0; b < blocks.size(); ++b) {
     const HpsiBlock& bk = blocks[b];
@@ -497,18 +507,36 @@ size_t plan_square(const std::vector<HpsiBlock>& blocks, std::vector<HpsiTask>& 
   return (size_t)part;
 }
 
-// Clocks of an item on a tile: two FMAs a clock, and the latency of the loads
-// of its k-steps (about 1200 clocks each, shared by four CTAs an SM).
+// bytes of the lists and partial tiles of that plan
+size_t square_bytes(const std::vector<HpsiBlock>& blocks) {
+  const int max_items = square_items(blocks);
+  size_t part = 0, tasks = 0, reds = 0;
+  for (const HpsiBlock& bk : blocks) {
+    if (bk.item_count == 0 || bk.m == 0 || bk.n == 0) continue;
+    const size_t tiles = (size_t)((bk.m + T - 1) / T) * ((bk.n + T - 1) / T);
+    const size_t nch = (bk.item_count + max_items - 1) / max_items;
+    tasks += tiles * nch;
+    if (nch > 1) {
+      reds += tiles;
+      part += tiles * nch * T * T;
+    }
+  }
+  return plan_bytes(part, tasks, reds);
+}
+
+// Clocks of an item on a tile: two FMAs a clock, and the latency of the item's
+// and its k-steps' loads (a thousand clocks and more each, shared by the CTAs
+// of an SM).
 double f64_item_cost(const HpsiItem& it, int mt, int nt) {
   const double ka = it.A ? it.ka : 0.0, kb = it.kb;
   double c = 0.5 * mt * (ka * (it.B ? kb : std::min<double>(kb, nt)) + (it.B ? kb * nt : 0.0));
-  return c + 300.0 * (1.0 + ka / KS * ((kb + kF64Chunk - 1) / kF64Chunk) + (it.B ? kb / KS : 0.0));
+  return c + 800.0 + 300.0 * (ka / KS * ((kb + kF64Chunk - 1) / kF64Chunk) + (it.B ? kb / KS : 0.0));
 }
 
 // Tiles of f64_tile, the items of a tile in chunks of about `target` clocks;
 // target < 0: one task per column tile, walking all rows and items.
-size_t plan_f64(const std::vector<HpsiBlock>& blocks, const std::vector<HpsiItem>& items, double target,
-                std::vector<HpsiTask>& tasks, std::vector<HpsiReduce>& reds) {
+size_t plan_f64(const std::vector<HpsiBlock>& blocks, const std::vector<double>& cost, const std::vector<double>& run,
+                double target, std::vector<HpsiTask>& tasks, std::vector<HpsiReduce>& reds) {
   tasks.clear();
   reds.clear();
   long long part = 0;
@@ -524,15 +552,10 @@ size_t plan_f64(const std::vector<HpsiBlock>& blocks, const std::vector<HpsiItem
       continue;
     }
     // cuts into chunks of equal cost, the same for every tile of the block
-    double total = 0.0;
-    for (int i = first; i < last; ++i) total += f64_item_cost(items[i], mt, nt);
-    const int nch = (int)std::max(1.0, std::min<double>(bk.item_count, total / target));
+    const int nch = (int)std::max(1.0, std::min<double>(bk.item_count, cost[b] / target));
     cut.assign(1, first);
-    double run = 0.0;
-    for (int i = first; i < last; ++i) {
-      run += f64_item_cost(items[i], mt, nt);
-      if (run >= total * cut.size() / nch && i + 1 < last && (int)cut.size() < nch) cut.push_back(i + 1);
-    }
+    for (int i = first; i + 1 < last && (int)cut.size() < nch; ++i)
+      if (run[i] >= cost[b] * cut.size() / nch) cut.push_back(i + 1);
     cut.push_back(last);
     const int n = (int)cut.size() - 1;
     for (int r0 = 0; r0 < bk.m; r0 += mt)
@@ -548,9 +571,9 @@ size_t plan_f64(const std::vector<HpsiBlock>& blocks, const std::vector<HpsiItem
   return (size_t)part;
 }
 
-size_t plan_bytes(size_t part, const std::vector<HpsiTask>& tasks, const std::vector<HpsiReduce>& reds) {
-  return part * sizeof(double) + ((tasks.size() * sizeof(HpsiTask) + 255) & ~size_t(255)) +
-         ((reds.size() * sizeof(HpsiReduce) + 255) & ~size_t(255));
+size_t plan_bytes(size_t part, size_t tasks, size_t reds) {
+  return part * sizeof(double) + ((tasks * sizeof(HpsiTask) + 255) & ~size_t(255)) +
+         ((reds * sizeof(HpsiReduce) + 255) & ~size_t(255));
 }
 
 }  // namespace
@@ -559,34 +582,43 @@ size_t hpsi_plan_tasks(const std::vector<HpsiBlock>& blocks, const std::vector<H
                        std::vector<HpsiTask>& tasks, std::vector<HpsiReduce>& reds, size_t* nominal_bytes) {
   tasks.clear();
   reds.clear();
-  const size_t square = plan_square(blocks, tasks, reds);
-  const size_t nominal = plan_bytes(square, tasks, reds);
+  if (prec != Precision::FP64) {
+    const size_t part = plan_square(blocks, tasks, reds);
+    if (nominal_bytes) *nominal_bytes = plan_bytes(part, tasks.size(), reds.size());
+    return part;
+  }
+  const size_t nominal = square_bytes(blocks);
   if (nominal_bytes) *nominal_bytes = nominal;
-  if (prec != Precision::FP64) return square;
-  // Two waves of the CTAs that the SMs hold at once (152 x 4), no chunk below
-  // 8000 clocks (a tenth of which a partial tile's store and reduction cost).
+  // Three tasks per CTA that the SMs hold at once (152 x 5): the last wave is
+  // then a third.  No chunk below 3500 clocks: an item of a small block is
+  // about 800 of latency, so a chunk is at most four of them where the launch
+  // does not fill the SMs anyway (sectors of 2..23: 41 -> 27 us against chunks
+  // of 8000 clocks).
   // Lists and partial tiles take no more than those of the 64 x 64 plan would,
-  // or than 8 MB of what the allocation-free entry has: longer chunks, at last
-  // one task per column tile.
+  // or than what the allocation-free entry has: longer chunks, at last one task
+  // per column tile.
   const size_t lists = (blocks.size() * sizeof(HpsiBlock) + 255) / 256 * 256 +
                        (items.size() * sizeof(HpsiItem) + 255) / 256 * 256;
   const size_t left = lists < kNoAllocScratchBytes ? kNoAllocScratchBytes - lists : 0;
-  const size_t limit = std::max(nominal, std::min(size_t(8) << 20, left));
+  const size_t limit = std::max(nominal, left);
+  // cost[b], run[i]: of the block's items, of those up to item i
+  std::vector<double> cost(blocks.size(), 0.0), run(items.size(), 0.0);
   double total = 0.0;
-  for (const HpsiBlock& bk : blocks) {
+  for (size_t b = 0; b < blocks.size(); ++b) {
+    const HpsiBlock& bk = blocks[b];
     if (bk.item_count == 0 || bk.m == 0 || bk.n == 0) continue;
     int mt, nt;
     f64_tile(bk.m, bk.n, mt, nt);
-    double c = 0.0;
-    for (int i = bk.item_begin; i < bk.item_begin + bk.item_count; ++i) c += f64_item_cost(items[i], mt, nt);
-    total += c * ((bk.m + mt - 1) / mt) * ((bk.n + nt - 1) / nt);
+    for (int i = bk.item_begin; i < bk.item_begin + bk.item_count; ++i)
+      run[i] = cost[b] += f64_item_cost(items[i], mt, nt);
+    total += cost[b] * ((bk.m + mt - 1) / mt) * ((bk.n + nt - 1) / nt);
   }
-  double target = std::max(8000.0, total / (152 * 4 * 2));
+  double target = std::max(3500.0, total / (152 * 5 * 3));
   for (int k = 0; k < 6; ++k, target *= 4.0) {
-    const size_t part = plan_f64(blocks, items, target, tasks, reds);
-    if (plan_bytes(part, tasks, reds) <= limit) return part;
+    const size_t part = plan_f64(blocks, cost, run, target, tasks, reds);
+    if (plan_bytes(part, tasks.size(), reds.size()) <= limit) return part;
   }
-  return plan_f64(blocks, items, -1.0, tasks, reds);
+  return plan_f64(blocks, cost, run, -1.0, tasks, reds);
 }
 
 void hpsi_launch(const HpsiBlock* blocks, const HpsiItem* items, const HpsiTask* tasks, int ntasks,
