@@ -112,7 +112,9 @@ typedef struct {
                              products with a new sector histogram run the
                              candidate schedules in turn (every one computes
                              the full product) and the fastest is kept for
-                             that histogram.  0 (default): the first candidate.
+                             that histogram.  0 (default): the first candidate
+                             (without its clusters where the sectors' tiles
+                             would leave their slots empty).
                              Results differ between schedules only by FP32
                              summation order                                  */
 } dmrg_opts;

@@ -748,10 +748,15 @@ dmrg_status dmrg_hpsi_contract(const double* A, int64_t a_len, const double* P, 
     void* pool = nullptr;
     size_t scr;
     if (tc) {
-      const dmrg::TcShape shape = dmrg::tc_shape_candidates()[g_kernel_tc_cand.load()];
-      const int tc_ctas = dmrg::hpsi_tc_max_ctas(shape.cluster);
-      dmrg::hpsi_tc_prepare(hb, hi, [&](size_t bytes) { return pool = be->alloc(bytes); }, tp,
-                            tc_ctas > 0 ? tc_ctas : be->sm_count() / shape.cluster * shape.cluster, shape);
+      const int cand = g_kernel_tc_cand.load();
+      dmrg::TcShape shape = dmrg::tc_shape_candidates()[cand];
+      auto ctas = [&](int cluster) {
+        const int n = dmrg::hpsi_tc_max_ctas(cluster);
+        return n > 0 ? n : be->sm_count() / cluster * cluster;
+      };
+      dmrg::hpsi_tc_operands(hb, hi, [&](size_t bytes) { return pool = be->alloc(bytes); }, tp);
+      if (cand == 0) shape = dmrg::tc_sized_shape(shape, hb, tp.items, ctas(shape.cluster), ctas(1));
+      dmrg::hpsi_tc_schedule(hb, tp, shape, ctas(shape.cluster));
       tasks = tp.tasks;
       reds = tp.reds;
       scr = tp.scratch;

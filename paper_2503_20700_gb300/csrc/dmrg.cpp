@@ -1707,8 +1707,10 @@ void Engine::plan_hpsi(Block& Le, Block& Re, HPsiPlan& plan) {
         while (plan.tc_cand < (int)nc && rec.ms[plan.tc_cand] >= 0) ++plan.tc_cand;
       }
     }
-    hpsi_tc_schedule(blocks, tp, tc_shape_candidates()[plan.tc_cand],
-                     tc_ctas_for(tc_shape_candidates()[plan.tc_cand].cluster));
+    TcShape shape = tc_shape_candidates()[plan.tc_cand];
+    if (!opt_.tc_autotune)
+      shape = tc_sized_shape(shape, blocks, tp.items, tc_ctas_for(shape.cluster), tc_ctas_for(1));
+    hpsi_tc_schedule(blocks, tp, shape, tc_ctas_for(shape.cluster));
     if (opt_.debug_bounds) {
       const std::string bad = tc_plan_check(tp, blocks);
       if (!bad.empty()) throw std::logic_error("internal: tcgen05 plan: " + bad);

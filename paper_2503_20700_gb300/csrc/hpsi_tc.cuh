@@ -138,6 +138,14 @@ void hpsi_tc_prepare(const std::vector<HpsiBlock>& blocks, const std::vector<Hps
 void hpsi_tc_operands(const std::vector<HpsiBlock>& blocks, const std::vector<HpsiItem>& items,
                       const std::function<void*(size_t)>& alloc, TcPlan& plan);
 void hpsi_tc_schedule(const std::vector<HpsiBlock>& blocks, TcPlan& plan, const TcShape& shape, int ncta = 0);
+// `shape`, with clusters of one in place of two where the sigma blocks' tiles
+// would leave so many cluster slots empty that the modelled work of the launch
+// is a tenth less without clusters: a block of up to 128 x 256 is one tile, and
+// half of its cluster a ghost.  Measured, kernel time per product: D = 256
+// sweep 329 -> 224 us, D = 512 bond 718 -> 378 us.  ncta, ncta1: CTAs of a launch in clusters of
+// two, of one.  Partial tiles and sums are the same either way.
+TcShape tc_sized_shape(const TcShape& shape, const std::vector<HpsiBlock>& blocks, const std::vector<TcItem>& items,
+                       int ncta, int ncta1);
 // Key of the sector histogram of a contraction (block shapes in 64-row and
 // 64-column steps with their item counts on a log scale, and the CTA count):
 // contractions with equal keys share an autotuned shape.

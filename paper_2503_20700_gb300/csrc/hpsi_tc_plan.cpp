@@ -72,6 +72,29 @@ void hpsi_tc_prepare(const std::vector<HpsiBlock>& blocks, const std::vector<Hps
   hpsi_tc_schedule(blocks, plan, shape, ncta);
 }
 
+TcShape tc_sized_shape(const TcShape& shape, const std::vector<HpsiBlock>& blocks, const std::vector<TcItem>& items,
+                       int ncta, int ncta1) {
+  if (shape.cluster != 2 || ncta < 2 || ncta1 < 1) return shape;
+  // CTA slots x work: in clusters of two, pairs of column tiles share stage 1,
+  // and the last tile of an odd row is paired with another row's or a ghost
+  double two = 0.0, one = 0.0;
+  for (const HpsiBlock& bk : blocks) {
+    if (bk.item_count == 0 || bk.m == 0 || bk.n == 0) continue;
+    const int mt = ceil_div(bk.m, TM), nt = ceil_div(bk.n, shape.tile_n);
+    const int N = std::min(shape.tile_n, (bk.n + 15) & ~15);
+    double s1 = 0.0, s2 = 0.0;
+    for (int k = bk.item_begin; k < bk.item_begin + bk.item_count; ++k) {
+      s1 += stage1_cost(items[k].ka, items[k].kb);
+      s2 += stage2_cost(items[k].kb, N);
+    }
+    two += 2.0 * mt * (nt / 2) * (0.5 * s1 + s2) + (nt % 2 ? 2.0 * ceil_div(mt, 2) * (s1 + s2) : 0.0);
+    one += (double)mt * nt * (s1 + s2);
+  }
+  TcShape r = shape;
+  if (one / ncta1 < 0.9 * (two / ncta)) r.cluster = 1;
+  return r;
+}
+
 void hpsi_tc_operands(const std::vector<HpsiBlock>& blocks, const std::vector<HpsiItem>& items,
                       const std::function<void*(size_t)>& alloc, TcPlan& plan) {
   plan = TcPlan();
