@@ -926,7 +926,7 @@ class CudaBackend : public Backend {
     for (int i = 0; i < m; ++i) out[i] = ((volatile double*)w.host)[2 + i];
     return ((volatile double*)w.host)[1];
   }
-  // Matrices up to kEighSmall: one launch of the Jacobi kernel.  Larger ones:
+  // Matrices up to kEighSmall (kEighLeaf beside larger ones): one launch of the Jacobi kernel.  Larger ones:
   // cooperative launches of the tridiagonalisation (largest matrices first,
   // group sizes from jac_assign_groups), then the levels of merges with their
   // products on the grouped GEMM, then the reflectors.  Work space (two more
@@ -938,8 +938,12 @@ class CudaBackend : public Backend {
     std::vector<EighTask> order(tasks);
     std::stable_sort(order.begin(), order.end(), [](const EighTask& x, const EighTask& y) { return x.n > y.n; });
     while (!order.empty() && order.back().n <= 0) order.pop_back();
+    if (order.empty()) return;
+    // beside larger matrices the middle ones (17..32) cost nothing there; alone
+    // they are faster by Jacobi (one launch)
+    const int small = order[0].n > kEighSmall ? kEighLeaf : kEighSmall;
     size_t big = 0;
-    while (big < order.size() && order[big].n > kEighSmall) ++big;
+    while (big < order.size() && order[big].n > small) ++big;
     Rec* rec = nullptr;
     if (profiling) {
       recs.push_back(Rec{ev(), ev(), 0.0, big ? 4 : 3});
@@ -993,12 +997,12 @@ class CudaBackend : public Backend {
       at += (bytes + 255) & ~size_t(255);
       return o;
     };
-    const size_t oB0 = take(sq * 8), oB1 = take(sq * 8), oX = take(4 * sum * 8);
+    const size_t oB0 = take(sq * 8), oB1 = take(sq * 8), oP = take(sum * sizeof(unsigned));
     size_t oD[11];
     for (auto& o : oD) o = take(sum * 8);
     const size_t oI = take(3 * sum * 4), oC = take(2 * sum * 4), oR = take(sum * sizeof(DcRot));
     const size_t oW = take(tridiag_wide(sizes[0], (int)sum, tri_cap) * 8);
-    const size_t obar = take(t.size() * sizeof(unsigned)), osc = take(t.size() * 8);
+    const size_t oX = take(8 * sum * 8), obar = take(t.size() * sizeof(unsigned)), osc = take(t.size() * 8);
     const size_t om = take(t.size() * sizeof(DcMatrix)), on = take(nodes.size() * sizeof(DcNode));
     char* ws = nullptr;
     if (cudaMallocAsync((void**)&ws, at, st) != cudaSuccess) {
@@ -1043,7 +1047,8 @@ class CudaBackend : public Backend {
         m.V = t[k].V;
         m.B[0] = dbl(oB0) + sqo;
         m.B[1] = dbl(oB1) + sqo;
-        m.xch = dbl(oX) + 4 * (size_t)off;
+        m.xch = dbl(oX) + 8 * (size_t)off;
+        m.peak = (unsigned*)(ws + oP) + off;
         m.bar = (unsigned*)(ws + obar) + k;
         m.n = n;
         m.off = off;
@@ -1062,7 +1067,7 @@ class CudaBackend : public Backend {
     char* d = upload({{mats.data(), mats.size() * sizeof(DcMatrix)}, {nodes.data(), nodes.size() * sizeof(DcNode)}}, uo);
     CK(cudaMemcpyAsync(ws + om, d + uo[0], mats.size() * sizeof(DcMatrix), cudaMemcpyDeviceToDevice, st));
     CK(cudaMemcpyAsync(ws + on, d + uo[1], nodes.size() * sizeof(DcNode), cudaMemcpyDeviceToDevice, st));
-    CK(cudaMemsetAsync(ws + obar, 0, t.size() * sizeof(unsigned), st));
+    CK(cudaMemsetAsync(ws + oX, 0, osc - oX, st));  // the exchange and the barriers
     const DcMatrix* dm = (const DcMatrix*)(ws + om);
     const DcNode* dn = (const DcNode*)(ws + on);
     for (size_t b = 0; b < batches.size(); ++b)

@@ -6,9 +6,9 @@
 // (this file's predecessor) spent 13 n^3 FMAs and 10 n group barriers on a
 // matrix.  Here a matrix costs n^3 FMAs and n barriers of tridiagonalisation,
 // n^3 FMAs of reflectors, and GEMMs on the tensor cores.  Measured, the 13
-// density matrices of 9..601 of a decimation: 184 ms before; now 12.2 ms, of
-// which the tridiagonalisation 6.7, the reflectors 2.8, the merges 2.1 with
-// their products, the small matrices and leaves 0.6; the largest error of the
+// density matrices of 9..601 of a decimation: 184 ms before; now 11.2 ms, of
+// which the tridiagonalisation 6.1, the reflectors 2.8, the merges 1.9 with
+// their products, the small matrices and leaves 0.4; the largest error of the
 // eigenvectors 3e-12 -> 4e-13.
 #include <algorithm>
 #include <cmath>
@@ -255,20 +255,27 @@ __global__ void __launch_bounds__(SMALL_THREADS) eigh_small_kernel(const EighTas
 }
 
 // ---------------------------------------------------------------- tridiagonalisation
-// T = Q^T A Q by reflectors H_k = 1 - tau v v^T (v_{k+1} = 1), the trailing
-// matrix kept whole and updated at once by - v w^T - w v^T.  The CTAs of a
-// group hold its rows interleaved, in shared memory where they fit.  All of
-// them know the next row, v and w, so a step needs one exchange: every CTA
-// publishes its part of p = A v and the owner of the next row that row before
-// its update, and after one group barrier everyone forms w, the updated row
-// and the next reflector, the same in every CTA.  The update of a row and its
-// product with the next v are one pass.
+// T = Q^T A Q by reflectors H_k = 1 - c v v^T, the trailing matrix kept whole
+// and updated at once by - v w^T - w v^T.  The CTAs of a group hold its rows
+// interleaved, in shared memory where they fit.  All of them know the next row,
+// v and w, so a step needs one exchange: every CTA publishes its part of
+// p = A v and the owner of the next row that row before its update, and with
+// both everyone forms w, the updated row and the next reflector, the same in
+// every CTA.  The update of a row and its product with the next v are one pass.
+// What is published carries its step in the same 16 bytes, so a reader waits
+// for the value itself and the exchange is one trip through L2 in place of a
+// barrier (fence, arrival, poll) and a read.  A step takes the place of the one
+// two before: everyone who reads a step publishes in the next (a CTA with
+// nothing to publish there leaves without reading), and everyone waits for all
+// of that before it publishes once more.
 // Bound by the float64 pipe (a warp-wide operation holds a quarter of an SM
 // for 64 clocks): three FMAs per entry, n^3 in all, and what every CTA repeats,
 // so a CTA is four warps, one per quarter, each with four rows in flight that
-// share the reads of v and w and one tree of sums; then by the barrier (about
-// 1.5 us a step).  With sixteen warps the sums, square roots and divisions
-// that every warp repeats took 6 us a step.
+// share the reads of v and w and one tree of sums.  The rest of a step is a
+// chain of latencies: v is not scaled (no division before the pass, the
+// division for c runs while the others' parts travel), the norm comes from an
+// inverse square root.  Measured, the tridiagonalisation of 13 matrices of 9..601:
+// 7.7 ms with sixteen warps and a barrier, 6.7 with four, 6.1 now.
 constexpr int TRI_WARPS = 4, TRI_THREADS = 32 * TRI_WARPS, TRI_ROWS = 4;
 constexpr size_t kTriSmem = 220 * 1024;
 
@@ -281,6 +288,21 @@ __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
   return t;
+}
+// a value and the step it belongs to, written and read as one
+__device__ __forceinline__ void publish(double2* at, double x, long long step) {
+  asm volatile("{\n.reg .b128 v;\nmov.b128 v, {%1, %2};\nst.relaxed.gpu.global.b128 [%0], v;\n}\n" ::"l"(at),
+               "l"(__double_as_longlong(x)), "l"(step)
+               : "memory");
+}
+__device__ __forceinline__ bool published(const double2* at, long long step, double& x) {
+  long long v, t;
+  asm volatile("{\n.reg .b128 v;\nld.relaxed.gpu.global.b128 v, [%2];\nmov.b128 {%0, %1}, v;\n}\n"
+               : "=l"(v), "=l"(t)
+               : "l"(at)
+               : "memory");
+  x = __longlong_as_double(v);
+  return t == step;
 }
 // waits until `target` CTAs have arrived; false when the wait ran out (a bound
 // of 0: when it was not over at its first probe)
@@ -308,16 +330,18 @@ __device__ void tridiag_one(const DcMatrix& mt, const DcArrays& ar, int mat, int
                             int* ok_s, int* err, unsigned long long wait_ns) {
   const int n = mt.n, g = mt.g, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   double* const A = mt.A;
-  double* const v = sm;          // of the step
-  double* const vo = v + n;      // of the step before, and its w
-  double* const wo = vo + n;
-  double* const x = wo + n;      // the trailing matrix's first row
-  double* const rows = x + n;    // kSmem: row lr g + me at lr n
-  const int nloc = (n - me + g - 1) / g;
+  double* v = sm;                // row k of the trailing matrix, then the reflector
+  double* vo = v + n;            // the reflector before, and its w
+  double* x = vo + n;            // the next row
+  double* const wo = x + n;
+  double* const pl = wo + n;     // p
+  double* const rows = pl + n;   // kSmem: row lr g + me at lr n
+  double* const first = red + 2 * TRI_WARPS;  // x[k + 1], by parity of k
+  const int nloc = (n - me + g - 1) / g, scribe = (n - 1) % g;
   auto row = [&](int lr) { return kSmem ? rows + (size_t)lr * n : A + (size_t)(lr * g + me) * n; };
-  // own rows, and the largest entry of all: one exchange
-  unsigned mx = 0u, arrived = g;
-  unsigned* const peak = (unsigned*)(mt.xch + 2 * n);
+  // own rows, and the largest entry of all: one barrier
+  unsigned mx = 0u;
+  unsigned* const peak = (unsigned*)mt.peak;
   double s = 0.0, scale, inv;
   for (int lr = warp; lr < nloc; lr += TRI_WARPS) {
     const double* src = A + (size_t)(lr * g + me) * n;
@@ -330,62 +354,67 @@ __device__ void tridiag_one(const DcMatrix& mt, const DcArrays& ar, int mat, int
   }
   if (tid == 0) *ok_s = 1;
   for (int j = tid; j < n; j += TRI_THREADS) {
-    x[j] = __ldcg(A + j);
+    v[j] = __ldcg(A + j);
     vo[j] = wo[j] = 0.0;
   }
   mx = block_max(mx, (unsigned*)red);
   if (g > 1) {
     if (tid == 0) __stcg(peak + me, mx);
-    if (!group_barrier(mt.bar, arrived, ok_s, wait_ns)) goto fail;
+    if (!group_barrier(mt.bar, g, ok_s, wait_ns)) goto fail;
     mx = 0u;
     for (int i = tid; i < g; i += TRI_THREADS) mx = max(mx, __ldcg(peak + i));
     mx = block_max(mx, (unsigned*)red);
   }
   power_of_two(mx, scale, inv);
-  if (me == 0 && tid == 0) ar.scale[mat] = scale;
+  if (me == scribe && tid == 0) ar.scale[mat] = scale;
   for (int lr = warp; lr < nloc; lr += TRI_WARPS) {
     double* const a = row(lr);
     for (int j = lane; j < n; j += 32) a[j] *= inv;
   }
-  for (int j = tid; j < n; j += TRI_THREADS) x[j] *= inv;
-  __syncthreads();
-  for (int j = 2 + tid; j < n; j += TRI_THREADS) s = fma(x[j], x[j], s);
+  for (int j = tid; j < n; j += TRI_THREADS) {
+    const double y = v[j] * inv;
+    v[j] = y;
+    if (j == 1) first[0] = y;
+    if (j > 1) s = fma(y, y, s);
+  }
+  __syncthreads();  // red is free again
   for (int k = 0; k + 1 < n; ++k) {
-    // the reflector of x[k + 1 ...], s = this thread's part of |x[k + 2 ...]|^2
+    // the reflector of v[k + 1 ...], s = this thread's part of |v[k + 2 ...]|^2
     s = block_sum(s, red);
-    const double alpha = x[k + 1];
-    double tau = 0.0, beta = alpha, f = 0.0;
+    const double alpha = first[k & 1];
     // a tail below 1e-30 of the matrix is left out (its squares would lose
     // digits to underflow, and H its orthogonality)
-    if (s > 1e-60) {
-      beta = -copysign(sqrt(fma(alpha, alpha, s)), alpha);
-      tau = (beta - alpha) / beta;
-      f = 1.0 / (alpha - beta);
-    }
-    for (int j = k + 1 + tid; j < n; j += TRI_THREADS)
-      v[j] = tau == 0.0 ? 0.0 : (j == k + 1 ? 1.0 : x[j] * f);
-    if (me == 0 && tid == 0) {
-      ar.d[mt.off + k] = x[k];
-      ar.e[mt.off + k] = beta;
-      ar.tau[mt.off + k] = tau;
+    const bool reflect = s > 1e-60;
+    const double s2 = fma(alpha, alpha, s), norm = reflect ? s2 * rsqrt(s2) : 0.0;
+    const double v1 = alpha + copysign(norm, alpha);
+    if (tid == 0) v[k + 1] = v1;
+    if (me == scribe && tid == 0) {
+      ar.d[mt.off + k] = v[k];
+      ar.e[mt.off + k] = reflect ? -copysign(norm, alpha) : alpha;
     }
     __syncthreads();
-    double* const pub = mt.xch + (size_t)(k & 1) * 2 * n;  // p, then the next row
-    const int live = k < me ? 0 : (k - me) / g + 1;        // first local row beyond k
-    if (live < nloc && live * g + me == k + 1) {
+    const long long step = k + 1;
+    double2* const pub = (double2*)mt.xch + (size_t)(k & 1) * 2 * n;  // p, then the next row
+    const int live = k < me ? 0 : (k - me) / g + 1;                   // first local row beyond k
+    if (g > 1 && live < nloc && live * g + me == k + 1) {
       // the next row before this step's update (its last update is below)
       const double* a = row(live);
       const double vi = vo[k + 1], wi = wo[k + 1];
-      for (int j = k + 1 + tid; j < n; j += TRI_THREADS) __stcg(pub + n + j, fma(-wi, vo[j], fma(-vi, wo[j], a[j])));
+      // rows in global memory: the scribe overwrites this one with a reflector,
+      // after what this CTA stored there
+      if (!kSmem) __threadfence();
+      for (int j = k + 1 + tid; j < n; j += TRI_THREADS) publish(pub + n + j, fma(-wi, vo[j], fma(-vi, wo[j], a[j])), step);
       __syncthreads();
     }
     for (int lr = live + TRI_ROWS * warp; lr < nloc; lr += TRI_ROWS * TRI_WARPS) {
       double* a[TRI_ROWS];
       double vi[TRI_ROWS], wi[TRI_ROWS], acc[TRI_ROWS];
+      bool keep[TRI_ROWS];  // the next row is the scribe's from here on
 #pragma unroll
       for (int r = 0; r < TRI_ROWS; ++r) {
         const int q = min(lr + r, nloc - 1);  // a row twice: the same values, stored once
         a[r] = row(q);
+        keep[r] = g == 1 || q * g + me != k + 1;
         vi[r] = vo[q * g + me];
         wi[r] = wo[q * g + me];
         acc[r] = 0.0;
@@ -398,7 +427,7 @@ __device__ void tridiag_one(const DcMatrix& mt, const DcArrays& ar, int mat, int
 #pragma unroll
           for (int r = 0; r < TRI_ROWS; ++r) {
             const double y = fma(-wi[r], vj, fma(-vi[r], wj, a[r][j]));
-            a[r][j] = y;
+            if (kSmem || keep[r]) a[r][j] = y;
             acc[r] = fma(y, nj, acc[r]);
           }
         }
@@ -409,7 +438,7 @@ __device__ void tridiag_one(const DcMatrix& mt, const DcArrays& ar, int mat, int
           for (int r = 0; r < TRI_ROWS - 1; ++r)
             if (r < rows_here) {
               const double y = fma(-wi[r], vj, fma(-vi[r], wj, a[r][j]));
-              a[r][j] = y;
+              if (kSmem || keep[r]) a[r][j] = y;
               acc[r] = fma(y, nj, acc[r]);
             }
         }
@@ -424,41 +453,84 @@ __device__ void tridiag_one(const DcMatrix& mt, const DcArrays& ar, int mat, int
 #pragma unroll
       for (int d = 4; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
       const int r = lane >> 3;
-      if ((lane & 7) == 0 && r < rows_here) __stcg(pub + (lr + r) * g + me, t);
+      if ((lane & 7) == 0 && r < rows_here) {
+        if (g > 1) publish(pub + (lr + r) * g + me, t, step);
+        else pl[lr + r] = t;
+      }
     }
     // row k of the matrix is done: it keeps the reflector
-    if (k % g == me)
+    if (me == scribe)
       for (int j = k + 1 + tid; j < n; j += TRI_THREADS) A[(size_t)k * n + j] = v[j];
+    // no rows after the next one: nothing to publish any more, so nobody would
+    // wait for this CTA's reading
+    if (me != scribe && (nloc - 1) * g + me <= k + 1) return;
+    const double c = reflect ? 1.0 / fma(fabs(alpha), norm, s2) : 0.0;
+    if (me == scribe && tid == 0) ar.tau[mt.off + k] = c;
+    // w = c p - c^2 (p v) / 2 v, and the next row
+    double pv = 0.0;
     if (g > 1) {
-      arrived += g;
-      if (!group_barrier(mt.bar, arrived, ok_s, wait_ns)) goto fail;
+      const unsigned long long t0 = global_ns();
+      constexpr int BATCH = 3;
+      for (int j0 = k + 1 + tid; j0 < n; j0 += BATCH * TRI_THREADS) {
+        double p[BATCH], y[BATCH];
+        bool all;
+        for (int probe = 0;; ++probe) {
+          all = true;
+#pragma unroll
+          for (int q = 0; q < BATCH; ++q) {
+            const int j = j0 + q * TRI_THREADS;
+            if (j < n) {
+              const bool a1 = published(pub + j, step, p[q]), a2 = published(pub + n + j, step, y[q]);
+              all = all && a1 && a2;
+            }
+          }
+          if (all) break;
+          if (wait_ns == 0 || ((probe & 63) == 63 && global_ns() - t0 >= wait_ns)) break;
+        }
+        if (!all) {
+          *ok_s = 0;
+          break;
+        }
+#pragma unroll
+        for (int q = 0; q < BATCH; ++q) {
+          const int j = j0 + q * TRI_THREADS;
+          if (j < n) {
+            pl[j] = p[q];
+            x[j] = y[q];
+            pv = fma(p[q], v[j], pv);
+          }
+        }
+      }
     } else {
       __syncthreads();
+      const double* a = row(k + 1);
+      for (int j = k + 1 + tid; j < n; j += TRI_THREADS) {
+        x[j] = a[j];
+        pv = fma(pl[j], v[j], pv);
+      }
     }
-    // w = tau p - tau^2 (p v) / 2 v, and the next row
-    double pv = 0.0;
-    for (int j = k + 1 + tid; j < n; j += TRI_THREADS) {
-      const double p = __ldcg(pub + j);
-      x[j] = __ldcg(pub + n + j);
-      wo[j] = p;
-      pv = fma(p, v[j], pv);
-    }
-    const double p1 = __ldcg(pub + k + 1), v1 = v[k + 1];
-    pv = 0.5 * tau * tau * block_sum(pv, red + TRI_WARPS);
-    const double w1 = fma(-pv, v1, tau * p1);
+    if (!kSmem) __threadfence();
+    pv = 0.5 * c * c * block_sum(pv, red + TRI_WARPS);
+    if (!*(volatile int*)ok_s) goto fail;
+    const double w1 = fma(-pv, v1, c * pl[k + 1]);
     s = 0.0;
     for (int j = k + 1 + tid; j < n; j += TRI_THREADS) {
-      const double vj = v[j], w = fma(-pv, vj, tau * wo[j]);
+      const double vj = v[j], w = fma(-pv, vj, c * pl[j]);
       wo[j] = w;
-      vo[j] = vj;
       const double y = fma(-w1, vj, fma(-v1, w, x[j]));
       x[j] = y;
+      if (j == k + 2) first[(k + 1) & 1] = y;
       if (j > k + 2) s = fma(y, y, s);  // for the next reflector
     }
-    __syncthreads();
+    // x is the next v; the barrier of the next sum makes it visible
+    double* const free_row = vo;
+    vo = v;
+    v = x;
+    x = free_row;
   }
-  if (me == 0 && tid == 0) {
-    ar.d[mt.off + n - 1] = x[n - 1];
+  __syncthreads();
+  if (me == scribe && tid == 0) {
+    ar.d[mt.off + n - 1] = v[n - 1];
     ar.e[mt.off + n - 1] = 0.0;
     ar.tau[mt.off + n - 1] = 0.0;
   }
@@ -471,7 +543,7 @@ __global__ void __launch_bounds__(TRI_THREADS, 1) tridiag_kernel(const DcMatrix*
                                                                  DcArrays ar, int* __restrict__ err,
                                                                  unsigned long long wait_ns) {
   extern __shared__ double sm[];
-  __shared__ double red[2 * TRI_WARPS];
+  __shared__ double red[2 * TRI_WARPS + 2];
   __shared__ int ok_s;
   // CTA b belongs to the last matrix whose first CTA is at most b
   int lo = m0, hi = m0 + count - 1;
@@ -482,9 +554,9 @@ __global__ void __launch_bounds__(TRI_THREADS, 1) tridiag_kernel(const DcMatrix*
   }
   const DcMatrix mt = mats[lo];
   const int me = (int)blockIdx.x - mt.cta0;
-  // four vectors beyond shared memory (n > 7040)
-  if (4 * (size_t)mt.n * sizeof(double) > kTriSmem)
-    tridiag_one<false>(mt, ar, lo, me, ar.wide + (size_t)blockIdx.x * 4 * mt.n, red, &ok_s, err, wait_ns);
+  // five vectors beyond shared memory (n > 5632)
+  if (5 * (size_t)mt.n * sizeof(double) > kTriSmem)
+    tridiag_one<false>(mt, ar, lo, me, ar.wide + (size_t)blockIdx.x * 5 * mt.n, red, &ok_s, err, wait_ns);
   else if (mt.rows_in_smem) tridiag_one<true>(mt, ar, lo, me, sm, red, &ok_s, err, wait_ns);
   else tridiag_one<false>(mt, ar, lo, me, sm, red, &ok_s, err, wait_ns);
 }
@@ -921,13 +993,13 @@ DcPlan dc_plan(const std::vector<int>& sizes) {
 }
 
 static size_t tri_bytes(int n, int g, bool rows) {
-  return (4 * (size_t)n + (rows ? (size_t)((n + g - 1) / g) * n : 0)) * sizeof(double);
+  return (5 * (size_t)n + (rows ? (size_t)((n + g - 1) / g) * n : 0)) * sizeof(double);
 }
 bool tridiag_rows_fit(int n, int g) { return tri_bytes(n, g, true) <= kTriSmem; }
 
 size_t tridiag_wide(int n, int total, int ctas) {
   size_t w = 0;
-  if (tri_bytes(n, 1, false) > kTriSmem) w = (size_t)ctas * 4 * n;
+  if (tri_bytes(n, 1, false) > kTriSmem) w = (size_t)ctas * 5 * n;
   if (n > kPrepMax) w = std::max(w, 4 * (size_t)total);
   return w;
 }

@@ -32,7 +32,8 @@ struct DcMatrix {
   double* w;        // eigenvalues, descending
   double* V;        // eigenvectors as rows; holds the rank-one update's until the end
   double* B[2];     // eigenvectors of T (rows) before and after a level of merges
-  double* xch;      // 4 n: what the CTAs of a group exchange
+  double* xch;      // 8 n: what the CTAs of a group exchange, zero at launch
+  unsigned* peak;   // largest entry of each CTA's rows
   unsigned* bar;    // arrivals of the group barrier, zero at launch
   int n, off;
   int g, cta0;      // CTAs of the group, the first one
@@ -54,7 +55,7 @@ struct DcRot {
 
 // flat arrays over all matrices (length: the sum of the sizes)
 struct DcArrays {
-  double *d, *e, *tau;      // T, and the reflectors' factors
+  double *d, *e, *tau;      // T, and the reflectors' factors c
   double* scale;            // per matrix
   double* val;              // eigenvalues of the current nodes, ascending
   double *dl, *zl;          // poles and z of a merge: kept ones, then deflated values
