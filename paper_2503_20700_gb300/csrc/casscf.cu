@@ -219,6 +219,27 @@ __global__ void k_poly(double* __restrict__ T, int n, double c0, double c1, doub
     T[e] = fma(c3, X3[e], fma(c2, X2[e], fma(c1, X[e], e / n == e % n ? c0 : 0.0)));
 }
 
+// out[p][k nc + i] = L^k[p][c0 + i], the columns of every vector side by side
+__global__ void k_gather_cols(const double* __restrict__ L, int rank, int nb, int c0, int nc,
+                              double* __restrict__ out) {
+  const size_t K = (size_t)rank * nc, tot = K * nb;
+  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (size_t)gridDim.x * blockDim.x) {
+    const size_t p = e / K, c = e - p * K;
+    const int k = (int)(c / nc), i = (int)(c - (size_t)k * nc);
+    out[e] = __ldg(L + ((size_t)k * nb + p) * nb + c0 + i);
+  }
+}
+
+// out[k nc + i][q] = L^k[c0 + i][q], the rows of every vector one below the other
+__global__ void k_gather_rows(const double* __restrict__ L, int rank, int nb, int c0, int nc,
+                              double* __restrict__ out) {
+  const size_t run = (size_t)nc * nb, tot = run * rank;
+  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (size_t)gridDim.x * blockDim.x) {
+    const size_t k = e / run;
+    out[e] = __ldg(L + k * nb * nb + (size_t)c0 * nb + (e - k * run));
+  }
+}
+
 // J = sum_k v_k L^k and, with w, JA = sum_k w_k L^k: one read of the vectors,
 // bound by HBM (as a 1 x rank by rank x nb^2 product they were split into digits
 // and multiplied on tiles of 128 rows).  A warp has 32 elements and an eighth of
@@ -362,9 +383,14 @@ struct Casscf::Dev {
     mem.push_back(p);
     return p;
   }
-  double* upload(const double* h, size_t n) {
+  // written whole before it is read
+  double* raw(size_t n) {
     double* p = (double*)be->alloc(std::max<size_t>(n, 1) * sizeof(double));
     mem.push_back(p);
+    return p;
+  }
+  double* upload(const double* h, size_t n) {
+    double* p = raw(n);
     be->copy_h2d(p, h, n * sizeof(double));
     return p;
   }
@@ -374,6 +400,27 @@ static void gemm1(Backend* be, double* C, int m, int n, int ldc, const double* A
                   const double* B, int ldb, int tb, int k, double alpha) {
   std::vector<GemmGroup> g{{C, m, n, ldc, 0, 1}};
   std::vector<GemmSeg> s{{A, B, k, lda, ldb, ta, tb, alpha}};
+  be->gemm(g, s, Precision::FP64);
+}
+
+// C (m x n) += A (m x K, row-major) op(B) with K in the tens of thousands (the
+// Cholesky vectors side by side).  Bound by the float64 combination of each
+// segment's digit products on an output tile (some 15000 clocks, as much as 160
+// of K take to multiply), so a segment is as long as leaves every SM two of
+// them; one segment per vector (a K of ncore or ncas) spent four fifths of
+// its time there.  Measured, 600 vectors of 200 x 200 (40 core, 30 active
+// orbitals), the seven products of the active space and the gradient with their
+// splits: 1.83 -> 0.82 ms.
+static void long_gemm(Backend* be, double* C, int m, int n, int ldc, const double* A, const double* B, size_t ldb,
+                      int transB, size_t K) {
+  const size_t tiles = (size_t)((m + 127) / 128) * ((n + 63) / 64);
+  const size_t want = std::max<size_t>(1, 304 / tiles);
+  const size_t step = std::min<size_t>(1024, std::max<size_t>(64, (K / want + 15) / 16 * 16));
+  std::vector<GemmGroup> g{{C, m, n, ldc, 0, 0}};
+  std::vector<GemmSeg> s;
+  for (size_t k = 0; k < K; k += step)
+    s.push_back({A + k, B + (transB ? k : k * ldb), (int)std::min(step, K - k), (int)K, (int)ldb, 0, transB, 1.0});
+  g[0].seg_count = (int)s.size();
   be->gemm(g, s, Precision::FP64);
 }
 
@@ -499,6 +546,7 @@ void Casscf::transform(const double* R, const double* h, const double* L, int ra
 // Pieces shared by the active-space problem and the gradient.
 struct FockParts {
   double *FI, *FA, *La, *v, *w;
+  double* Aa;  // L^k[q][act] as [q][k, act] (with an active density)
 };
 
 static FockParts fock_parts(Backend* be, Casscf::Dev& d, const double* dh, const double* dL, int rank,
@@ -517,30 +565,25 @@ static FockParts fock_parts(Backend* be, Casscf::Dev& d, const double* dh, const
   // Kc = sum_k L^k[:, core] L^k[core, :]
   double* Kc = d.alloc(nn);
   if (ncore > 0) {
-    std::vector<GemmGroup> g{{Kc, nb, nb, nb, 0, rank}};
-    std::vector<GemmSeg> s;
-    for (int k = 0; k < rank; ++k) s.push_back({dL + nn * k, dL + nn * k, ncore, nb, nb, 0, 0, 1.0});
-    be->gemm(g, s, Precision::FP64);
+    const size_t K = (size_t)rank * ncore;
+    double *Ac = d.raw(K * nb), *Bc = d.raw(K * nb);
+    k_gather_cols<<<grid_for(K * nb), 256, 0, ST>>>(dL, rank, nb, 0, ncore, Ac);
+    k_gather_rows<<<grid_for(K * nb), 256, 0, ST>>>(dL, rank, nb, 0, ncore, Bc);
+    long_gemm(be, Kc, nb, nb, nb, Ac, Bc, nb, 0, K);
   }
   f.FI = d.alloc(nn);
   k_axpbypcz<<<grid_for(nn), 256, 0, ST>>>(f.FI, nn, 1.0, dh, 2.0, J, -1.0, Kc);
   f.FA = nullptr;
   if (dgamma) {
     // M^k = L^k[:, act] gamma ; KA = sum_k M^k L^k[act, :]
-    double* M = d.alloc((size_t)rank * nb * ncas);
-    std::vector<GemmGroup> g1;
-    std::vector<GemmSeg> s1;
-    for (int k = 0; k < rank; ++k) {
-      g1.push_back({M + (size_t)k * nb * ncas, nb, ncas, ncas, (int)s1.size(), 1});
-      s1.push_back({dL + nn * k + ncore, dgamma, ncas, nb, ncas, 0, 0, 1.0});
-    }
-    be->gemm(g1, s1, Precision::FP64);
+    const size_t K = (size_t)rank * ncas;
+    f.Aa = d.raw(K * nb);
+    double *Ba = d.raw(K * nb), *M = d.alloc(K * nb);
+    k_gather_cols<<<grid_for(K * nb), 256, 0, ST>>>(dL, rank, nb, ncore, ncas, f.Aa);
+    k_gather_rows<<<grid_for(K * nb), 256, 0, ST>>>(dL, rank, nb, ncore, ncas, Ba);
+    gemm1(be, M, nb * rank, ncas, ncas, f.Aa, ncas, 0, dgamma, ncas, 0, ncas, 1.0);
     double* KA = d.alloc(nn);
-    std::vector<GemmGroup> g2{{KA, nb, nb, nb, 0, rank}};
-    std::vector<GemmSeg> s2;
-    for (int k = 0; k < rank; ++k)
-      s2.push_back({M + (size_t)k * nb * ncas, dL + nn * k + (size_t)ncore * nb, ncas, ncas, nb, 0, 0, 1.0});
-    be->gemm(g2, s2, Precision::FP64);
+    long_gemm(be, KA, nb, nb, nb, M, Ba, nb, 0, K);
     f.FA = d.alloc(nn);
     k_axpbypcz<<<grid_for(nn), 256, 0, ST>>>(f.FA, nn, 1.0, JA, -0.5, KA, 0.0, nullptr);
   }
@@ -640,15 +683,18 @@ void Casscf::fock_dev(const double* dh, const double* dL, int rank, int nb, int 
   // d[t,u,v,w] = Gamma[t,v,w,u];  W (rank x a2) = La (rank x a2) d^T (a2 x a2)
   double* dd = d.alloc((size_t)a2 * a2);
   k_permute_rdm2<<<grid_for((size_t)a2 * a2), 256, 0, ST>>>(dG, ncas, dd);
+  // as W[t][k, u], which F2 contracts
   double* W = d.alloc((size_t)rank * a2);
-  gemm1(be_, W, rank, a2, a2, f.La, a2, 0, dd, a2, 1, a2, 1.0);
+  std::vector<GemmGroup> g;
+  std::vector<GemmSeg> s;
+  for (int t = 0; t < ncas; ++t) {
+    g.push_back({W + (size_t)t * rank * ncas, rank, ncas, ncas, t, 1});
+    s.push_back({f.La, dd + (size_t)t * ncas * a2, a2, a2, a2, 0, 1, 1.0});
+  }
+  be_->gemm(g, s, Precision::FP64);
   // F2[t, q] = sum_k sum_u W^k[t,u] L^k[q, c+u]
   double* F2 = d.alloc((size_t)ncas * nb);
-  std::vector<GemmGroup> g{{F2, ncas, nb, nb, 0, rank}};
-  std::vector<GemmSeg> s;
-  for (int k = 0; k < rank; ++k)
-    s.push_back({W + (size_t)k * a2, dL + nn * k + ncore, ncas, ncas, nb, 0, 1, 1.0});
-  be_->gemm(g, s, Precision::FP64);
+  long_gemm(be_, F2, ncas, nb, nb, W, f.Aa, (size_t)rank * ncas, 1, (size_t)rank * ncas);
   k_assemble_fock<<<grid_for(nn), 256, 0, ST>>>(f.FI, f.FA, dg, F2, nb, ncore, ncas, F);
   if (fdiag) k_fock_diag<<<grid_for(nb), 256, 0, ST>>>(f.FI, f.FA, nb, fdiag);
   be_->sync();
