@@ -6,14 +6,15 @@
 // (this file's predecessor) spent 13 n^3 FMAs and 10 n group barriers on a
 // matrix.  Here a matrix costs n^3 FMAs and n barriers of tridiagonalisation,
 // n^3 FMAs of reflectors, and GEMMs on the tensor cores.  Measured, the 13
-// density matrices of 9..601 of a decimation: 184 ms before; now 11.2 ms, of
-// which the tridiagonalisation 6.1, the reflectors 2.8, the merges 1.9 with
+// density matrices of 9..601 of a decimation: 184 ms before; now 10.6 ms, of
+// which the tridiagonalisation 5.5, the reflectors 2.8, the merges 1.9 with
 // their products, the small matrices and leaves 0.4; the largest error of the
 // eigenvectors 3e-12 -> 4e-13.
 #include <algorithm>
 #include <cmath>
 #include <stdexcept>
 #include <string>
+#include <type_traits>
 
 #include "eigh.cuh"
 #include "kattr.hpp"
@@ -270,12 +271,15 @@ __global__ void __launch_bounds__(SMALL_THREADS) eigh_small_kernel(const EighTas
 // of that before it publishes once more.
 // Bound by the float64 pipe (a warp-wide operation holds a quarter of an SM
 // for 64 clocks): three FMAs per entry, n^3 in all, and what every CTA repeats,
-// so a CTA is four warps, one per quarter, each with four rows in flight that
-// share the reads of v and w and one tree of sums.  The rest of a step is a
+// so a CTA is four warps, one per quarter, each with up to four rows in flight
+// that share the reads of v and w and one tree of sums (always four left the
+// quarters unevenly loaded: 11600 clocks of the pass of the largest of 13
+// matrices, 4800 of them FMAs of an even load).  The rest of a step is a
 // chain of latencies: v is not scaled (no division before the pass, the
 // division for c runs while the others' parts travel), the norm comes from an
 // inverse square root.  Measured, the tridiagonalisation of 13 matrices of 9..601:
-// 7.7 ms with sixteen warps and a barrier, 6.7 with four, 6.1 now.
+// 7.7 ms with sixteen warps and a barrier, 6.7 with four, 6.1 without it, 5.5 with
+// the rows dealt evenly.
 constexpr int TRI_WARPS = 4, TRI_THREADS = 32 * TRI_WARPS, TRI_ROWS = 4;
 constexpr size_t kTriSmem = 220 * 1024;
 
@@ -406,57 +410,85 @@ __device__ void tridiag_one(const DcMatrix& mt, const DcArrays& ar, int mat, int
       for (int j = k + 1 + tid; j < n; j += TRI_THREADS) publish(pub + n + j, fma(-wi, vo[j], fma(-vi, wo[j], a[j])), step);
       __syncthreads();
     }
-    for (int lr = live + TRI_ROWS * warp; lr < nloc; lr += TRI_ROWS * TRI_WARPS) {
-      double* a[TRI_ROWS];
-      double vi[TRI_ROWS], wi[TRI_ROWS], acc[TRI_ROWS];
-      bool keep[TRI_ROWS];  // the next row is the scribe's from here on
+    // rows of a warp at a time: as many as deal the rows evenly to the warps
+    const int active = nloc - live, rounds = (active + TRI_ROWS * TRI_WARPS - 1) / (TRI_ROWS * TRI_WARPS);
+    auto update = [&](auto per_warp) {
+      constexpr int R = decltype(per_warp)::value;
+      for (int lr = live + R * warp; lr < nloc; lr += R * TRI_WARPS) {
+        double* a[R];
+        double vi[R], wi[R], acc[R];
+        bool keep[R];  // the next row is the scribe's from here on
 #pragma unroll
-      for (int r = 0; r < TRI_ROWS; ++r) {
-        const int q = min(lr + r, nloc - 1);  // a row twice: the same values, stored once
-        a[r] = row(q);
-        keep[r] = g == 1 || q * g + me != k + 1;
-        vi[r] = vo[q * g + me];
-        wi[r] = wo[q * g + me];
-        acc[r] = 0.0;
-      }
-      const int rows_here = min(TRI_ROWS, nloc - lr);
-      if (rows_here == TRI_ROWS) {
-#pragma unroll 2
-        for (int j = k + 1 + lane; j < n; j += 32) {
-          const double vj = vo[j], wj = wo[j], nj = v[j];
-#pragma unroll
-          for (int r = 0; r < TRI_ROWS; ++r) {
-            const double y = fma(-wi[r], vj, fma(-vi[r], wj, a[r][j]));
-            if (kSmem || keep[r]) a[r][j] = y;
-            acc[r] = fma(y, nj, acc[r]);
-          }
+        for (int r = 0; r < R; ++r) {
+          const int q = min(lr + r, nloc - 1);
+          a[r] = row(q);
+          keep[r] = g == 1 || q * g + me != k + 1;
+          vi[r] = vo[q * g + me];
+          wi[r] = wo[q * g + me];
+          acc[r] = 0.0;
         }
-      } else {
-        for (int j = k + 1 + lane; j < n; j += 32) {
-          const double vj = vo[j], wj = wo[j], nj = v[j];
+        const int rows_here = min(R, nloc - lr);
+        if (rows_here == R) {
+#pragma unroll 2
+          for (int j = k + 1 + lane; j < n; j += 32) {
+            const double vj = vo[j], wj = wo[j], nj = v[j];
 #pragma unroll
-          for (int r = 0; r < TRI_ROWS - 1; ++r)
-            if (r < rows_here) {
+            for (int r = 0; r < R; ++r) {
               const double y = fma(-wi[r], vj, fma(-vi[r], wj, a[r][j]));
               if (kSmem || keep[r]) a[r][j] = y;
               acc[r] = fma(y, nj, acc[r]);
             }
+          }
+        } else {
+          for (int j = k + 1 + lane; j < n; j += 32) {
+            const double vj = vo[j], wj = wo[j], nj = v[j];
+#pragma unroll
+            for (int r = 0; r < R - 1; ++r)
+              if (r < rows_here) {
+                const double y = fma(-wi[r], vj, fma(-vi[r], wj, a[r][j]));
+                if (kSmem || keep[r]) a[r][j] = y;
+                acc[r] = fma(y, nj, acc[r]);
+              }
+          }
+        }
+        // the sums in one tree: the first lane of each quarter (half, for two
+        // rows; warp, for one) ends with a row's
+        double t = acc[0];
+        int r = 0, lanes = 32;
+        if constexpr (R > 2) {
+          const bool up = lane & 16, odd = lane & 8;
+          const double a3 = R > 3 ? acc[R - 1] : 0.0;
+          double t0 = up ? acc[2] : acc[0], t1 = up ? a3 : acc[1];
+          t0 += __shfl_xor_sync(0xffffffffu, up ? acc[0] : acc[2], 16);
+          t1 += __shfl_xor_sync(0xffffffffu, up ? acc[1] : a3, 16);
+          t = odd ? t1 : t0;
+          t += __shfl_xor_sync(0xffffffffu, odd ? t0 : t1, 8);
+          r = lane >> 3;
+          lanes = 8;
+        } else if constexpr (R == 2) {
+          const bool up = lane & 16;
+          t = up ? acc[1] : acc[0];
+          t += __shfl_xor_sync(0xffffffffu, up ? acc[0] : acc[1], 16);
+          t += __shfl_xor_sync(0xffffffffu, t, 8);
+          r = lane >> 4;
+          lanes = 16;
+        } else {
+          t += __shfl_xor_sync(0xffffffffu, t, 16);
+          t += __shfl_xor_sync(0xffffffffu, t, 8);
+        }
+#pragma unroll
+        for (int d = 4; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+        if ((lane & (lanes - 1)) == 0 && r < rows_here) {
+          if (g > 1) publish(pub + (lr + r) * g + me, t, step);
+          else pl[lr + r] = t;
         }
       }
-      // four sums in one tree: lanes 8 r ... end with the sum of row r
-      const bool up = lane & 16, odd = lane & 8;
-      double t0 = up ? acc[2] : acc[0], t1 = up ? acc[3] : acc[1];
-      t0 += __shfl_xor_sync(0xffffffffu, up ? acc[0] : acc[2], 16);
-      t1 += __shfl_xor_sync(0xffffffffu, up ? acc[1] : acc[3], 16);
-      double t = odd ? t1 : t0;
-      t += __shfl_xor_sync(0xffffffffu, odd ? t0 : t1, 8);
-#pragma unroll
-      for (int d = 4; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
-      const int r = lane >> 3;
-      if ((lane & 7) == 0 && r < rows_here) {
-        if (g > 1) publish(pub + (lr + r) * g + me, t, step);
-        else pl[lr + r] = t;
-      }
+    };
+    switch (rounds > 0 ? (active + TRI_WARPS * rounds - 1) / (TRI_WARPS * rounds) : 0) {
+      case 1: update(std::integral_constant<int, 1>()); break;
+      case 2: update(std::integral_constant<int, 2>()); break;
+      case 3: update(std::integral_constant<int, 3>()); break;
+      case 4: update(std::integral_constant<int, 4>()); break;
     }
     // row k of the matrix is done: it keeps the reflector
     if (me == scribe)
