@@ -55,6 +55,7 @@
 
 #include "hpsi_tc.cuh"
 #include "kattr.hpp"
+#include "tf32_bits.cuh"
 
 namespace dmrg {
 
@@ -97,11 +98,7 @@ __device__ __forceinline__ uint64_t desc(uint32_t saddr, uint32_t sbo) {
 __device__ __forceinline__ uint32_t idesc_tf32(int M, int N) {
   return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-__device__ __forceinline__ uint32_t tf32(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return r;
-}
+__device__ __forceinline__ uint32_t tf32(float x) { return tf32_round(x); }
 __device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
@@ -867,7 +864,7 @@ __global__ void __launch_bounds__(256) hpsi_tc_reduce(const HpsiBlock* __restric
 #pragma unroll 16
     for (int p = 0; p < rd.nparts; ++p) {
       const float2 v = __ldg(part + (size_t)p * TM * TNMAX);
-      acc += (double)v.x + (double)v.y;
+      acc += widen(v.x) + widen(v.y);
     }
     turn[warp][lane] = acc;
   }
@@ -884,7 +881,9 @@ __global__ void __launch_bounds__(256) hpsi_tc_reduce(const HpsiBlock* __restric
 // Measured: 1066 us of a contraction of some 60 operands of 280..600 with one
 // CTA per operand (the whole call 3.17 -> 2.20 ms, 0.1 ms of it the reduction);
 // the operands of a D = 256 sweep 63 -> 40 us per launch, of a D = 512 bond
-// 51 -> 29 us.
+// 51 -> 29 us.  Four float64 conversions and differences per element then kept
+// the float64 pipe busy for 88 % of the time; by integers (tf32_bits.cuh) 150 ->
+// 65 us for the 60 operands, 40 -> 25 and 29 -> 18 us.
 __global__ void __launch_bounds__(256) split_kernel(const SplitJob* __restrict__ jobs, float* __restrict__ pool) {
   const SplitJob jb = jobs[blockIdx.x];
   const int G = (jb.rows + 7) >> 3;
@@ -907,9 +906,10 @@ __global__ void __launch_bounds__(256) split_kernel(const SplitJob* __restrict__
     float* const u = base + (size_t)pr * 2 * kTcUnitFloats;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const float h = __uint_as_float(tf32((float)v[i]));
-      u[32 * i] = h;
-      u[kTcUnitFloats + 32 * i] = __uint_as_float(tf32((float)(v[i] - (double)h)));
+      float hi, lo;
+      split_tf32(v[i], hi, lo);
+      u[32 * i] = hi;
+      u[kTcUnitFloats + 32 * i] = lo;
     }
   }
 }
