@@ -3,6 +3,7 @@
 #include <string>
 
 #include "gemm_split.cuh"
+#include "tf32_bits.cuh"
 
 namespace dmrg {
 
@@ -10,18 +11,12 @@ namespace {
 
 constexpr int SM = 64, SN = 64, SK = 16;
 
-__device__ __forceinline__ uint32_t to_tf32(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return r;
-}
-
 // split a float64 into two TF32 words: hi = tf32(x), lo = tf32(x - hi)
 __device__ __forceinline__ void split(double x, uint32_t& hi, uint32_t& lo) {
-  float xf = (float)x;
-  hi = to_tf32(xf);
-  double r = x - (double)__uint_as_float(hi);
-  lo = to_tf32((float)r);
+  float h, l;
+  split_tf32(x, h, l);
+  hi = __float_as_uint(h);
+  lo = __float_as_uint(l);
 }
 
 __device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
@@ -110,7 +105,7 @@ __global__ void __launch_bounds__(256) gemm_tf32x3_mma(const GemmGroup* __restri
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc64[nt][q] += (double)acc[nt][q];
+      for (int q = 0; q < 4; ++q) acc64[nt][q] += widen(acc[nt][q]);
   }
   // C fragment: c0 (gid, 2tig), c1 (gid, 2tig+1), c2 (gid+8, 2tig), c3 (gid+8, 2tig+1)
 #pragma unroll

@@ -6,6 +6,7 @@
 #include "hpsi_fused.cuh"
 #include "hpsi_noalloc.hpp"
 #include "kattr.hpp"
+#include "tf32_bits.cuh"
 
 namespace dmrg {
 
@@ -15,14 +16,14 @@ constexpr int T = 64;   // tile edge of sigma and of the psi column chunk
 constexpr int KS = 16;  // k-step of the staged operand tiles
 
 // ---------------------------------------------------------------- helpers
-__device__ __forceinline__ uint32_t tf32(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return r;
-}
+__device__ __forceinline__ uint32_t tf32(float x) { return tf32_round(x); }
+// by integers: the float64 pipe converts two numbers a clock and SM, which bound
+// this kernel (a call with sectors of some tens, 1258 -> 831 us)
 __device__ __forceinline__ void split64(double x, uint32_t& hi, uint32_t& lo) {
-  hi = tf32((float)x);
-  lo = tf32((float)(x - (double)__uint_as_float(hi)));
+  float h, l;
+  split_tf32(x, h, l);
+  hi = __float_as_uint(h);
+  lo = __float_as_uint(l);
 }
 __device__ __forceinline__ void mma(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
   asm volatile(
@@ -213,7 +214,7 @@ __global__ void __launch_bounds__(256) hpsi_tf32x3_kernel(const HpsiBlock* __res
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) s64[nt][q] += (double)sacc[nt][q];
+      for (int q = 0; q < 4; ++q) s64[nt][q] += widen(sacc[nt][q]);
   }
   // write: partial tile or direct add
 #pragma unroll

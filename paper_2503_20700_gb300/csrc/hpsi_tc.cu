@@ -843,7 +843,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 // through shared memory.  Measured, per launch: the products of a D = 256 sweep
 // 227 -> 116 us with 32 x 32 CTAs and four chunks in flight -> 54 us, of a
 // D = 512 bond 392 -> 101 -> 59 us (a CTA of 128 rows that walked 32 columns
-// two at a time and wrote sigma by columns at first).
+// two at a time and wrote sigma by columns at first).  The float64 pipe was then
+// busy for 83 % of the time; with the sum of a pair by integers (tf32_bits.cuh)
+// 54 -> 34 us and 66 -> 41 us.
 constexpr int RED_R = 32, RED_C = 8;
 __global__ void __launch_bounds__(256) hpsi_tc_reduce(const HpsiBlock* __restrict__ blocks,
                                                       const HpsiReduce* __restrict__ reds,
@@ -864,7 +866,7 @@ __global__ void __launch_bounds__(256) hpsi_tc_reduce(const HpsiBlock* __restric
 #pragma unroll 16
     for (int p = 0; p < rd.nparts; ++p) {
       const float2 v = __ldg(part + (size_t)p * TM * TNMAX);
-      acc += widen(v.x) + widen(v.y);
+      acc += pair_sum(v.x, v.y);
     }
     turn[warp][lane] = acc;
   }
@@ -883,7 +885,7 @@ __global__ void __launch_bounds__(256) hpsi_tc_reduce(const HpsiBlock* __restric
 // the operands of a D = 256 sweep 63 -> 40 us per launch, of a D = 512 bond
 // 51 -> 29 us.  Four float64 conversions and differences per element then kept
 // the float64 pipe busy for 88 % of the time; by integers (tf32_bits.cuh) 150 ->
-// 65 us for the 60 operands, 40 -> 25 and 29 -> 18 us.
+// 65 us for the 60 operands, 40 -> 15 and 29 -> 12 us.
 __global__ void __launch_bounds__(256) split_kernel(const SplitJob* __restrict__ jobs, float* __restrict__ pool) {
   const SplitJob jb = jobs[blockIdx.x];
   const int G = (jb.rows + 7) >> 3;

@@ -78,4 +78,34 @@ __host__ __device__ __forceinline__ void split_tf32(double v, float& hi, float& 
   lo = bits_float(tf32_round(sign ? -l : l));
 }
 
+__host__ __device__ __forceinline__ int leading_zeros(uint64_t x) {
+#ifdef __CUDA_ARCH__
+  return __clzll((long long)x);
+#else
+  return x ? __builtin_clzll(x) : 64;
+#endif
+}
+
+// (double)x + (double)y of a pair whose second part is the smaller
+__host__ __device__ __forceinline__ double pair_sum(float x, float y) {
+  const uint32_t ux = float_bits(x), uy = float_bits(y), ex = (ux >> 23) & 0xFFu, ey = (uy >> 23) & 0xFFu;
+  if ((uy << 1) == 0u) return widen(x);
+  // both ordinary, the second at least one binary place down
+  if (ex - 1u >= 254u || ey - 1u >= 254u || ey >= ex) return widen(x) + widen(y);
+  const uint32_t d = ex - ey;
+  const uint64_t mx = (uint64_t)((ux & 0x7FFFFFu) | 0x800000u) << 39;  // leading one at bit 62
+  uint64_t my = (uint64_t)((uy & 0x7FFFFFu) | 0x800000u) << 39;
+  // what is shifted out leaves its trace in the last bit
+  my = d < 63u ? (my >> d) | (uint64_t)((my & ((1ull << d) - 1)) != 0) : 1u;
+  const uint64_t s = ((ux ^ uy) >> 31) ? mx - my : mx + my;
+  const int n = leading_zeros(s);  // 0 ... 2
+  const uint64_t top = s << n, q = top >> 11;
+  const uint32_t rest = (uint32_t)top & 0x7FFu;
+  const uint64_t up = rest > 0x400u || (rest == 0x400u && (q & 1u));
+  const uint64_t b = (((uint64_t)(ex + 896u - (uint32_t)n) << 52) + q + up) | (uint64_t)(ux >> 31) << 63;
+  double r;
+  memcpy(&r, &b, 8);
+  return r;
+}
+
 }  // namespace dmrg

@@ -47,6 +47,21 @@ int main() {
       check(from(e << 52 | m));
   for (float x : {0.0f, -0.0f, 1.17549435e-38f, 3.4028234e38f, -1e-40f, INFINITY, -INFINITY})
     if (of(widen(x)) != of((double)x)) ++bad;
+  for (long i = 0; i < 8000000; ++i) {
+    const uint64_t b = r();
+    const float x = bits_float((uint32_t)b);
+    uint32_t u = (uint32_t)(b >> 32);
+    // most of them near below x
+    if (i % 4) {
+      const uint32_t ex = (float_bits(x) >> 23) & 0xFFu, dn = (uint32_t)(r() % 70);
+      u = (u & 0x807FFFFFu) | (ex > dn ? ex - dn : 0u) << 23;
+      if (i % 4 == 1) u &= ~0u << (r() % 24);
+    }
+    const float y = bits_float(u);
+    if (std::isnan(x) || std::isnan(y) || std::isinf(x) || std::isinf(y)) continue;
+    if (of(pair_sum(x, y)) != of((double)x + (double)y) && ++bad < 20)
+      std::printf("%a + %a: %a, not %a\n", x, y, pair_sum(x, y), (double)x + (double)y);
+  }
   if (bad) return 1;
   std::printf("conversions agree\n");
   return 0;
