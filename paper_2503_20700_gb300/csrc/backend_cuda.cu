@@ -399,6 +399,7 @@ class CudaBackend : public Backend {
     if (dtask) cudaFreeAsync(dtask, st);
     if (part) cudaFreeAsync(part, st);
     if (dav_dev) cudaFreeAsync(dav_dev, st);
+    if (dig_ws) cudaFreeAsync(dig_ws, st);
     if (dflag) cudaFreeAsync(dflag, st);
     cudaStreamSynchronize(st);
     PinnedPool::get().put(htask, task_cap);
@@ -737,6 +738,10 @@ class CudaBackend : public Backend {
     }
     run_digits(pl.plan);
   }
+  static constexpr size_t kDigKept = size_t(64) << 20;
+  char* dig_ws = nullptr;
+  size_t dig_ws_cap = 0;
+  std::vector<char> dig_zero;
   void run_digits(DigPlan& p) {
     if (p.tasks.empty()) return;
     // longest tasks first, dealt round-robin over the persistent CTAs
@@ -753,19 +758,40 @@ class CudaBackend : public Backend {
     auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
     const size_t ox = al(p.pool_bytes()), ok = ox + al(p.nexp * sizeof(int));
     const size_t osp = ok + al(p.nkmax * sizeof(uint2)), osc = osp + al(p.ops.size() * sizeof(int));
+    // Work space of a launch sequence: small ones share a block that the backend
+    // keeps (stream order separates them), larger ones come and go.  The part
+    // that starts at zero is uploaded with the lists while it is small.
     char* ws = nullptr;
-    const size_t bytes = osc + (size_t)p.scratch * sizeof(double);
-    if (cudaMallocAsync((void**)&ws, bytes, st) != cudaSuccess) {
-      cudaGetLastError();
-      throw std::runtime_error("out of device memory (" + std::to_string(bytes) + " bytes)");
+    const size_t bytes = osc + (size_t)p.scratch * sizeof(double), nzero = osc - ok;
+    const bool keep = bytes <= kDigKept;
+    if (keep && bytes <= dig_ws_cap) {
+      ws = dig_ws;
+    } else {
+      const size_t want = keep ? std::min(kDigKept, std::max(2 * bytes, size_t(1) << 20)) : bytes;
+      if (keep && dig_ws) {
+        CK(cudaFreeAsync(dig_ws, st));
+        dig_ws = nullptr;
+        dig_ws_cap = 0;
+      }
+      if (cudaMallocAsync((void**)&ws, want, st) != cudaSuccess) {
+        cudaGetLastError();
+        throw std::runtime_error("out of device memory (" + std::to_string(want) + " bytes)");
+      }
+      if (keep) {
+        dig_ws = ws;
+        dig_ws_cap = want;
+      }
     }
-    CK(cudaMemsetAsync(ws + ok, 0, osc - ok, st));
+    const bool inline_zero = nzero <= size_t(32) << 10;
+    if (inline_zero) dig_zero.resize(std::max(dig_zero.size(), nzero), 0);
+    else CK(cudaMemsetAsync(ws + ok, 0, nzero, st));
     std::vector<size_t> off;
     char* d = upload({{p.ops.data(), p.ops.size() * sizeof(DigOperand)},
                       {p.splits.data(), p.splits.size() * sizeof(DigSplit)},
                       {p.segs.data(), p.segs.size() * sizeof(DigSeg)},
                       {tasks.data(), tasks.size() * sizeof(DigTask)},
-                      {p.reds.data(), p.reds.size() * sizeof(DigReduce)}},
+                      {p.reds.data(), p.reds.size() * sizeof(DigReduce)},
+                      {dig_zero.data(), inline_zero ? nzero : 0}},
                      off);
     DigLaunch L{};
     L.ops = (const DigOperand*)(d + off[0]);
@@ -779,14 +805,14 @@ class CudaBackend : public Backend {
     L.nops = (int)p.ops.size();
     L.pool = (unsigned char*)ws;
     L.exps = (int*)(ws + ox);
-    L.kmax = (uint2*)(ws + ok);
-    L.special = (int*)(ws + osp);
+    L.kmax = (uint2*)(inline_zero ? d + off[5] : ws + ok);
+    L.special = (int*)(inline_zero ? d + off[5] + (osp - ok) : ws + osp);
     L.scratch = (double*)(ws + osc);
     L.err = dig_err;
     L.sms = sms;
     dig_launch(L, st);
     launches += 2 + (L.nreds > 0);
-    CK(cudaFreeAsync(ws, st));
+    if (!keep) CK(cudaFreeAsync(ws, st));
   }
 
   void hpsi(const HpsiBlock* blocks, const HpsiItem* items, const HpsiTask* tasks, int ntasks,
