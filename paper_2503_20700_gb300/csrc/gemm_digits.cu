@@ -459,6 +459,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       double* out = nullptr;
       long long part = -1;
       int W = 0, ldc = 0, nrow = 0, gc = 0, gr0 = 0, sc = 1;
+      bool busy = false;  // the warp has outputs of the block
       for (int k = 0; ok && k < sc; ++k, ++q) {
         ok = __all_sync(0xffffffffu, wait_bar(&bar[B_MF + (q & 1)], (uint32_t)((q >> 1) & 1), abort));
         if (!ok) break;
@@ -472,6 +473,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           gr0 = m.t.r0 + (warp & 3) * 32;
           gc = m.t.c0 + half * NC + lane;
           nrow = gc < m.t.n ? max(0, min(32, m.t.m - gr0)) : 0;
+          busy = gr0 < m.t.m && m.t.c0 + half * NC < m.t.n;
           out = m.t.C + (size_t)gr0 * ldc + gc;
           // a tile summed by one task starts from C, loaded while the first
           // products run
@@ -494,7 +496,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
           for (int c = 0; c < NC; c += 4) {
-            if (half * NC + c >= W) break;
+            if (!busy || half * NC + c >= W) break;
             uint32_t v[kDigSlices][4];
 #pragma unroll
             for (int d = 0; d < kDigSlices; ++d) tmem_ld4(lanes + (uint32_t)(W * d + half * NC + c), v[d]);
@@ -532,15 +534,25 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           arrive(&bar[B_ME + (q & 1)]);
           continue;
         }
+        if (!busy) {
+          // nothing of the block in this warp's rows and columns: the float64
+          // pipe belongs to the others (the 442 launches of a D = 256 sweep, whose
+          // blocks are mostly below 128 x 64: 14.7 -> 11.8 ms)
+          arrive(&bar[B_ME + (q & 1)]);
+          continue;
+        }
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
+          if (c % 16 == 0 && half * NC + c >= W) break;
           turn[lane * TURN_LD + c] = combined(h[c], l[c]);
         }
         __syncwarp();
         const double alpha = m.alpha;
+        const int m_rows = m.t.m;
         const int eb = m.eb[half * NC + lane];
 #pragma unroll
         for (int r = 0; r < 32; ++r) {
+          if (r % 8 == 0 && gr0 + r >= m_rows) break;
           // times 2^e: the value is zero or in [1, 2^84), |e| <= 872
           const int e = eb + m.ea[(warp & 3) * 32 + r];
           const double d = turn[r * TURN_LD + lane];
