@@ -399,10 +399,10 @@ dmrg_status dmrg_profile(dmrg_ctx* ctx, int on);
  * since profiling was turned on.  which = 1: the H_eff psi contraction
  * launches (the kernel and the reduction of its item chunks), 0: all other
  * GEMM launches (renormalisation, complementary operators, density
- * matrices), 2: the blocking placement kernel, 3: the eigensolver of a single
- * small matrix (the Davidson subspace problem), 4: the batched eigensolver
- * (the density-matrix sectors of a decimation, one cooperative launch per
- * batch), 5: the TF32 hi/lo splits of the tcgen05 path's operands. */
+ * matrices), 2: the blocking placement kernel, 3: the eigensolver of batches
+ * of small matrices only (up to 32), 4: the eigensolver of batches with larger
+ * ones (the density-matrix sectors of a decimation; all of its launches), 5:
+ * the TF32 hi/lo splits of the tcgen05 path's operands. */
 dmrg_status dmrg_kernel_stats(dmrg_ctx* ctx, int which, double* ms, double* flops,
                               int64_t* launches);
 
@@ -536,8 +536,9 @@ dmrg_status dmrg_last_contract_ms(double* ms);
  * device scratch of 32 MiB (file-scope __device__ array, one per device) and
  * enqueues the copies and the kernels on `stream` (a cudaStream_t; NULL: the
  * legacy default stream); it returns without synchronising.  A request whose
- * task lists and partial tiles exceed the 32 MiB returns DMRG_EINVAL with the
- * size it needed (use dmrg_hpsi_contract for it).  precision: DMRG_FP64 or
+ * task lists and partial tiles (of a plan of 64 x 64 tiles; the float64 plan
+ * takes no more) exceed the 32 MiB returns DMRG_EINVAL with the size it needed
+ * (use dmrg_hpsi_contract for it).  precision: DMRG_FP64 or
  * DMRG_SPLIT_TF32.  Nothing in the scratch has to start at zero: every
  * partial tile is written in full before the reduction reads it.
  *

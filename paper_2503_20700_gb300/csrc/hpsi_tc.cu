@@ -1,6 +1,6 @@
 // tcgen05 fused H_eff psi contraction (see hpsi_tc.cuh), persistent and
 // warp-specialised, with operand tiles brought in by TMA, in clusters of
-// two or four CTAs (a launch parameter of the schedule).
+// one, two or four CTAs (a launch parameter of the schedule).
 //
 // Per item of a task (a 128 x N, N <= 256, sigma tile) and per super-chunk
 // of up to 256 columns of psi (columns [c, c+256) of P):
