@@ -236,11 +236,12 @@ __global__ void __launch_bounds__(256) hpsi_tf32x3_kernel(const HpsiBlock* __res
 // Bound by the float64 pipe (two FMAs a clock and SM: one warp-wide FMA is 16
 // clocks of it), so what counts is that no FMA is spent on padding or done
 // twice; shared memory and issue slots have room to spare.  A task's tile is
-// mt x nt with nt all of a block's columns (up to 256: stage 1, X = alpha
-// op(A) P, is then computed once, not once per column tile) and mt x nt at
-// most kF64Out; its outputs are dealt to the threads one by one, 128 at a
-// time, and so are those of X, so a 20 x 20 block costs 512 FMAs a k instead
-// of a padded 4096.  The two shared-memory reads per FMA this takes (one
+// mt x nt with nt all of a block's columns (up to 480: stage 1, X = alpha
+// op(A) P, is then computed once, not once per column tile: sectors of 300..350
+// 4.86 -> 3.61 ms against tiles of at most 256 columns) and mt x nt at most
+// kF64Out; its outputs are dealt to the threads one by one, 128 at a time, and
+// so are those of X, so a 20 x 20 block costs 512 FMAs a k instead of a padded
+// 4096.  The two shared-memory reads per FMA this takes (one
 // broadcast, one along the lanes) are a quarter of the FMA's own time.  128
 // threads and 44 KB: five CTAs an SM hide each other's loads.  1024 outputs
 // rather than 2048: the rows of a large block make twice the tasks, whose last
@@ -251,10 +252,10 @@ __global__ void __launch_bounds__(256) hpsi_tf32x3_kernel(const HpsiBlock* __res
 constexpr int kF64Threads = 128;
 constexpr int kF64Slots = 8;                        // outputs per thread
 constexpr int kF64Out = kF64Threads * kF64Slots;    // outputs of a tile
-constexpr int kF64Cols = 256;                       // columns of a tile
+constexpr int kF64Cols = 480;                       // columns of a tile
 constexpr int kF64Rows = 128;                       // rows of a tile
 constexpr int kF64Chunk = 128;                      // columns of psi per X chunk
-constexpr int F64_A = kF64Rows * (KS + 1), F64_P = KS * kF64Chunk, F64_B = kF64Cols * (KS + 1);
+constexpr int F64_A = kF64Rows * (KS + 1), F64_P = KS * kF64Chunk, F64_B = 256 * (KS + 1);  // 480 x 9 beyond 256 columns
 constexpr int F64_STAGE = F64_A + F64_P > F64_B ? F64_A + F64_P : F64_B;
 constexpr int F64_X = kF64Out + kF64Rows;           // rows of odd length
 constexpr size_t kF64Smem = (size_t)(F64_STAGE + F64_X) * sizeof(double);
@@ -269,8 +270,8 @@ __host__ __device__ inline void f64_tile(int m, int n, int& mt, int& nt) {
   const int rt = (m + mt - 1) / mt;
   mt = (m + rt - 1) / rt;
 }
-// e / d and e % d of e < 2048, 1 <= d <= 256: the rounding of 2^20 / d is worth
-// less than 2^-9 of a quotient, a remainder at least 2^-8
+// e / d and e % d of e < 2048, 1 <= d <= 512: the rounding of 2^20 / d is worth
+// less than 2^-9 of a quotient, a remainder at least 2^-9
 __device__ __forceinline__ int div_tile(int e, unsigned inv) { return (int)(((unsigned)e * inv) >> 20); }
 __device__ __forceinline__ unsigned inv_tile(int d) { return (unsigned)(((1 << 20) + d - 1) / d); }
 
@@ -294,6 +295,47 @@ __device__ __forceinline__ void f64_products(int ns, double (&acc)[kF64Slots], c
   }
 }
 
+// Stage 2 of a tile of more than 256 columns: k-steps of eight, so that the
+// buffer is no larger.  A function of its own: inlined, it cost the tiles of up
+// to 256 columns 3 %.
+struct F64Sums {
+  double v[kF64Slots];
+};
+__device__ __noinline__ F64Sums f64_stage2_wide(F64Sums w, const double* B, int ldb, int transB, int nt, int kc,
+                                                int outs, unsigned inv_n, const double* Xs, double* Bs) {
+  constexpr int ks = 8;
+  const int tid = threadIdx.x, ldx = kc | 1;
+  double s[kF64Slots];
+  int off[kF64Slots];
+#pragma unroll
+  for (int i = 0; i < kF64Slots; ++i) {
+    const int e = tid + i * kF64Threads;
+    const int r = e < outs ? div_tile(e, inv_n) : 0, c = e < outs ? e - r * nt : 0;
+    off[i] = r * ldx | (c * (ks + 1)) << 16;
+    s[i] = w.v[i];
+  }
+  for (int k0 = 0; k0 < kc; k0 += ks) {
+    const int kn = min(ks, kc - k0);
+    if (transB) {
+      for (int e = tid; e < nt * kn; e += kF64Threads) {
+        const int k = e / nt, c = e - k * nt;
+        Bs[c * (ks + 1) + k] = __ldg(B + (size_t)(k0 + k) * ldb + c);
+      }
+    } else {
+      for (int e = tid; e < nt * ks; e += kF64Threads) {
+        const int c = e / ks, k = e % ks;
+        if (k < kn) Bs[c * (ks + 1) + k] = __ldg(B + (size_t)c * ldb + k0 + k);
+      }
+    }
+    __syncthreads();
+    f64_products((outs + kF64Threads - 1) / kF64Threads, s, off, Xs + k0, Bs, 1, kn);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < kF64Slots; ++i) w.v[i] = s[i];
+  return w;
+}
+
 __global__ void __launch_bounds__(kF64Threads, 5) hpsi_f64_kernel(const HpsiBlock* __restrict__ blocks,
                                                                   const HpsiItem* __restrict__ items,
                                                                   const HpsiTask* __restrict__ tasks,
@@ -301,7 +343,7 @@ __global__ void __launch_bounds__(kF64Threads, 5) hpsi_f64_kernel(const HpsiBloc
   extern __shared__ double smd[];
   double* const As = smd;          // [row][KS + 1]
   double* const Ps = smd + F64_A;  // [k][kc]
-  double* const Bs = smd;          // [column][KS + 1]; shares the buffer with A and P
+  double* const Bs = smd;          // [column][ks + 1]; shares the buffer with A and P
   double* const Xs = smd + F64_STAGE;  // [row][kc | 1]
   const HpsiTask tk = tasks[blockIdx.x];
   const HpsiBlock bk = blocks[tk.block];
@@ -390,6 +432,16 @@ __global__ void __launch_bounds__(kF64Threads, 5) hpsi_f64_kernel(const HpsiBloc
             }
           }
           __syncthreads();
+          continue;
+        }
+        if (tn > 256) {
+          F64Sums w;
+#pragma unroll
+          for (int i = 0; i < kF64Slots; ++i) w.v[i] = s[i];
+          w = f64_stage2_wide(w, it.B + (it.transB ? (size_t)jc * it.ldb + tk.c0 : (size_t)tk.c0 * it.ldb + jc), it.ldb,
+                              it.transB, nt, kc, outs, inv_n, Xs, Bs);
+#pragma unroll
+          for (int i = 0; i < kF64Slots; ++i) s[i] = w.v[i];
           continue;
         }
         int off[kF64Slots];

@@ -335,10 +335,10 @@ def test_fused_hpsi_many_items_split_into_chunks(pkg):
 
 
 @pytest.mark.parametrize("m,n", [(1, 1), (1, 257), (300, 1), (128, 16), (129, 15), (8, 256), (9, 255), (45, 46),
-                                 (23, 512), (200, 208)])
+                                 (23, 512), (200, 208), (9, 300), (5, 480), (3, 481)])
 def test_fused_hpsi_f64_tile_edges(pkg, m, n):
     """Float64 kernel at the edges of its tiles (1024 outputs, at most 128 rows
-    and 256 columns), of the 128-column chunks of psi and of its k-steps of
+    and 480 columns; k-steps of 8 beyond 256), of the 128-column chunks of psi and of its k-steps of
     16, with identities on either side.  Tolerance: a chain of ka + kb FMAs
     over ka kb products of unit normals, next to the largest result."""
     rng = np.random.default_rng(1000 * m + n)
