@@ -141,6 +141,9 @@ class Backend {
   virtual void axpby(double* y, double a, const double* x, double b, size_t len) = 0;
   // y[t] = x[t] / (d[t] - e) with a guarded denominator (Davidson preconditioner)
   virtual void precondition(double* y, const double* x, const double* d, double e, size_t len) = 0;
+  // Work space of the steps below for up to `rows` rows: taken once per solve,
+  // because a result of one step is still read after the next has begun.
+  virtual void dav_reserve(int rows) = 0;
   // Steps of a Davidson iteration on m rows of V and HV (length and stride len).
   // x = sum_i c[i] V_i (c on the host), r = sum_i c[i] HV_i - e x and, with t,
   // t = r / (d - e) with a guarded denominator (r without d); returns |r|^2.

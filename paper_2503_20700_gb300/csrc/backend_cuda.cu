@@ -903,27 +903,29 @@ class CudaBackend : public Backend {
   double* dav_host = nullptr;
   size_t dav_host_cap = 0;
   int dav_rows = 0;
+  void dav_reserve(int rows) override {
+    if (rows <= dav_rows) return;
+    CK(cudaStreamSynchronize(st));
+    if (dav_dev) CK(cudaFreeAsync(dav_dev, st));
+    PinnedPool::get().put(dav_host, dav_host_cap);
+    dav_dev = dav_host = nullptr;
+    dav_rows = 0;
+    rows = std::max(rows, 32);
+    // per row: partials, a counter, two coefficients; and |t|^2
+    const size_t n = (size_t)rows * (kDavParts + 3) + 1;
+    CK(cudaMallocAsync((void**)&dav_dev, n * sizeof(double), st));
+    CK(cudaMemsetAsync(dav_dev, 0, n * sizeof(double), st));
+    dav_host = (double*)PinnedPool::get().take((size_t)(rows + 2) * sizeof(double), &dav_host_cap);
+    dav_rows = rows;
+  }
   DavWork dav_work(int m) {
-    if (m > dav_rows) {
-      CK(cudaStreamSynchronize(st));
-      if (dav_dev) CK(cudaFreeAsync(dav_dev, st));
-      PinnedPool::get().put(dav_host, dav_host_cap);
-      dav_dev = dav_host = nullptr;
-      dav_rows = 0;
-      const int rows = std::max(m, 32);
-      // per row: partials, a counter, two coefficients; and |t|^2
-      const size_t n = (size_t)rows * (kDavParts + 3) + 1;
-      CK(cudaMallocAsync((void**)&dav_dev, n * sizeof(double), st));
-      CK(cudaMemsetAsync(dav_dev, 0, n * sizeof(double), st));
-      dav_host = (double*)PinnedPool::get().take((size_t)(rows + 2) * sizeof(double), &dav_host_cap);
-      dav_rows = rows;
-    }
+    if (m > dav_rows) throw std::logic_error("internal: Davidson rows beyond the reserved work space");
     return DavWork{dav_dev, (unsigned*)(dav_dev + (size_t)dav_rows * kDavParts), dav_host};
   }
   double* dav_coefs() { return dav_dev + (size_t)dav_rows * (kDavParts + 1); }
   double dav_residual(double* x, double* r, double* t, const double* d, const double* V, const double* HV, int m,
                       size_t len, const double* c, double e) override {
-    const DavWork w = dav_work(m + 1);
+    const DavWork w = dav_work(m);
     if (m > kDavCoefs) {
       CK(cudaMemcpyAsync(dav_coefs(), c, m * sizeof(double), cudaMemcpyHostToDevice, st));
       c = dav_coefs();
@@ -934,7 +936,7 @@ class CudaBackend : public Backend {
     return ((volatile double*)w.host)[0];
   }
   void dav_orthonormalise(double* V, int m, size_t len, double* in) override {
-    const DavWork w = dav_work(m + 1);
+    const DavWork w = dav_work(m);
     double *t = V + (size_t)m * len, *c = dav_coefs(), *norm2 = c + 2 * (size_t)dav_rows;
     for (int pass = 0; pass < 2; ++pass) {
       dav_dots_launch(V, m, len, t, nullptr, w, c, st);
@@ -944,7 +946,7 @@ class CudaBackend : public Backend {
     launches += 5;
   }
   double dav_project(const double* V, int m, size_t len, const double* y, double* hv, double* out) override {
-    const DavWork w = dav_work(m + 1);
+    const DavWork w = dav_work(m);
     dav_dots_launch(V, m, len, y, hv, w, w.host + 2, st);
     ++launches;
     CK(cudaStreamSynchronize(st));

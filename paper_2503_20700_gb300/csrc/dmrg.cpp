@@ -1921,6 +1921,7 @@ double Engine::davidson(HPsiPlan& plan, double* psi, int* iters) {
   double* V = (double*)be_->alloc((size_t)M * len * sizeof(double));
   double* HV = (double*)be_->alloc((size_t)M * len * sizeof(double));
   double* dZ = (double*)be_->alloc((size_t)M * sizeof(double));  // coefficients of a restart
+  be_->dav_reserve(M);
   std::vector<double> A((size_t)M * M, 0.0), w(M), Z((size_t)M * M), tmpv(M);
   // guess: provided psi (if nonzero) else a deterministic pseudo-random vector
   {
