@@ -896,14 +896,15 @@ __global__ void __launch_bounds__(256) dc_norm_kernel(const DcNode* __restrict__
 
 // U (DcMatrix::V, the node's diagonal block): row = row of the children's
 // eigenvectors, column = rank of the new eigenvalue; then the rotations of the
-// deflation, last one first.  CTA: 128 columns of a node.
+// deflation, last one first.  CTA: 128 columns of a node.  The nodes are the
+// grid's x: a batch of small matrices has more of them than y may count (65535).
 constexpr int FILL_COLS = 128;
 __global__ void __launch_bounds__(FILL_COLS) dc_fill_kernel(const DcMatrix* __restrict__ mats,
                                                             const DcNode* __restrict__ nodes, DcArrays ar) {
-  const DcNode nd = nodes[blockIdx.y];
+  const DcNode nd = nodes[blockIdx.x];
   const DcMatrix& mt = mats[nd.mat];
   const int N = nd.n1 + nd.n2, K = ar.count[2 * nd.off];
-  const int c = blockIdx.x * FILL_COLS + threadIdx.x;
+  const int c = blockIdx.y * FILL_COLS + threadIdx.x;
   if (c >= N) return;
   const int j = ar.inv[nd.off + c];
   const double *d = ar.dl + nd.off, *zh = ar.zhat + nd.off;
@@ -922,9 +923,9 @@ __global__ void __launch_bounds__(FILL_COLS) dc_fill_kernel(const DcMatrix* __re
 }
 __global__ void __launch_bounds__(FILL_COLS) dc_rotate_kernel(const DcMatrix* __restrict__ mats,
                                                               const DcNode* __restrict__ nodes, DcArrays ar) {
-  const DcNode nd = nodes[blockIdx.y];
+  const DcNode nd = nodes[blockIdx.x];
   const DcMatrix& mt = mats[nd.mat];
-  const int c = blockIdx.x * FILL_COLS + threadIdx.x, nrot = ar.count[2 * nd.off + 1];
+  const int c = blockIdx.y * FILL_COLS + threadIdx.x, nrot = ar.count[2 * nd.off + 1];
   if (c >= nd.n1 + nd.n2) return;
   double* const U = mt.V + (size_t)nd.lo * mt.n + nd.lo + c;
   for (int r = nrot - 1; r >= 0; --r) {
@@ -1080,8 +1081,8 @@ void dc_merge_launch(const DcMatrix* mats, const DcNode* nodes, int count, int p
   // eight per SM
   const int cols = (largest + FILL_COLS - 1) / FILL_COLS;
   const int parts = std::max(1, std::min({64, (largest + 7) / 8, 2432 / std::max(1, cols * count)}));
-  dc_fill_kernel<<<dim3(cols, count, parts), FILL_COLS, 0, st>>>(mats, nodes, ar);
-  dc_rotate_kernel<<<dim3(cols, count), FILL_COLS, 0, st>>>(mats, nodes, ar);
+  dc_fill_kernel<<<dim3(count, cols, parts), FILL_COLS, 0, st>>>(mats, nodes, ar);
+  dc_rotate_kernel<<<dim3(count, cols), FILL_COLS, 0, st>>>(mats, nodes, ar);
   check_launch("merge");
 }
 
