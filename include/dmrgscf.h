@@ -246,8 +246,8 @@ dmrg_status dmrg_set_davidson(dmrg_ctx* ctx, int max_iter, double tol);
 dmrg_status dmrg_set_wait_timeout(dmrg_ctx* ctx, double seconds);
 
 /* The same bound, process-wide, for the kernel-level entry points
- * (dmrg_hpsi_contract, dmrg_eigh_batched and the CAS-SCF routines) called
- * after it; default 2 s. */
+ * (dmrg_grouped_gemm, dmrg_hpsi_contract, dmrg_eigh_batched and the CAS-SCF
+ * routines) called after it; default 2 s. */
 dmrg_status dmrg_set_kernel_wait_timeout(double seconds);
 
 /* tc_drain_terms (see dmrg_opts) of the kernel-level dmrg_hpsi_contract,

@@ -110,6 +110,9 @@ class Backend {
   virtual void copy_h2d_later(void* dst, const void* src, size_t bytes) = 0;
   virtual void copy_d2h(void* dst, const void* src, size_t bytes) = 0;
   virtual void sync() = 0;
+  // the same; throws "timeout: ..." when a wait of a float64 GEMM ran out
+  // (so do the copies to the host)
+  virtual void sync_checked() = 0;
   // Reads and clears the device error flag that bounded waits in kernels set;
   // throws "timeout: ..." when it was set.  Synchronises the stream.
   virtual void check_device_flag() = 0;

@@ -529,6 +529,10 @@ class CudaBackend : public Backend {
     }
   }
   void sync() override { CK(cudaStreamSynchronize(st)); }
+  void sync_checked() override {
+    CK(cudaStreamSynchronize(st));
+    check_digits();
+  }
   int* dflag = nullptr;  // device error flag of the bounded waits
   int* flag() {
     if (!dflag) {
@@ -809,6 +813,7 @@ class CudaBackend : public Backend {
     L.special = (int*)(inline_zero ? d + off[5] + (osp - ok) : ws + osp);
     L.scratch = (double*)(ws + osc);
     L.err = dig_err;
+    L.wait_ns = wait_ns_;
     L.sms = sms;
     dig_launch(L, st);
     launches += 2 + (L.nreds > 0);

@@ -1216,7 +1216,7 @@ void Engine::build_comp_from_normal(const Block& b, OpSet& dst, const std::vecto
           }
         }
         pb.run(be_);
-        be_->sync();
+        be_->sync_checked();
         be_->free(Y);
         be_->free(Gdev);
       }
@@ -1411,7 +1411,7 @@ std::unique_ptr<Block> Engine::renormalize(Block& enl, const SavedU& U, bool swi
       g1.run(be_, opt_.prec_renorm);
       g2.run(be_, opt_.prec_renorm);
     }
-    be_->sync();
+    be_->sync_checked();
     be_->free(T);
   }
   if (switch_to_comp) {
@@ -1437,7 +1437,7 @@ std::unique_ptr<Block> Engine::renormalize(Block& enl, const SavedU& U, bool swi
       }
     }
     build_comp_from_normal(*nb, *cb->ops, ck);
-    be_->sync();
+    be_->sync_checked();
     return cb;
   }
   return nb;
@@ -2624,7 +2624,7 @@ double Engine::optimize_bond(int i, bool l2r, double* trunc) {
   std::unique_ptr<Block> Re = l2r ? take(keep_R_, i) : nullptr;
   if (!Le) Le = enlarge(*L_[i], i);
   if (!Re) Re = enlarge(*R_[n_ - i - 2], i + 1);
-  be_->sync();
+  be_->sync_checked();
   double t1 = now_s();
   stats_.t_enlarge += t1 - t0;
   HPsiPlan plan;
@@ -2687,7 +2687,7 @@ double Engine::optimize_bond(int i, bool l2r, double* trunc) {
     R_[n_ - i - 1] = renormalize(*Re, *U, sw);
     RU_[n_ - i - 1] = std::move(U);
   }
-  be_->sync();
+  be_->sync_checked();
   const double t6 = now_s();
   stats_.t_renorm += t6 - t5;
   save_prev(i, *Le, *Re, plan, psi);

@@ -39,7 +39,7 @@ constexpr int OFF_TURN = NSTAGE * STAGE, TURN_BYTES = 32 * TURN_LD * 8;
 constexpr int SMEM_BYTES = OFF_TURN + 8 * TURN_BYTES + 1024;
 constexpr int CHUNK = 16;  // k-steps of 16 between drains: 256 exact terms
 constexpr int NTHREADS = 384;
-constexpr unsigned long long kWaitNs = 20000000000ull;  // every wait is on this CTA's own work
+constexpr unsigned long long kDrainNs = 2000000000ull;  // what a CTA that gave up waits for its own work in flight
 constexpr int kExpRange = 400;
 constexpr int kGraded = 8;  // the largest product may lie 2^8 below the product of the maxima
 
@@ -104,13 +104,25 @@ __device__ __forceinline__ bool try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return done != 0;
 }
-// bounded wait; false when it ran out or another role of the CTA gave up
-__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatile int* abort) {
-  if (try_wait(bar, parity)) return true;
+__device__ __forceinline__ bool test_wait(uint64_t* bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(done)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+// wait bounded by wait_ns (0: by its first probe); false when it ran out or
+// another role of the CTA gave up.  Every wait is on this CTA's own work.
+__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatile int* abort,
+                                         unsigned long long wait_ns) {
+  if (test_wait(bar, parity)) return true;
+  if (wait_ns == 0) return false;
   const unsigned long long t0 = global_ns();
   for (;;) {
     if (try_wait(bar, parity)) return true;
-    if (*abort || global_ns() - t0 > kWaitNs) return false;
+    if (*abort || global_ns() - t0 > wait_ns) return false;
   }
 }
 // columns of a tile on the tensor pipe (steps of 16)
@@ -262,7 +274,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     gemm_digits_kernel(const DigOperand* __restrict__ ops, const DigSeg* __restrict__ segs,
                        const DigTask* __restrict__ tasks, int ntasks, const unsigned char* __restrict__ pool,
                        const int* __restrict__ exps, const uint2* __restrict__ kmax,
-                       const int* __restrict__ special, double* __restrict__ scratch, int* __restrict__ err) {
+                       const int* __restrict__ special, double* __restrict__ scratch, int* __restrict__ err,
+                       unsigned long long wait_ns) {
   extern __shared__ unsigned char smraw[];
   __shared__ __align__(8) uint64_t bar[B_COUNT];
   __shared__ uint32_t tmem_base;
@@ -328,7 +341,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           const uint32_t total = (uint32_t)(na + nb) * kDigSlices * kDigUnit;
           for (int kb = 0; kb < nkb; ++kb, src += step) {
             const int st = q % NSTAGE;
-            if (!wait_bar(&bar[B_EMPTY + st], (uint32_t)(((q / NSTAGE) & 1) ^ 1), abort)) ok = false;
+            if (!wait_bar(&bar[B_EMPTY + st], (uint32_t)(((q / NSTAGE) & 1) ^ 1), abort, wait_ns)) ok = false;
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             if (lane == 0) arrive_expect(&bar[B_FULL + st], total);
@@ -353,12 +366,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           const int nkb = (ops[segs[k].a].k + 15) >> 4;
           for (int kb = 0; kb < nkb; ++kb) {
             const bool fresh = kb % CHUNK == 0;
-            if (fresh && nd > 0 && !wait_bar(&bar[B_SE], (uint32_t)((nd - 1) & 1), abort)) {
+            if (fresh && nd > 0 && !wait_bar(&bar[B_SE], (uint32_t)((nd - 1) & 1), abort, wait_ns)) {
               ok = false;
               break;
             }
             const int st = q % NSTAGE;
-            if (!wait_bar(&bar[B_FULL + st], (uint32_t)((q / NSTAGE) & 1), abort)) {
+            if (!wait_bar(&bar[B_FULL + st], (uint32_t)((q / NSTAGE) & 1), abort, wait_ns)) {
               ok = false;
               break;
             }
@@ -394,7 +407,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       consumed = q;
       commit(&bar[B_DONE]);
       const unsigned long long t0 = global_ns();
-      while (!try_wait(&bar[B_DONE], 0u) && global_ns() - t0 < kWaitNs) __nanosleep(64);
+      while (!try_wait(&bar[B_DONE], 0u) && global_ns() - t0 < kDrainNs) __nanosleep(64);
     } else if (warp == 2) {
       // ---------------------------------------------------------- segment data
       int q = 0;
@@ -425,7 +438,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           bmax = __reduce_max_sync(0xffffffffu, bmax);
           const int plain = (special[sg.a] | special[sg.b]) ||
                             (rel && (rel + kGraded < 8192u || top + kGraded < amax + bmax));
-          ok = __all_sync(0xffffffffu, wait_bar(&bar[B_ME + (q & 1)], (uint32_t)(((q >> 1) & 1) ^ 1), abort));
+          ok = __all_sync(0xffffffffu, wait_bar(&bar[B_ME + (q & 1)], (uint32_t)(((q >> 1) & 1) ^ 1), abort, wait_ns));
           if (!ok) break;
           Meta& m = meta[q & 1];
           const int r0 = tasks[t].r0, c0 = tasks[t].c0, mm = tasks[t].m, nn = tasks[t].n;
@@ -461,7 +474,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       int W = 0, ldc = 0, nrow = 0, gc = 0, gr0 = 0, sc = 1;
       bool busy = false;  // the warp has outputs of the block
       for (int k = 0; ok && k < sc; ++k, ++q) {
-        ok = __all_sync(0xffffffffu, wait_bar(&bar[B_MF + (q & 1)], (uint32_t)((q >> 1) & 1), abort));
+        ok = __all_sync(0xffffffffu, wait_bar(&bar[B_MF + (q & 1)], (uint32_t)((q >> 1) & 1), abort, wait_ns));
         if (!ok) break;
         const Meta& m = meta[q & 1];
         if (k == 0) {
@@ -491,7 +504,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           l[c] = 0u;
         }
         for (int kb = 0; kb < nkb; kb += CHUNK) {
-          ok = __all_sync(0xffffffffu, wait_bar(&bar[B_SF], (uint32_t)(nd & 1), abort));
+          ok = __all_sync(0xffffffffu, wait_bar(&bar[B_SF], (uint32_t)(nd & 1), abort, wait_ns));
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
@@ -581,7 +594,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     // copies still in flight land before the CTA exits
     for (int q = consumed; q < produced; ++q) {
       const unsigned long long t0 = global_ns();
-      while (!try_wait(&bar[B_FULL + q % NSTAGE], (uint32_t)((q / NSTAGE) & 1)) && global_ns() - t0 < kWaitNs)
+      while (!try_wait(&bar[B_FULL + q % NSTAGE], (uint32_t)((q / NSTAGE) & 1)) && global_ns() - t0 < kDrainNs)
         __nanosleep(64);
     }
   }
@@ -614,7 +627,7 @@ void dig_launch(const DigLaunch& L, cudaStream_t st) {
   e = cudaGetLastError();
   if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: digit split: ") + cudaGetErrorString(e));
   gemm_digits_kernel<<<std::min(L.sms, L.ntasks), NTHREADS, SMEM_BYTES, st>>>(
-      L.ops, L.segs, L.tasks, L.ntasks, L.pool, L.exps, L.kmax, L.special, L.scratch, L.err);
+      L.ops, L.segs, L.tasks, L.ntasks, L.pool, L.exps, L.kmax, L.special, L.scratch, L.err, L.wait_ns);
   e = cudaGetLastError();
   if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: digit gemm: ") + cudaGetErrorString(e));
   if (L.nreds > 0) {

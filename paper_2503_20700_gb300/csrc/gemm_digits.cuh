@@ -142,6 +142,7 @@ struct DigLaunch {
                        // of the rows divided by their maxima (x) and as they are (y); 0: a zero column
   int* special;        // nops, zero at launch
   int* err;            // host-mapped flag, set when a bounded wait ran out
+  unsigned long long wait_ns;  // bound of every wait (0: its first probe)
   int sms;
 };
 void dig_launch(const DigLaunch& L, cudaStream_t st);
