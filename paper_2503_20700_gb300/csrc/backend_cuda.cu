@@ -409,23 +409,34 @@ class CudaBackend : public Backend {
   }
   std::string name() const override { return "cuda"; }
   void* alloc(size_t b) override {
+    void* p = try_alloc(b);
+    if (!p) {
+      if (budget_ && used + b > budget_)
+        throw std::runtime_error("out of device memory (budget of " + std::to_string(budget_) + " bytes: " +
+                                 std::to_string(used) + " held, " + std::to_string(b) + " requested)");
+      throw std::runtime_error("out of device memory (" + std::to_string(b) + " bytes)");
+    }
+    return p;
+  }
+  // the same; nullptr when there is no room for it
+  void* try_alloc(size_t& b) {
     void* p = nullptr;
     if (b == 0) b = 8;
     while (budget_ && used + b > budget_ && make_room && make_room()) {
     }
-    if (budget_ && used + b > budget_)
-      throw std::runtime_error("out of device memory (budget of " + std::to_string(budget_) + " bytes: " +
-                               std::to_string(used) + " held, " + std::to_string(b) + " requested)");
-    cudaError_t e = cudaMallocAsync(&p, b, st);
-    if (e != cudaSuccess) {
+    if (budget_ && used + b > budget_) return nullptr;
+    if (cudaMallocAsync(&p, b, st) != cudaSuccess) {
       cudaGetLastError();
-      throw std::runtime_error("out of device memory (" + std::to_string(b) + " bytes)");
+      return nullptr;
     }
+    count(b);
+    live.push_back({p, b});
+    return p;
+  }
+  void count(size_t b) {
     used += b;
     peak_bytes = std::max(peak_bytes, used);
     window_peak = std::max(window_peak, used);
-    live.push_back({p, b});
-    return p;
   }
   void free(void* p) override {
     if (!p) return;
@@ -655,6 +666,10 @@ class CudaBackend : public Backend {
     }
     std::vector<char> digits;
     const bool any = choose_digits(groups, segs, digits);
+    if (any) {
+      if (rec) CK(cudaEventRecord(rec->a, st));
+      gemm_digits(groups, segs, digits);
+    }
     std::vector<GemmTile> tiles;
     for (size_t gi = 0; gi < groups.size(); ++gi) {
       auto& g = groups[gi];
@@ -662,13 +677,9 @@ class CudaBackend : public Backend {
       for (int r = 0; r < g.m; r += kTM)
         for (int c = 0; c < g.n; c += kTN) tiles.push_back({(int)gi, r, c, 0});
     }
-    if (any) {
-      if (rec) CK(cudaEventRecord(rec->a, st));
-      gemm_digits(groups, segs, digits);
-      if (tiles.empty()) {
-        if (rec) CK(cudaEventRecord(rec->b, st));
-        return;
-      }
+    if (any && tiles.empty()) {
+      if (rec) CK(cudaEventRecord(rec->b, st));
+      return;
     }
     std::vector<size_t> off;
     char* d = upload({{groups.data(), groups.size() * sizeof(GemmGroup)},
@@ -710,9 +721,9 @@ class CudaBackend : public Backend {
     return any && std::max(dd / sms, td) + kDigLaunchClocks < std::max(df / sms, tf);
   }
   // Digit pool of one launch (bytes): groups are taken until their operands
-  // reach it (a single larger group still runs whole).  The pool is work
-  // space like the task lists: it is outside the context's budget, so under a
-  // budget it is kept to a sixteenth of it.
+  // reach it.  It counts against the context's budget like any allocation, and
+  // is kept to a sixteenth of it; a single larger group is tried whole, and one
+  // that there is no room for runs on the FMA kernel, which needs none.
   size_t dig_pool_cap() const {
     const size_t cap = size_t(2) << 30;
     return budget_ ? std::max<size_t>(size_t(16) << 20, std::min(cap, budget_ / 16)) : cap;
@@ -725,29 +736,44 @@ class CudaBackend : public Backend {
       throw std::runtime_error("timeout: a bounded wait in the digit GEMM ran out");
     }
   }
+  // clears digits[i] of the groups left to the FMA kernel
   void gemm_digits(const std::vector<GemmGroup>& groups, const std::vector<GemmSeg>& segs,
-                   const std::vector<char>& digits) {
+                   std::vector<char>& digits) {
     if (!dig_err) {
       dig_err = (int*)PinnedPool::get().take(sizeof(int), &dig_err_cap);
       *dig_err = 0;
     }
     DigPlanner pl;
     const size_t cap = dig_pool_cap();
+    std::vector<size_t> planned;
+    auto add = [&](size_t i) { pl.add(groups[i], segs.data(), dig_parts(groups[i], segs.data())); };
+    auto run = [&]() {
+      if (!run_digits(pl.plan)) {
+        // no room: its groups one by one
+        for (size_t i : planned) {
+          pl.clear();
+          add(i);
+          if (planned.size() == 1 || !run_digits(pl.plan)) digits[i] = 0;
+        }
+      }
+      pl.clear();
+      planned.clear();
+    };
     for (size_t i = 0; i < groups.size(); ++i) {
       if (!digits[i]) continue;
-      pl.add(groups[i], segs.data(), dig_parts(groups[i], segs.data()));
-      if (pl.pool_bytes() < cap) continue;
-      run_digits(pl.plan);
-      pl.clear();
+      add(i);
+      planned.push_back(i);
+      if (pl.pool_bytes() >= cap) run();
     }
-    run_digits(pl.plan);
+    run();
   }
   static constexpr size_t kDigKept = size_t(64) << 20;
   char* dig_ws = nullptr;
   size_t dig_ws_cap = 0;
   std::vector<char> dig_zero;
-  void run_digits(DigPlan& p) {
-    if (p.tasks.empty()) return;
+  // false when there is no room for the work space
+  bool run_digits(DigPlan& p) {
+    if (p.tasks.empty()) return true;
     // longest tasks first, dealt round-robin over the persistent CTAs
     std::vector<double> w(p.tasks.size());
     std::vector<int> order(p.tasks.size());
@@ -763,28 +789,32 @@ class CudaBackend : public Backend {
     const size_t ox = al(p.pool_bytes()), ok = ox + al(p.nexp * sizeof(int));
     const size_t osp = ok + al(p.nkmax * sizeof(uint2)), osc = osp + al(p.ops.size() * sizeof(int));
     // Work space of a launch sequence: small ones share a block that the backend
-    // keeps (stream order separates them), larger ones come and go.  The part
-    // that starts at zero is uploaded with the lists while it is small.
+    // keeps (stream order separates them; not under a budget, which it would
+    // take from), larger ones come and go.  The part that starts at zero is
+    // uploaded with the lists while it is small.
     char* ws = nullptr;
-    const size_t bytes = osc + (size_t)p.scratch * sizeof(double), nzero = osc - ok;
-    const bool keep = bytes <= kDigKept;
-    if (keep && bytes <= dig_ws_cap) {
-      ws = dig_ws;
+    size_t bytes = osc + (size_t)p.scratch * sizeof(double);
+    const size_t nzero = osc - ok;
+    const bool keep = !budget_ && bytes <= kDigKept;
+    if (!keep) {
+      ws = (char*)try_alloc(bytes);
+      if (!ws) return false;
     } else {
-      const size_t want = keep ? std::min(kDigKept, std::max(2 * bytes, size_t(1) << 20)) : bytes;
-      if (keep && dig_ws) {
-        CK(cudaFreeAsync(dig_ws, st));
+      if (bytes > dig_ws_cap) {
+        if (dig_ws) CK(cudaFreeAsync(dig_ws, st));
         dig_ws = nullptr;
         dig_ws_cap = 0;
-      }
-      if (cudaMallocAsync((void**)&ws, want, st) != cudaSuccess) {
-        cudaGetLastError();
-        throw std::runtime_error("out of device memory (" + std::to_string(want) + " bytes)");
-      }
-      if (keep) {
-        dig_ws = ws;
+        const size_t want = std::min(kDigKept, std::max(2 * bytes, size_t(1) << 20));
+        if (cudaMallocAsync((void**)&dig_ws, want, st) != cudaSuccess) {
+          cudaGetLastError();
+          dig_ws = nullptr;
+          return false;
+        }
         dig_ws_cap = want;
       }
+      ws = dig_ws;
+      count(bytes);  // what a budget has to leave for this launch
+      used -= bytes;
     }
     const bool inline_zero = nzero <= size_t(32) << 10;
     if (inline_zero) dig_zero.resize(std::max(dig_zero.size(), nzero), 0);
@@ -817,7 +847,8 @@ class CudaBackend : public Backend {
     L.sms = sms;
     dig_launch(L, st);
     launches += 2 + (L.nreds > 0);
-    if (!keep) CK(cudaFreeAsync(ws, st));
+    if (!keep) free(ws);
+    return true;
   }
 
   void hpsi(const HpsiBlock* blocks, const HpsiItem* items, const HpsiTask* tasks, int ntasks,
@@ -963,8 +994,9 @@ class CudaBackend : public Backend {
   // cooperative launches of the tridiagonalisation (largest matrices first,
   // group sizes from jac_assign_groups), then the levels of merges with their
   // products on the grouped GEMM, then the reflectors.  Work space (two more
-  // copies of the matrices) is kept to the digit pool's bound, the batch cut
-  // into parts of it; a larger single matrix runs whole.
+  // copies of the matrices) counts against the budget and is kept to the digit
+  // pool's bound, the batch cut into parts of it, and into smaller ones where
+  // there is no room; a single matrix runs whole.
   int tri_cap = 0;
   void eigh(const std::vector<EighTask>& tasks) override {
     if (tasks.empty()) return;
@@ -1037,16 +1069,23 @@ class CudaBackend : public Backend {
     const size_t oW = take(tridiag_wide(sizes[0], (int)sum, tri_cap) * 8);
     const size_t oX = take(8 * sum * 8), obar = take(t.size() * sizeof(unsigned)), osc = take(t.size() * 8);
     const size_t om = take(t.size() * sizeof(DcMatrix)), on = take(nodes.size() * sizeof(DcNode));
-    char* ws = nullptr;
-    if (cudaMallocAsync((void**)&ws, at, st) != cudaSuccess) {
-      cudaGetLastError();
-      throw std::runtime_error("out of device memory (" + std::to_string(at) + " bytes)");
+    char* ws = t.size() > 1 ? (char*)try_alloc(at) : (char*)alloc(at);
+    if (!ws) {
+      // no room for all at once
+      eigh_large(std::vector<EighTask>(t.begin(), t.begin() + t.size() / 2));
+      eigh_large(std::vector<EighTask>(t.begin() + t.size() / 2, t.end()));
+      return;
     }
     struct Free {
-      char* p;
-      cudaStream_t s;
-      ~Free() { cudaFreeAsync(p, s); }
-    } release{ws, st};
+      CudaBackend* b;
+      void* p;
+      ~Free() {
+        try {
+          b->free(p);
+        } catch (...) {  // a sticky error is thrown by the next call
+        }
+      }
+    } release{this, ws};
     auto dbl = [&](size_t o) { return (double*)(ws + o); };
     DcArrays ar{};
     ar.d = dbl(oD[0]);
