@@ -411,17 +411,25 @@ static void gemm1(Backend* be, double* C, int m, int n, int ldc, const double* A
 // its time there.  Measured, 600 vectors of 200 x 200 (40 core, 30 active
 // orbitals), the seven products of the active space and the gradient with their
 // splits: 1.83 -> 0.82 ms.
-static void long_gemm(Backend* be, double* C, int m, int n, int ldc, const double* A, const double* B, size_t ldb,
-                      int transB, size_t K) {
+static void long_gemm(Backend* be, double* C, int m, int n, int ldc, const double* A, size_t lda, const double* B,
+                      size_t ldb, int transB, size_t K) {
   const size_t tiles = (size_t)((m + 127) / 128) * ((n + 63) / 64);
   const size_t want = std::max<size_t>(1, 304 / tiles);
   const size_t step = std::min<size_t>(1024, std::max<size_t>(64, (K / want + 15) / 16 * 16));
   std::vector<GemmGroup> g{{C, m, n, ldc, 0, 0}};
   std::vector<GemmSeg> s;
   for (size_t k = 0; k < K; k += step)
-    s.push_back({A + k, B + (transB ? k : k * ldb), (int)std::min(step, K - k), (int)K, (int)ldb, 0, transB, 1.0});
+    s.push_back({A + k, B + (transB ? k : k * ldb), (int)std::min(step, K - k), (int)lda, (int)ldb, 0, transB, 1.0});
   g[0].seg_count = (int)s.size();
   be->gemm(g, s, Precision::FP64);
+}
+
+// Vectors of a piece of such a product, `doubles` gathered per vector: its
+// copies of columns and rows stay below kPieceBytes each (and their digits below
+// four times that), whatever the rank; 600 vectors of 200 x 40 are one piece.
+constexpr size_t kPieceBytes = size_t(128) << 20;
+static int piece_vectors(int rank, size_t doubles) {
+  return (int)std::max<size_t>(1, std::min<size_t>(rank, kPieceBytes / (8 * std::max<size_t>(1, doubles))));
 }
 
 Casscf::Casscf(Backend* be) : be_(be) {}
@@ -546,7 +554,8 @@ void Casscf::transform(const double* R, const double* h, const double* L, int ra
 // Pieces shared by the active-space problem and the gradient.
 struct FockParts {
   double *FI, *FA, *La, *v, *w;
-  double* Aa;  // L^k[q][act] as [q][k, act] (with an active density)
+  double* Aa;  // L^k[q][act] as [q][k, act] of the last `piece` vectors or fewer (with an active density)
+  int piece;
 };
 
 static FockParts fock_parts(Backend* be, Casscf::Dev& d, const double* dh, const double* dL, int rank,
@@ -565,25 +574,36 @@ static FockParts fock_parts(Backend* be, Casscf::Dev& d, const double* dh, const
   // Kc = sum_k L^k[:, core] L^k[core, :]
   double* Kc = d.alloc(nn);
   if (ncore > 0) {
-    const size_t K = (size_t)rank * ncore;
-    double *Ac = d.raw(K * nb), *Bc = d.raw(K * nb);
-    k_gather_cols<<<grid_for(K * nb), 256, 0, ST>>>(dL, rank, nb, 0, ncore, Ac);
-    k_gather_rows<<<grid_for(K * nb), 256, 0, ST>>>(dL, rank, nb, 0, ncore, Bc);
-    long_gemm(be, Kc, nb, nb, nb, Ac, Bc, nb, 0, K);
+    const size_t per = (size_t)ncore * nb;
+    const int piece = piece_vectors(rank, per);
+    double *Ac = d.raw(piece * per), *Bc = d.raw(piece * per);
+    for (int k0 = 0; k0 < rank; k0 += piece) {
+      const int kn = std::min(piece, rank - k0);
+      k_gather_cols<<<grid_for(kn * per), 256, 0, ST>>>(dL + nn * k0, kn, nb, 0, ncore, Ac);
+      k_gather_rows<<<grid_for(kn * per), 256, 0, ST>>>(dL + nn * k0, kn, nb, 0, ncore, Bc);
+      const size_t K = (size_t)kn * ncore;
+      long_gemm(be, Kc, nb, nb, nb, Ac, K, Bc, nb, 0, K);
+    }
   }
   f.FI = d.alloc(nn);
   k_axpbypcz<<<grid_for(nn), 256, 0, ST>>>(f.FI, nn, 1.0, dh, 2.0, J, -1.0, Kc);
   f.FA = nullptr;
   if (dgamma) {
     // M^k = L^k[:, act] gamma ; KA = sum_k M^k L^k[act, :]
-    const size_t K = (size_t)rank * ncas;
-    f.Aa = d.raw(K * nb);
-    double *Ba = d.raw(K * nb), *M = d.alloc(K * nb);
-    k_gather_cols<<<grid_for(K * nb), 256, 0, ST>>>(dL, rank, nb, ncore, ncas, f.Aa);
-    k_gather_rows<<<grid_for(K * nb), 256, 0, ST>>>(dL, rank, nb, ncore, ncas, Ba);
-    gemm1(be, M, nb * rank, ncas, ncas, f.Aa, ncas, 0, dgamma, ncas, 0, ncas, 1.0);
+    const size_t per = (size_t)ncas * nb;
+    f.piece = piece_vectors(rank, per);
+    f.Aa = d.raw(f.piece * per);
     double* KA = d.alloc(nn);
-    long_gemm(be, KA, nb, nb, nb, M, Ba, nb, 0, K);
+    double *Ba = d.raw(f.piece * per), *M = d.raw(f.piece * per);
+    for (int k0 = 0; k0 < rank; k0 += f.piece) {
+      const int kn = std::min(f.piece, rank - k0);
+      k_gather_cols<<<grid_for(kn * per), 256, 0, ST>>>(dL + nn * k0, kn, nb, ncore, ncas, f.Aa);
+      k_gather_rows<<<grid_for(kn * per), 256, 0, ST>>>(dL + nn * k0, kn, nb, ncore, ncas, Ba);
+      be->memset0(M, kn * per * sizeof(double));
+      gemm1(be, M, nb * kn, ncas, ncas, f.Aa, ncas, 0, dgamma, ncas, 0, ncas, 1.0);
+      const size_t K = (size_t)kn * ncas;
+      long_gemm(be, KA, nb, nb, nb, M, K, Ba, nb, 0, K);
+    }
     f.FA = d.alloc(nn);
     k_axpbypcz<<<grid_for(nn), 256, 0, ST>>>(f.FA, nn, 1.0, JA, -0.5, KA, 0.0, nullptr);
   }
@@ -694,7 +714,13 @@ void Casscf::fock_dev(const double* dh, const double* dL, int rank, int nb, int 
   be_->gemm(g, s, Precision::FP64);
   // F2[t, q] = sum_k sum_u W^k[t,u] L^k[q, c+u]
   double* F2 = d.alloc((size_t)ncas * nb);
-  long_gemm(be_, F2, ncas, nb, nb, W, f.Aa, (size_t)rank * ncas, 1, (size_t)rank * ncas);
+  for (int k0 = 0; k0 < rank; k0 += f.piece) {
+    const int kn = std::min(f.piece, rank - k0);
+    if (f.piece < rank)
+      k_gather_cols<<<grid_for((size_t)kn * ncas * nb), 256, 0, ST>>>(dL + nn * k0, kn, nb, ncore, ncas, f.Aa);
+    const size_t K = (size_t)kn * ncas;
+    long_gemm(be_, F2, ncas, nb, nb, W + (size_t)k0 * ncas, (size_t)rank * ncas, f.Aa, K, 1, K);
+  }
   k_assemble_fock<<<grid_for(nn), 256, 0, ST>>>(f.FI, f.FA, dg, F2, nb, ncore, ncas, F);
   if (fdiag) k_fock_diag<<<grid_for(nb), 256, 0, ST>>>(f.FI, f.FA, nb, fdiag);
   be_->sync();
