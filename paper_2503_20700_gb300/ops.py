@@ -173,8 +173,8 @@ def eigh_batched(mats, device=0):
     if st != 0:
         raise DmrgError(st, lib.dmrg_last_error(None).decode())
     out, o, ow = [], 0, 0
-    for n in ns.tolist():  # disjoint parts of the two results
-        out.append((w[ow:ow + n], v[o:o + n * n].reshape(n, n)))
+    for n in ns.tolist():  # arrays of their own: one that is kept does not keep the batch
+        out.append((w[ow:ow + n].copy(), v[o:o + n * n].reshape(n, n).copy()))
         o += n * n
         ow += n
     return out

@@ -1,5 +1,6 @@
-"""A batch of the float64 eigensolver with more merges on a level than a grid's
-y and z dimensions count (65535): two for each 33 x 33 matrix.
+"""Batches of the float64 eigensolver: one with more merges on a level than a
+grid's y and z dimensions count (65535: two for each 33 x 33 matrix), and what
+the results hold on to.
 
 Tolerances as in test_gpu_eigh.py: 30 n eps ||A||, and 30 n eps from
 orthonormal."""
@@ -25,3 +26,11 @@ def test_many_small_matrices():
     # the same numbers wherever a matrix stands in the batch
     for i in range(60, count):
         assert np.array_equal(res[i][0], w[i % 60]) and np.array_equal(res[i][1], V[i % 60])
+
+
+def test_results_are_arrays_of_their_own():
+    import paper_2503_20700_gb300 as pkg
+    pkg.load()
+    for n in (5, 70):
+        for w, V in pkg.ops.eigh_batched([np.eye(n), 2.0 * np.eye(n)]):
+            assert w.base is None and V.base is None and V.flags.c_contiguous and V.flags.writeable
