@@ -112,9 +112,7 @@ typedef struct {
                              products with a new sector histogram run the
                              candidate schedules in turn (every one computes
                              the full product) and the fastest is kept for
-                             that histogram.  0 (default): the first candidate
-                             (without its clusters where the sectors' tiles
-                             would leave their slots empty).
+                             that histogram.  0 (default): the first candidate.
                              Results differ between schedules only by FP32
                              summation order                                  */
 } dmrg_opts;
@@ -263,11 +261,15 @@ dmrg_status dmrg_set_kernel_tc_drain_terms(int terms);
  * tile grouped that many at a time share stage 1)}.  dmrg_tc_shape_candidates
  * writes the candidates the autotuner times, the default first, as groups of
  * four ints into shapes (room for cap groups; *count receives their number).
+ * The default runs without its clusters of two where the sectors' tiles would
+ * leave their slots empty, with autotuning as without it (dmrg_tc_launch_cluster
+ * tells); the other candidates run as listed.
  */
 dmrg_status dmrg_tc_shape_candidates(int* shapes, int cap, int* count);
 
 /* Schedule candidate (index into dmrg_tc_shape_candidates) of the kernel-level
- * dmrg_hpsi_contract with DMRG_SPLIT_HPSI_TC (process-wide; default 0). */
+ * dmrg_hpsi_contract with DMRG_SPLIT_HPSI_TC (process-wide; default 0, the
+ * default schedule). */
 dmrg_status dmrg_set_kernel_tc_shape(int candidate);
 
 /* Turns the autotuning of tc_autotune (see dmrg_opts) on or off for a
@@ -275,10 +277,14 @@ dmrg_status dmrg_set_kernel_tc_shape(int candidate);
 dmrg_status dmrg_set_tc_autotune(dmrg_ctx* ctx, int on);
 
 /* The schedule of the last planned tcgen05 H_eff psi launch of ctx: shape[4]
- * as above; ms[k] (k < min(cap, *count)) the CUDA-event time in ms of one
+ * the candidate as listed; ms[k] (k < min(cap, *count)) the CUDA-event time in ms of one
  * product under candidate k for that product's sector histogram (-1: not
  * timed, or autotuning off).  DMRG_ESTATE before the first tcgen05 product. */
 dmrg_status dmrg_tc_schedule_info(const dmrg_ctx* ctx, int* shape, double* ms, int cap, int* count);
+
+/* CTAs per cluster (1, 2 or 4) of that launch.  DMRG_ESTATE before the first
+ * tcgen05 product. */
+dmrg_status dmrg_tc_launch_cluster(const dmrg_ctx* ctx, int* cluster);
 
 /* Change the bond dimension used by subsequent sweeps. */
 dmrg_status dmrg_set_bond_dim(dmrg_ctx* ctx, int D);

@@ -94,6 +94,8 @@ def load(path=None):
     lib.dmrg_set_tc_autotune.restype = I
     lib.dmrg_tc_schedule_info.argtypes = [P, ip, dp, I, ip]
     lib.dmrg_tc_schedule_info.restype = I
+    lib.dmrg_tc_launch_cluster.argtypes = [P, ip]
+    lib.dmrg_tc_launch_cluster.restype = I
     lib.dmrg_set_kernel_wait_timeout.argtypes = [D]
     lib.dmrg_set_kernel_wait_timeout.restype = I
     lib.dmrg_set_davidson.argtypes = [P, I, D]
@@ -344,14 +346,17 @@ class DMRG:
 
     def tc_schedule(self):
         """Schedule of the last planned tcgen05 product: {"shape": (tile width,
-        chunks per CTA, order, CTAs per cluster), "ms": per-candidate product
-        times (-1: not timed)}."""
+        chunks per CTA, order, CTAs per cluster) of the candidate, "ms":
+        per-candidate product times (-1: not timed), "cluster": CTAs per cluster
+        of the launch}."""
         shape = np.zeros(4, dtype=np.int32)
         n = ctypes.c_int()
         ms = np.full(16, -1.0)
         _check(self._lib, self._ctx, self._lib.dmrg_tc_schedule_info(self._ctx, _ip(shape), _dp(ms), 16,
                                                                       ctypes.byref(n)))
-        return {"shape": tuple(int(x) for x in shape), "ms": [float(x) for x in ms[:n.value]]}
+        cl = ctypes.c_int()
+        _check(self._lib, self._ctx, self._lib.dmrg_tc_launch_cluster(self._ctx, ctypes.byref(cl)))
+        return {"shape": tuple(int(x) for x in shape), "ms": [float(x) for x in ms[:n.value]], "cluster": cl.value}
 
     def set_davidson(self, max_iter, tol):
         _check(self._lib, self._ctx, self._lib.dmrg_set_davidson(self._ctx, int(max_iter), float(tol)))

@@ -394,6 +394,13 @@ dmrg_status dmrg_tc_schedule_info(const dmrg_ctx* c, int* shape, double* ms, int
   return DMRG_OK;
 }
 
+dmrg_status dmrg_tc_launch_cluster(const dmrg_ctx* c, int* cluster) {
+  if (!c || !c->eng || !cluster) return fail(nullptr, DMRG_EINVAL, "invalid argument");
+  *cluster = c->eng->tc_launch_cluster();
+  if (*cluster == 0) return fail(nullptr, DMRG_ESTATE, "no tcgen05 product planned yet");
+  return DMRG_OK;
+}
+
 dmrg_status dmrg_set_kernel_wait_timeout(double seconds) {
   if (!(seconds >= 0.0) || seconds > 3600.0) return fail(nullptr, DMRG_EINVAL, "seconds must be in [0, 3600]");
   g_kernel_wait_ns.store((unsigned long long)(seconds * 1e9));
@@ -748,14 +755,12 @@ dmrg_status dmrg_hpsi_contract(const double* A, int64_t a_len, const double* P, 
     void* pool = nullptr;
     size_t scr;
     if (tc) {
-      const int cand = g_kernel_tc_cand.load();
-      dmrg::TcShape shape = dmrg::tc_shape_candidates()[cand];
       auto ctas = [&](int cluster) {
         const int n = dmrg::hpsi_tc_max_ctas(cluster);
         return n > 0 ? n : be->sm_count() / cluster * cluster;
       };
       dmrg::hpsi_tc_operands(hb, hi, [&](size_t bytes) { return pool = be->alloc(bytes); }, tp);
-      if (cand == 0) shape = dmrg::tc_sized_shape(shape, hb, tp.items, ctas(shape.cluster), ctas(1));
+      const dmrg::TcShape shape = dmrg::tc_candidate_shape(g_kernel_tc_cand.load(), hb, tp.items, ctas);
       dmrg::hpsi_tc_schedule(hb, tp, shape, ctas(shape.cluster));
       tasks = tp.tasks;
       reds = tp.reds;

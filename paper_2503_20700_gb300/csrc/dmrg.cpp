@@ -1707,9 +1707,8 @@ void Engine::plan_hpsi(Block& Le, Block& Re, HPsiPlan& plan) {
         while (plan.tc_cand < (int)nc && rec.ms[plan.tc_cand] >= 0) ++plan.tc_cand;
       }
     }
-    TcShape shape = tc_shape_candidates()[plan.tc_cand];
-    if (!opt_.tc_autotune)
-      shape = tc_sized_shape(shape, blocks, tp.items, tc_ctas_for(shape.cluster), tc_ctas_for(1));
+    const TcShape shape =
+        tc_candidate_shape(plan.tc_cand, blocks, tp.items, [&](int cluster) { return tc_ctas_for(cluster); });
     hpsi_tc_schedule(blocks, tp, shape, tc_ctas_for(shape.cluster));
     if (opt_.debug_bounds) {
       const std::string bad = tc_plan_check(tp, blocks);
@@ -1717,6 +1716,7 @@ void Engine::plan_hpsi(Block& Le, Block& Re, HPsiPlan& plan) {
     }
     last_tc_key_ = opt_.tc_autotune ? plan.tune_key : 0;
     last_tc_cand_ = plan.tc_cand;
+    last_tc_cluster_ = shape.cluster;
     have_tc_plan_ = true;
   } else {
     scr = hpsi_plan_tasks(blocks, items, plan.prec, tasks, reds);
@@ -1846,14 +1846,16 @@ int Engine::tc_ctas_for(int cluster) const {
 
 void Engine::tc_reschedule(HPsiPlan& plan, int candidate) {
   be_->sync();  // the old lists and scratch may still be read by queued work
-  hpsi_tc_schedule(plan.tc_blocks, *plan.tcp, tc_shape_candidates()[candidate],
-                   tc_ctas_for(tc_shape_candidates()[candidate].cluster));
+  const TcShape shape = tc_candidate_shape(candidate, plan.tc_blocks, plan.tcp->items,
+                                           [&](int cluster) { return tc_ctas_for(cluster); });
+  hpsi_tc_schedule(plan.tc_blocks, *plan.tcp, shape, tc_ctas_for(shape.cluster));
   if (opt_.debug_bounds) {
     const std::string bad = tc_plan_check(*plan.tcp, plan.tc_blocks);
     if (!bad.empty()) throw std::logic_error("internal: tcgen05 plan: " + bad);
   }
   plan.tc_cand = candidate;
   last_tc_cand_ = candidate;
+  last_tc_cluster_ = shape.cluster;
   tc_upload_schedule(plan);
 }
 

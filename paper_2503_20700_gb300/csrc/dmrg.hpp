@@ -290,6 +290,7 @@ class Engine {
   // tc_shape_candidates() for its sector histogram (-1: not timed); returns
   // false when no tcgen05 product was planned yet.
   bool tc_schedule_info(int shape[4], std::vector<double>* ms) const;
+  int tc_launch_cluster() const { return have_tc_plan_ ? last_tc_cluster_ : 0; }
   // device and pinned-host bytes of the stored blocks, the largest one, and
   // the largest working memory of a bond beyond the stored blocks so far
   void memory_detail(size_t* dev, size_t* host, size_t* max_block, size_t* max_extra,
@@ -380,6 +381,7 @@ class Engine {
   std::map<uint64_t, TuneRec> tune_cache_;
   uint64_t last_tc_key_ = 0;
   int last_tc_cand_ = -1;
+  int last_tc_cluster_ = 0;
   bool have_tc_plan_ = false;
   void build_initial_right();
   void plan_hpsi(Block& Le, Block& Re, struct HPsiPlan& plan);

@@ -146,6 +146,11 @@ void hpsi_tc_schedule(const std::vector<HpsiBlock>& blocks, TcPlan& plan, const 
 // two, of one.  Partial tiles and sums are the same either way.
 TcShape tc_sized_shape(const TcShape& shape, const std::vector<HpsiBlock>& blocks, const std::vector<TcItem>& items,
                        int ncta, int ncta1);
+// Candidate `cand` of tc_shape_candidates for these blocks: the default (0) is
+// sized by that rule, wherever it is asked for (with autotuning or without, by
+// index or not), the others are as listed.  ctas: CTAs of a launch by cluster.
+TcShape tc_candidate_shape(int cand, const std::vector<HpsiBlock>& blocks, const std::vector<TcItem>& items,
+                           const std::function<int(int)>& ctas);
 // Key of the sector histogram of a contraction (block shapes in 64-row and
 // 64-column steps with their item counts on a log scale, and the CTA count):
 // contractions with equal keys share an autotuned shape.

@@ -95,6 +95,12 @@ TcShape tc_sized_shape(const TcShape& shape, const std::vector<HpsiBlock>& block
   return r;
 }
 
+TcShape tc_candidate_shape(int cand, const std::vector<HpsiBlock>& blocks, const std::vector<TcItem>& items,
+                           const std::function<int(int)>& ctas) {
+  const TcShape s = tc_shape_candidates()[cand];
+  return cand == 0 ? tc_sized_shape(s, blocks, items, ctas(s.cluster), ctas(1)) : s;
+}
+
 void hpsi_tc_operands(const std::vector<HpsiBlock>& blocks, const std::vector<HpsiItem>& items,
                       const std::function<void*(size_t)>& alloc, TcPlan& plan) {
   plan = TcPlan();
