@@ -372,6 +372,9 @@ __device__ void tridiag_one(const DcMatrix& mt, const DcArrays& ar, int mat, int
   power_of_two(mx, scale, inv);
   if (me == scribe && tid == 0) ar.scale[mat] = scale;
   for (int lr = warp; lr < nloc; lr += TRI_WARPS) {
+    // row 0 goes on in v alone; in global memory the scribe puts its reflector
+    // there without waiting for anyone
+    if (!kSmem && lr == 0 && me == 0) continue;
     double* const a = row(lr);
     for (int j = lane; j < n; j += 32) a[j] *= inv;
   }
