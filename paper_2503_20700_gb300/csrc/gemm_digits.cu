@@ -117,8 +117,8 @@ __device__ __forceinline__ bool test_wait(uint64_t* bar, uint32_t parity) {
 // another role of the CTA gave up.  Every wait is on this CTA's own work.
 __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatile int* abort,
                                          unsigned long long wait_ns) {
-  if (test_wait(bar, parity)) return true;
-  if (wait_ns == 0) return false;
+  if (wait_ns == 0) return test_wait(bar, parity);
+  if (try_wait(bar, parity)) return true;  // before the clock is read, which takes longer than most waits
   const unsigned long long t0 = global_ns();
   for (;;) {
     if (try_wait(bar, parity)) return true;
