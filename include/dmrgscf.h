@@ -567,7 +567,8 @@ dmrg_status dmrg_hpsi_contract_noalloc(const double* dA, int64_t a_len, const do
  * dmrg_eigh_batched -- symmetric eigendecompositions in float64 on the device
  * (the sector density matrices of the decimation step, Sec. II.C).  mats holds
  * the row-major matrices back to back (sizes n[i]); w receives eigenvalues in
- * descending order and vecs the eigenvectors as rows (same packing as mats).
+ * descending order and vecs the eigenvectors as rows (same packing as mats;
+ * vecs may be mats).
  * Largest-magnitude component of every eigenvector is made positive.
  */
 dmrg_status dmrg_eigh_batched(const double* mats, const int* n, int count, double* w, double* vecs,

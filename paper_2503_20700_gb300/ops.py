@@ -167,7 +167,7 @@ def eigh_batched(mats, device=0):
     flat = np.concatenate([m.ravel() if type(m) is np.ndarray and m.dtype == np.float64 else
                            np.ascontiguousarray(m, dtype=np.float64).ravel() for m in mats])
     w = np.empty(int(ns.sum()))
-    v = np.empty_like(flat)
+    v = flat  # the call has read it by the time it writes
     st = lib.dmrg_eigh_batched(_dp(flat), ns.ctypes.data_as(ctypes.POINTER(ctypes.c_int)),
                                len(mats), _dp(w), _dp(v), device)
     if st != 0:
