@@ -787,14 +787,15 @@ class CudaBackend : public Backend {
     for (size_t t = 0; t < tasks.size(); ++t) tasks[t] = p.tasks[order[t]];
     auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
     const size_t ox = al(p.pool_bytes()), ok = ox + al(p.nexp * sizeof(int));
-    const size_t osp = ok + al(p.nkmax * sizeof(uint2)), osc = osp + al(p.ops.size() * sizeof(int));
+    const size_t osp = ok + al(p.nkmax * sizeof(uint2)), ofl = osp + al((p.ops.size() + 1) * sizeof(int));
+    const size_t omi = ofl + al(p.marks), osc = omi + al((size_t)p.marks * 32 * sizeof(uint32_t));
     // Work space of a launch sequence: small ones share a block that the backend
     // keeps (stream order separates them; not under a budget, which it would
     // take from), larger ones come and go.  The part that starts at zero is
     // uploaded with the lists while it is small.
     char* ws = nullptr;
     size_t bytes = osc + (size_t)p.scratch * sizeof(double);
-    const size_t nzero = osc - ok;
+    const size_t nzero = ofl - ok;
     const bool keep = !budget_ && bytes <= kDigKept;
     if (!keep) {
       ws = (char*)try_alloc(bytes);
@@ -841,12 +842,14 @@ class CudaBackend : public Backend {
     L.exps = (int*)(ws + ox);
     L.kmax = (uint2*)(inline_zero ? d + off[5] : ws + ok);
     L.special = (int*)(inline_zero ? d + off[5] + (osp - ok) : ws + osp);
+    L.flag = (unsigned char*)(ws + ofl);
+    L.miss = (uint32_t*)(ws + omi);
     L.scratch = (double*)(ws + osc);
     L.err = dig_err;
     L.wait_ns = wait_ns_;
     L.sms = sms;
     dig_launch(L, st);
-    launches += 2 + (L.nreds > 0);
+    launches += 3 + (L.nreds > 0);
     if (!keep) free(ws);
     return true;
   }

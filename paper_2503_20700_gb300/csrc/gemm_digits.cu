@@ -274,7 +274,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     gemm_digits_kernel(const DigOperand* __restrict__ ops, const DigSeg* __restrict__ segs,
                        const DigTask* __restrict__ tasks, int ntasks, const unsigned char* __restrict__ pool,
                        const int* __restrict__ exps, const uint2* __restrict__ kmax,
-                       const int* __restrict__ special, double* __restrict__ scratch, int* __restrict__ err,
+                       int* __restrict__ special, int nops, unsigned char* __restrict__ flag,
+                       uint32_t* __restrict__ miss, double* __restrict__ scratch, int* __restrict__ err,
                        unsigned long long wait_ns) {
   extern __shared__ unsigned char smraw[];
   __shared__ __align__(8) uint64_t bar[B_COUNT];
@@ -534,16 +535,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           ++nd;
         }
         if (!ok) break;
-        if (m.plain) {
-          // float64 FMAs on the operands themselves
-          const DigOperand &a = ops[m.a], &b = ops[m.b];
-          if (nrow > 0)
-            for (int kk = 0; kk < m.k; ++kk) {
-              const double y = elem(b, gc, kk);
-#pragma unroll
-              for (int r = 0; r < 32; ++r)
-                if (r < nrow) acc[r] = fma(m.alpha * elem(a, gr0 + r, kk), y, acc[r]);
-            }
+        const int mark = m.t.mark + 8 * k + warp - 4;
+        const bool left = busy && m.plain;  // to fma_missing_kernel
+        if (lane == 0) {
+          flag[mark] = left;
+          if (left) special[nops] = 1;
+        }
+        if (left) {
+          miss[(size_t)mark * 32 + lane] = 0xFFFFFFFFu;
           arrive(&bar[B_ME + (q & 1)]);
           continue;
         }
@@ -604,6 +603,100 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
 }
 
+// What gemm_digits_kernel left out: per mark, the missing outputs of a 32 x 32
+// block are dealt to the threads one by one, four each, and their products
+// added to the tile by float64 FMAs.  Bound by the float64 pipe (two FMAs a
+// clock and SM) where whole blocks are missing: two shared-memory reads an FMA,
+// one along the lanes and one broadcast, are a fifth of its time, and blocks of
+// 32 x 32 spread even a single product over the SMs.  Measured, whole calls with
+// every operand graded: 400 x 400 x 400 2.19 -> 0.42 ms, 601 of 200 x 200 x 200
+// 39.6 -> 19.2 ms (one in ten graded: 9.5 -> 7.0) against FMAs on unstaged
+// operands in the epilogue of the digit kernel; gemm_f64_kernel alone takes 0.96
+// and 18.4 ms.  Without marks the launch costs 1.3 us and 2 us of the host.
+constexpr int FIX_THREADS = 256, FIX_K = 64, FIX_LD = FIX_K + 1, FIX_OUT = 1024 / FIX_THREADS, FIX_CTAS = 5;
+__global__ void __launch_bounds__(FIX_THREADS, FIX_CTAS)
+    fma_missing_kernel(const DigOperand* __restrict__ ops, const DigSeg* __restrict__ segs,
+                       const DigTask* __restrict__ tasks, int ntasks, const int* __restrict__ any,
+                       const unsigned char* __restrict__ flag, const uint32_t* __restrict__ miss,
+                       double* __restrict__ scratch) {
+  if (*any == 0) return;
+  __shared__ double As[32 * FIX_LD], Bs[32 * FIX_LD];
+  __shared__ unsigned short list[1024];
+  __shared__ int count;
+  const int tid = threadIdx.x;
+  for (int u = blockIdx.x; u < ntasks * 8; u += gridDim.x) {
+    const int w = u / ntasks;  // every CTA meets all eight: the last ones of a ragged tile are empty
+    const DigTask t = tasks[u - w * ntasks];
+    const int r0 = t.r0 + (w & 3) * 32, c0 = t.c0 + (w >> 2) * 32;
+    const int nr = min(32, t.m - r0), nc = min(32, t.n - c0);
+    if (nr <= 0 || nc <= 0) continue;
+    for (int s = 0; s < t.seg_count; ++s) {
+      const int mark = t.mark + 8 * s + w;
+      if (!flag[mark]) continue;
+      __syncthreads();  // the list and the tiles are free, the block's outputs visible
+      if (tid < 32) {
+        uint32_t bits = tid < nr ? miss[(size_t)mark * 32 + tid] & (0xFFFFFFFFu >> (32 - nc)) : 0u;
+        int at = __popc(bits);
+#pragma unroll
+        for (int d = 1; d < 32; d *= 2) {
+          const int x = __shfl_up_sync(0xffffffffu, at, d);
+          if (tid >= d) at += x;
+        }
+        if (tid == 31) count = at;
+        at -= __popc(bits);
+        for (; bits; bits &= bits - 1) list[at++] = (unsigned short)(tid * 32 + __ffs(bits) - 1);
+      }
+      __syncthreads();
+      const int n = count;
+      const DigSeg sg = segs[t.seg_begin + s];
+      const DigOperand a = ops[sg.a], b = ops[sg.b];
+      double acc[FIX_OUT];
+      int ao[FIX_OUT], bo[FIX_OUT];
+#pragma unroll
+      for (int q = 0; q < FIX_OUT; ++q) {
+        const int i = tid + q * FIX_THREADS, e = i < n ? list[i] : 0;
+        acc[q] = 0.0;
+        ao[q] = (e >> 5) * FIX_LD;
+        bo[q] = (e & 31) * FIX_LD;
+      }
+      const int nq = (n - tid + FIX_THREADS - 1) / FIX_THREADS;  // of this thread
+      for (int k0 = 0; k0 < a.k; k0 += FIX_K) {
+        const int kn = min(FIX_K, a.k - k0);
+        for (int e = tid; e < 32 * FIX_K; e += FIX_THREADS) {
+          const int r = a.trans ? e & 31 : e / FIX_K, k = a.trans ? e >> 5 : e % FIX_K;
+          if (r < nr && k < kn) As[r * FIX_LD + k] = sg.alpha * elem(a, r0 + r, k0 + k);
+        }
+        for (int e = tid; e < 32 * FIX_K; e += FIX_THREADS) {
+          const int c = b.trans ? e & 31 : e / FIX_K, k = b.trans ? e >> 5 : e % FIX_K;
+          if (c < nc && k < kn) Bs[c * FIX_LD + k] = elem(b, c0 + c, k0 + k);
+        }
+        __syncthreads();
+        if (nq == FIX_OUT) {
+#pragma unroll 4
+          for (int k = 0; k < kn; ++k)
+#pragma unroll
+            for (int q = 0; q < FIX_OUT; ++q) acc[q] = fma(As[ao[q] + k], Bs[bo[q] + k], acc[q]);
+        } else {
+#pragma unroll
+          for (int q = 0; q < FIX_OUT - 1; ++q)
+            if (q < nq)
+              for (int k = 0; k < kn; ++k) acc[q] = fma(As[ao[q] + k], Bs[bo[q] + k], acc[q]);
+        }
+        __syncthreads();
+      }
+#pragma unroll
+      for (int q = 0; q < FIX_OUT; ++q) {
+        if (q >= nq) break;
+        const int e = list[tid + q * FIX_THREADS], r = e >> 5, c = e & 31;
+        double* const out = t.part >= 0
+                                ? scratch + t.part + (size_t)(r0 - t.r0 + r) * kDigTileN + (c0 - t.c0) + c
+                                : t.C + (size_t)(r0 + r) * t.ldc + c0 + c;
+        *out += acc[q];
+      }
+    }
+  }
+}
+
 // C += the partial tiles of one output tile, in order; a CTA sums 4 rows
 __global__ void __launch_bounds__(256) reduce_digits_kernel(const DigReduce* __restrict__ reds,
                                                             const double* __restrict__ scratch) {
@@ -627,9 +720,14 @@ void dig_launch(const DigLaunch& L, cudaStream_t st) {
   e = cudaGetLastError();
   if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: digit split: ") + cudaGetErrorString(e));
   gemm_digits_kernel<<<std::min(L.sms, L.ntasks), NTHREADS, SMEM_BYTES, st>>>(
-      L.ops, L.segs, L.tasks, L.ntasks, L.pool, L.exps, L.kmax, L.special, L.scratch, L.err, L.wait_ns);
+      L.ops, L.segs, L.tasks, L.ntasks, L.pool, L.exps, L.kmax, L.special, L.nops, L.flag, L.miss, L.scratch, L.err,
+      L.wait_ns);
   e = cudaGetLastError();
   if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: digit gemm: ") + cudaGetErrorString(e));
+  fma_missing_kernel<<<std::min(L.sms * FIX_CTAS, L.ntasks * 8), FIX_THREADS, 0, st>>>(
+      L.ops, L.segs, L.tasks, L.ntasks, L.special + L.nops, L.flag, L.miss, L.scratch);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: digit remainder: ") + cudaGetErrorString(e));
   if (L.nreds > 0) {
     reduce_digits_kernel<<<dim3(L.nreds, kDigTileM / 4), 256, 0, st>>>(L.reds, L.scratch);
     e = cudaGetLastError();

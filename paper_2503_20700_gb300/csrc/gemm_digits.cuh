@@ -16,7 +16,8 @@
 // in integers, and each segment is added to the output tile in float64.
 //
 // Operands whose scaling makes that bound useless are not multiplied by
-// digits but by float64 FMAs in the same kernel: a segment with a non-finite
+// digits: their products are left out and marked, and a second kernel adds them
+// by float64 FMAs (fma_missing_kernel).  These are a segment with a non-finite
 // entry, with a row maximum outside 2^+-400, or graded along k, that is, whose
 // largest product |a_ik b_kj| is more than 2^8 below the product of the
 // largest entries of A and B, or is so after every row is divided by its
@@ -66,7 +67,8 @@ struct DigTask {
   double* C;
   long long part;
   int m, n, ldc, r0, c0;
-  int seg_begin, seg_count, pad;
+  int seg_begin, seg_count;
+  int mark;  // first of its marks (DigLaunch::flag): 8 a segment
 };
 
 struct DigReduce {
@@ -85,6 +87,7 @@ struct DigPlan {
   long long units = 0;    // of the digit pool
   long long scratch = 0;  // doubles of partial tiles
   int nexp = 0, nkmax = 0;
+  int marks = 0;
   size_t pool_bytes() const { return (size_t)units * kDigUnit; }
 };
 
@@ -140,7 +143,12 @@ struct DigLaunch {
   int* exps;           // nexp
   uint2* kmax;         // nkmax, zero at launch; exponents of the columns' largest entries,
                        // of the rows divided by their maxima (x) and as they are (y); 0: a zero column
-  int* special;        // nops, zero at launch
+  int* special;        // nops, and one for all marks (any), zero at launch
+  // A mark stands for a segment on a 32 x 32 block of a task's tile (row quarter
+  // + 4 column half): flag 1 when products of it are left out, then bit c of
+  // miss[32 mark + r] says that the product of row r and column c is.
+  unsigned char* flag;
+  uint32_t* miss;
   int* err;            // host-mapped flag, set when a bounded wait ran out
   unsigned long long wait_ns;  // bound of every wait (0: its first probe)
   int sms;

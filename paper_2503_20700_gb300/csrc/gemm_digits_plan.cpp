@@ -88,8 +88,10 @@ void DigPlanner::add(const GemmGroup& g, const GemmSeg* segs, int parts) {
       if (parts > 1) plan.reds.push_back({g.C, plan.scratch, g.m, g.n, g.ldc, r, c, parts});
       for (int p = 0; p < parts; ++p) {
         const int b = p * per;
-        plan.tasks.push_back({g.C, parts > 1 ? plan.scratch : -1, g.m, g.n, g.ldc, r, c, first + b,
-                              std::min(per, cnt - b), 0});
+        const int segs_here = std::min(per, cnt - b);
+        plan.tasks.push_back({g.C, parts > 1 ? plan.scratch : -1, g.m, g.n, g.ldc, r, c, first + b, segs_here,
+                              plan.marks});
+        plan.marks += 8 * segs_here;
         if (parts > 1) plan.scratch += (long long)kDigTileM * kDigTileN;
       }
     }
