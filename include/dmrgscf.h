@@ -478,6 +478,10 @@ typedef struct {
  * group), by renormalisation and by the complementary-operator contractions.
  * C (c_len doubles) is read and updated in place; A and B are read only.
  * Output blocks must not overlap.  precision: DMRG_FP64 or DMRG_SPLIT_TF32.
+ * DMRG_FP64: every output is within 2 k 2^-53 sum |alpha a b| of the exact sum
+ * per segment, whatever the scales of its rows (products on bf16 digits where
+ * they are at least as accurate as a float64 multiply-add chain, such a chain
+ * elsewhere), rounded when it is added to C.
  * Returns DMRG_EINVAL for out-of-range offsets, DMRG_ECUDA without a device.
  */
 dmrg_status dmrg_grouped_gemm(const double* A, int64_t a_len, const double* B, int64_t b_len,

@@ -650,8 +650,9 @@ class CudaBackend : public Backend {
     gemm_impl(groups, segs, prec, nullptr);
   }
 
+  // by_entry = false: products of orthogonal matrices (gemm_digits.cuh)
   void gemm_impl(const std::vector<GemmGroup>& groups, const std::vector<GemmSeg>& segs,
-                 Precision prec, Rec* rec) {
+                 Precision prec, Rec* rec, bool by_entry = true) {
     if (prec != Precision::FP64) {
       gemm_split_launch(groups, segs, prec, st,
                         [&](const std::vector<std::pair<const void*, size_t>>& parts,
@@ -668,7 +669,7 @@ class CudaBackend : public Backend {
     const bool any = choose_digits(groups, segs, digits);
     if (any) {
       if (rec) CK(cudaEventRecord(rec->a, st));
-      gemm_digits(groups, segs, digits);
+      gemm_digits(groups, segs, digits, by_entry);
     }
     std::vector<GemmTile> tiles;
     for (size_t gi = 0; gi < groups.size(); ++gi) {
@@ -738,7 +739,7 @@ class CudaBackend : public Backend {
   }
   // clears digits[i] of the groups left to the FMA kernel
   void gemm_digits(const std::vector<GemmGroup>& groups, const std::vector<GemmSeg>& segs,
-                   std::vector<char>& digits) {
+                   std::vector<char>& digits, bool by_entry) {
     if (!dig_err) {
       dig_err = (int*)PinnedPool::get().take(sizeof(int), &dig_err_cap);
       *dig_err = 0;
@@ -748,12 +749,12 @@ class CudaBackend : public Backend {
     std::vector<size_t> planned;
     auto add = [&](size_t i) { pl.add(groups[i], segs.data(), dig_parts(groups[i], segs.data())); };
     auto run = [&]() {
-      if (!run_digits(pl.plan)) {
+      if (!run_digits(pl.plan, by_entry)) {
         // no room: its groups one by one
         for (size_t i : planned) {
           pl.clear();
           add(i);
-          if (planned.size() == 1 || !run_digits(pl.plan)) digits[i] = 0;
+          if (planned.size() == 1 || !run_digits(pl.plan, by_entry)) digits[i] = 0;
         }
       }
       pl.clear();
@@ -772,7 +773,7 @@ class CudaBackend : public Backend {
   size_t dig_ws_cap = 0;
   std::vector<char> dig_zero;
   // false when there is no room for the work space
-  bool run_digits(DigPlan& p) {
+  bool run_digits(DigPlan& p, bool by_entry) {
     if (p.tasks.empty()) return true;
     // longest tasks first, dealt round-robin over the persistent CTAs
     std::vector<double> w(p.tasks.size());
@@ -787,15 +788,17 @@ class CudaBackend : public Backend {
     for (size_t t = 0; t < tasks.size(); ++t) tasks[t] = p.tasks[order[t]];
     auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
     const size_t ox = al(p.pool_bytes()), ok = ox + al(p.nexp * sizeof(int));
-    const size_t osp = ok + al(p.nkmax * sizeof(uint2)), ofl = osp + al((p.ops.size() + 1) * sizeof(int));
-    const size_t omi = ofl + al(p.marks), osc = omi + al((size_t)p.marks * 32 * sizeof(uint32_t));
+    const size_t onz = ok + al((p.units + 32) * sizeof(DigMask)), osp = onz + al((p.units + 32) * sizeof(uint16_t));
+    const size_t ofl = osp + al((p.ops.size() + 1) * sizeof(int));
+    const size_t omi = ofl + al(p.marks), olb = omi + al((size_t)p.marks * 32 * sizeof(uint32_t));
+    const size_t osc = olb + al(p.tasks.size() * 8 * sizeof(int));
     // Work space of a launch sequence: small ones share a block that the backend
     // keeps (stream order separates them; not under a budget, which it would
     // take from), larger ones come and go.  The part that starts at zero is
     // uploaded with the lists while it is small.
     char* ws = nullptr;
     size_t bytes = osc + (size_t)p.scratch * sizeof(double);
-    const size_t nzero = ofl - ok;
+    const size_t nzero = ofl - osp;
     const bool keep = !budget_ && bytes <= kDigKept;
     if (!keep) {
       ws = (char*)try_alloc(bytes);
@@ -819,7 +822,7 @@ class CudaBackend : public Backend {
     }
     const bool inline_zero = nzero <= size_t(32) << 10;
     if (inline_zero) dig_zero.resize(std::max(dig_zero.size(), nzero), 0);
-    else CK(cudaMemsetAsync(ws + ok, 0, nzero, st));
+    else CK(cudaMemsetAsync(ws + osp, 0, nzero, st));
     std::vector<size_t> off;
     char* d = upload({{p.ops.data(), p.ops.size() * sizeof(DigOperand)},
                       {p.splits.data(), p.splits.size() * sizeof(DigSplit)},
@@ -840,10 +843,13 @@ class CudaBackend : public Backend {
     L.nops = (int)p.ops.size();
     L.pool = (unsigned char*)ws;
     L.exps = (int*)(ws + ox);
-    L.kmax = (uint2*)(inline_zero ? d + off[5] : ws + ok);
-    L.special = (int*)(inline_zero ? d + off[5] + (osp - ok) : ws + osp);
+    L.masks = (DigMask*)(ws + ok);
+    L.nonzero = (uint16_t*)(ws + onz);
+    L.by_entry = by_entry;
+    L.special = (int*)(inline_zero ? d + off[5] : ws + osp);
     L.flag = (unsigned char*)(ws + ofl);
     L.miss = (uint32_t*)(ws + omi);
+    L.left = (int*)(ws + olb);
     L.scratch = (double*)(ws + osc);
     L.err = dig_err;
     L.wait_ns = wait_ns_;
@@ -1173,7 +1179,7 @@ class CudaBackend : public Backend {
       }
       dc_merge_launch(dm, dn + first[l], (int)level.size(), positions, largest, (int)l, ar, st);
       CK(cudaMemsetAsync(mats[0].B[(l + 1) & 1], 0, prefix * sizeof(double), st));
-      gemm_impl(groups, segs, Precision::FP64, nullptr);
+      gemm_impl(groups, segs, Precision::FP64, nullptr, false);
       launches += 6;
     }
     dc_back_launch(dm, (int)mats.size(), (int)sum, sizes[0], ar, st);

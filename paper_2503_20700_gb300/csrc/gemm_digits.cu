@@ -15,8 +15,10 @@
 // because eight accumulators of that size are all of TMEM; N = 64 alone would
 // read shared memory at 48 clocks per 32-clock MMA, which the stacked form
 // avoids.  Measured, 601 products of 200 x 200 x 200 (the rotation of 600
-// Cholesky vectors): 0.43 ms and 0.17 ms for the split, 16 TFLOP/s of float64;
-// the FMA kernel needs 13 ms (0.74 TFLOP/s, 1.25 nominal peak).
+// Cholesky vectors): 0.46 ms (0.52 ms where the right operand decays away from
+// its diagonal and its outputs take longer to test) and 0.16 ms for the split,
+// 15 TFLOP/s of float64; the FMA kernel needs 13 ms (0.74 TFLOP/s, 1.25 nominal
+// peak).
 #include <algorithm>
 #include <stdexcept>
 #include <string>
@@ -41,18 +43,19 @@ constexpr int CHUNK = 16;  // k-steps of 16 between drains: 256 exact terms
 constexpr int NTHREADS = 384;
 constexpr unsigned long long kDrainNs = 2000000000ull;  // what a CTA that gave up waits for its own work in flight
 constexpr int kExpRange = 400;
-constexpr int kGraded = 8;  // the largest product may lie 2^8 below the product of the maxima
 
 enum { B_FULL = 0, B_EMPTY = B_FULL + NSTAGE, B_SF = B_EMPTY + NSTAGE, B_SE, B_MF, B_ME = B_MF + 2,
        B_DONE = B_ME + 2, B_COUNT };
 
 // what the epilogue needs of a segment, gathered one segment ahead by a warp
-// of its own (the dependent loads task - segment - operand - column maxima
-// took a third of the epilogue's time)
+// of its own (the dependent loads task - segment - operand took a third of the
+// epilogue's time)
 struct Meta {
   DigTask t;
   double alpha;
-  int a, b, k, plain;
+  long long ua, ub;  // masks of the operands
+  int sa, sb;        // their rows per 16 columns
+  int k, plain;
   int ea[kDigTileM], eb[kDigTileN];  // row and column exponents
 };
 
@@ -158,7 +161,7 @@ __device__ __forceinline__ float digit_float(uint32_t word, int byte) {
 
 // 32 rows of one operand per CTA: row maxima, then the digits.  Bound by the
 // latency of its loads for the matrices of a sweep and by HBM and the integer
-// pipe together for large ones (8 B read twice, 16 B written, about 35
+// pipe together for large ones (8 B read twice, 16 B written, some forty
 // integer operations per element), so a thread loads the eight columns of its
 // row before it uses the first.  Its eight 16-byte stores, one per digit, fill
 // 512 contiguous bytes each with those of its warp.
@@ -172,7 +175,8 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_digits_kernel(const DigOp
                                                                      const DigSplit* __restrict__ splits,
                                                                      unsigned char* __restrict__ pool,
                                                                      int* __restrict__ exps,
-                                                                     uint2* __restrict__ kmax,
+                                                                     DigMask* __restrict__ masks,
+                                                                     uint16_t* __restrict__ nonzero,
                                                                      int* __restrict__ special) {
   __shared__ unsigned rowmax[32];
   constexpr int KSTEP = SPLIT_THREADS / 64;  // k-blocks of 16 in flight
@@ -214,7 +218,8 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_digits_kernel(const DigOp
     double x[8];
     load8(o, r, c0, x);
     uint32_t w[kDigSlices][4];
-    unsigned rel = 0u, top = 0u;  // column c0 + (lane & 7), once the loop is done
+    DigMask mk = make_uint2(0u, 0u);
+    unsigned nz = 0u;
 #pragma unroll
     for (int i = 0; i < 8; i += 2) {
       float f[2][kDigSlices];
@@ -235,18 +240,12 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_digits_kernel(const DigOp
           f[q][s] = digit_float(uh, 3 - s);
           f[q][4 + s] = digit_float(ul, 3 - s);
         }
-        // largest entry of the column over the eight rows: relative to its
-        // row's maximum (shifted by 4096, so that 0 is a zero) and absolute
-        unsigned a = be ? (unsigned)(4096 + be - be_row) : 0u, b = (unsigned)be;
-#pragma unroll
-        for (int d = 1; d < 8; d *= 2) {
-          a = max(a, __shfl_xor_sync(0xffffffffu, a, d));
-          b = max(b, __shfl_xor_sync(0xffffffffu, b, d));
-        }
-        if ((lane & 7) == i + q) {
-          rel = a;
-          top = b;
-        }
+        const int down = be_row - be;
+        mk.x |= be && down <= 2 ? 1u << (i + q) : 0u;
+        mk.x |= be && down <= 3 ? 0x10000u << (i + q) : 0u;
+        mk.y |= be && down <= 1 ? 1u << (i + q) : 0u;
+        mk.y |= be && down <= 4 ? 0x10000u << (i + q) : 0u;
+        nz |= bits << 1 ? 1u << (i + q) : 0u;
       }
 #pragma unroll
       for (int s = 0; s < kDigSlices; ++s)
@@ -258,24 +257,89 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_digits_kernel(const DigOp
         *reinterpret_cast<uint4*>(base + ((size_t)kb * kDigSlices + s) * o.groups * kDigUnit) =
             make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
     }
-    // the two row groups of the warp, then all rows of the operand
-    rel = max(rel, __shfl_xor_sync(0xffffffffu, rel, 16));
-    top = max(top, __shfl_xor_sync(0xffffffffu, top, 16));
-    const int c = c0 + (lane & 7);
-    if (lane < 16 && c < o.k && rel) {
-      atomicMax(&kmax[o.koff + c].x, rel);
-      atomicMax(&kmax[o.koff + c].y, top);
+    // the two halves of the 16 columns
+    mk.x <<= 8 * kc;
+    mk.y <<= 8 * kc;
+    mk.x |= __shfl_xor_sync(0xffffffffu, mk.x, 8);
+    mk.y |= __shfl_xor_sync(0xffffffffu, mk.y, 8);
+    nz <<= 8 * kc;
+    nz |= __shfl_xor_sync(0xffffffffu, nz, 8);
+    if (stored && kc == 0) {
+      const size_t at = (size_t)o.unit + (size_t)kb * 8 * o.groups + r;
+      masks[at] = mk;
+      nonzero[at] = (uint16_t)nz;
     }
   }
 }
 
 // ---------------------------------------------------------------- products
+// Bit c: the output of this lane's row and column c (of `ncol`) is to be left
+// out: no term of it is known to reach 2^-7 of 2^ea 2^eb, and not all are zero.
+// ma, na: this lane's row (has_row: there is one), mb, nb: column 0, at k-block 0.
+// Two k-blocks at a time, for the latency of their loads; they settle a dense
+// operand, and 400 integer operations of a warp stand beside 3000 clocks of the
+// products of two k-blocks.
+__device__ __forceinline__ uint32_t outputs_left(bool has_row, const DigMask* ma, const uint16_t* na, int sa,
+                                                 const DigMask* mb, const uint16_t* nb, int sb, int nkb, int ncol) {
+  uint32_t open = has_row ? 0xFFFFFFFFu >> (32 - ncol) : 0u;  // not settled yet
+  for (int kb = 0; kb < nkb; kb += 2) {
+    const int k1 = min(kb + 1, nkb - 1);
+    const uint2 z = make_uint2(0u, 0u);
+    const uint2 a0 = has_row ? __ldg(ma + (size_t)kb * sa) : z, a1 = has_row ? __ldg(ma + (size_t)k1 * sa) : z;
+    const uint4* p0 = reinterpret_cast<const uint4*>(mb + (size_t)kb * sb);
+    const uint4* p1 = reinterpret_cast<const uint4*>(mb + (size_t)k1 * sb);
+    auto swapped = [](uint32_t x) { return __byte_perm(x, 0u, 0x1032); };
+#pragma unroll
+    for (int c = 0; c < 32; c += 16) {
+      uint4 b0[8], b1[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        b0[i] = __ldg(p0 + c / 2 + i);
+        b1[i] = __ldg(p1 + c / 2 + i);
+      }
+      uint32_t hit = 0u;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        if ((a0.x & swapped(b0[i].x)) | (a0.y & swapped(b0[i].y)) | (a1.x & swapped(b1[i].x)) |
+            (a1.y & swapped(b1[i].y)))
+          hit |= 1u << (2 * i);
+        if ((a0.x & swapped(b0[i].z)) | (a0.y & swapped(b0[i].w)) | (a1.x & swapped(b1[i].z)) |
+            (a1.y & swapped(b1[i].w)))
+          hit |= 2u << (2 * i);
+      }
+      open &= ~(hit << c);
+    }
+    if (__all_sync(0xffffffffu, open == 0u)) return 0u;
+  }
+  uint32_t zero = open;  // open ones with no term found so far
+  for (int kb = 0; kb < nkb; ++kb) {
+    const uint32_t a = has_row ? __ldg(na + (size_t)kb * sa) * 0x10001u : 0u;
+    const uint4* p = reinterpret_cast<const uint4*>(nb + (size_t)kb * sb);
+    uint32_t hit = 0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint4 b = __ldg(p + i);
+      const uint32_t w[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (a & w[j] & 0xFFFFu) hit |= 1u << (8 * i + 2 * j);
+        if (a & w[j] & 0xFFFF0000u) hit |= 2u << (8 * i + 2 * j);
+      }
+    }
+    zero &= ~hit;
+    if (__all_sync(0xffffffffu, zero == 0u)) break;
+  }
+  return open & ~zero;
+}
+
 __global__ void __launch_bounds__(NTHREADS, 1)
     gemm_digits_kernel(const DigOperand* __restrict__ ops, const DigSeg* __restrict__ segs,
                        const DigTask* __restrict__ tasks, int ntasks, const unsigned char* __restrict__ pool,
-                       const int* __restrict__ exps, const uint2* __restrict__ kmax,
+                       const int* __restrict__ exps, const DigMask* __restrict__ masks,
+                       const uint16_t* __restrict__ nonzero, int by_entry,
                        int* __restrict__ special, int nops, unsigned char* __restrict__ flag,
-                       uint32_t* __restrict__ miss, double* __restrict__ scratch, int* __restrict__ err,
+                       uint32_t* __restrict__ miss, int* __restrict__ left_blocks, double* __restrict__ scratch,
+                       int* __restrict__ err,
                        unsigned long long wait_ns) {
   extern __shared__ unsigned char smraw[];
   __shared__ __align__(8) uint64_t bar[B_COUNT];
@@ -419,26 +483,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           const DigSeg sg = segs[k];
           const DigOperand &a = ops[sg.a], &b = ops[sg.b];
           const int K = a.k;
-          // may the digits be used: the largest products of the segment against
-          // the products of the maxima (no overlapping column: an exact zero)
-          unsigned rel = 0u, top = 0u, amax = 0u, bmax = 0u;
-          const uint2 *ka = kmax + a.koff, *kb = kmax + b.koff;
-#pragma unroll 4
-          for (int c = lane; c < K; c += 32) {
-            const uint2 x = __ldg(ka + c), y = __ldg(kb + c);
-            if (x.x && y.x) {
-              rel = max(rel, x.x + y.x);
-              top = max(top, x.y + y.y);
-            }
-            amax = max(amax, x.y);
-            bmax = max(bmax, y.y);
-          }
-          rel = __reduce_max_sync(0xffffffffu, rel);
-          top = __reduce_max_sync(0xffffffffu, top);
-          amax = __reduce_max_sync(0xffffffffu, amax);
-          bmax = __reduce_max_sync(0xffffffffu, bmax);
-          const int plain = (special[sg.a] | special[sg.b]) ||
-                            (rel && (rel + kGraded < 8192u || top + kGraded < amax + bmax));
+          const int plain = special[sg.a] | special[sg.b];
           ok = __all_sync(0xffffffffu, wait_bar(&bar[B_ME + (q & 1)], (uint32_t)(((q >> 1) & 1) ^ 1), abort, wait_ns));
           if (!ok) break;
           Meta& m = meta[q & 1];
@@ -448,8 +493,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           if (lane == 0) {
             m.t = tasks[t];
             m.alpha = sg.alpha;
-            m.a = sg.a;
-            m.b = sg.b;
+            m.ua = a.unit;
+            m.ub = b.unit;
+            m.sa = 8 * a.groups;
+            m.sb = 8 * b.groups;
             m.k = K;
             m.plain = plain;
           }
@@ -474,6 +521,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       long long part = -1;
       int W = 0, ldc = 0, nrow = 0, gc = 0, gr0 = 0, sc = 1;
       bool busy = false;  // the warp has outputs of the block
+      bool marked = false;
       for (int k = 0; ok && k < sc; ++k, ++q) {
         ok = __all_sync(0xffffffffu, wait_bar(&bar[B_MF + (q & 1)], (uint32_t)((q >> 1) & 1), abort, wait_ns));
         if (!ok) break;
@@ -495,6 +543,20 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           for (int r = 0; r < 32; ++r) acc[r] = (part < 0 && r < nrow) ? out[(size_t)r * ldc] : 0.0;
         }
         const int nkb = (m.k + 15) >> 4;
+        // outputs left to fma_missing_kernel: bit c of a lane's row
+        uint32_t left = 0u;
+        if (busy && m.plain) {
+          left = 0xFFFFFFFFu;
+        } else if (busy && by_entry) {
+          const int r = gr0 + lane, c0 = m.t.c0 + half * NC;
+          left = outputs_left(r < m.t.m, masks + m.ua + r, nonzero + m.ua + r, m.sa, masks + m.ub + c0,
+                              nonzero + m.ub + c0, m.sb, nkb, min(NC, m.t.n - c0));
+        }
+        const int mark = m.t.mark + 8 * k + warp - 4;
+        const bool some = __any_sync(0xffffffffu, left != 0u);
+        if (some) miss[(size_t)mark * 32 + lane] = left;
+        if (lane == 0) flag[mark] = some;
+        marked = marked || some;
         // the combined accumulators of row gr0 + lane: h 2^32 + l, in units of
         // 2^(ea + eb)
         long long h[NC];
@@ -535,18 +597,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           ++nd;
         }
         if (!ok) break;
-        const int mark = m.t.mark + 8 * k + warp - 4;
-        const bool left = busy && m.plain;  // to fma_missing_kernel
-        if (lane == 0) {
-          flag[mark] = left;
-          if (left) special[nops] = 1;
-        }
-        if (left) {
-          miss[(size_t)mark * 32 + lane] = 0xFFFFFFFFu;
-          arrive(&bar[B_ME + (q & 1)]);
-          continue;
-        }
-        if (!busy) {
+        if (!busy || m.plain) {
           // nothing of the block in this warp's rows and columns: the float64
           // pipe belongs to the others (the 442 launches of a D = 256 sweep, whose
           // blocks are mostly below 128 x 64: 14.7 -> 11.8 ms)
@@ -559,6 +610,15 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           turn[lane * TURN_LD + c] = combined(h[c], l[c]);
         }
         __syncwarp();
+        // bit r: this lane's column of row r is an output of the digits
+        uint32_t live = nrow > 0 ? 0xFFFFFFFFu >> (32 - nrow) : 0u;
+        if (some) {
+#pragma unroll 4
+          for (int c = 0; c < 32; ++c) {
+            const uint32_t rows = __ballot_sync(0xffffffffu, left >> c & 1u);
+            if (lane == c) live &= ~rows;
+          }
+        }
         const double alpha = m.alpha;
         const int m_rows = m.t.m;
         const int eb = m.eb[half * NC + lane];
@@ -569,12 +629,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           const int e = eb + m.ea[(warp & 3) * 32 + r];
           const double d = turn[r * TURN_LD + lane];
           const int hi = __double2hiint(d);
-          if (r < nrow) acc[r] = fma(alpha, __hiloint2double(hi ? hi + (e << 20) : 0, __double2loint(d)), acc[r]);
+          if (live >> r & 1u) acc[r] = fma(alpha, __hiloint2double(hi ? hi + (e << 20) : 0, __double2loint(d)), acc[r]);
         }
         __syncwarp();
         arrive(&bar[B_ME + (q & 1)]);
       }
       if (!ok) break;
+      if (marked && lane == 0) left_blocks[atomicAdd(&special[nops], 1)] = 8 * t + warp - 4;
       if (part >= 0) {
         // row-major partial tile of 128 x 64
         double* p = scratch + part + (size_t)((warp & 3) * 32) * kDigTileN + half * NC + lane;
@@ -603,39 +664,67 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
 }
 
-// What gemm_digits_kernel left out: per mark, the missing outputs of a 32 x 32
-// block are dealt to the threads one by one, four each, and their products
-// added to the tile by float64 FMAs.  Bound by the float64 pipe (two FMAs a
-// clock and SM) where whole blocks are missing: two shared-memory reads an FMA,
-// one along the lanes and one broadcast, are a fifth of its time, and blocks of
-// 32 x 32 spread even a single product over the SMs.  Measured, whole calls with
-// every operand graded: 400 x 400 x 400 2.19 -> 0.42 ms, 601 of 200 x 200 x 200
-// 39.6 -> 19.2 ms (one in ten graded: 9.5 -> 7.0) against FMAs on unstaged
-// operands in the epilogue of the digit kernel; gemm_f64_kernel alone takes 0.96
-// and 18.4 ms.  Without marks the launch costs 1.3 us and 2 us of the host.
-constexpr int FIX_THREADS = 256, FIX_K = 64, FIX_LD = FIX_K + 1, FIX_OUT = 1024 / FIX_THREADS, FIX_CTAS = 5;
+// What gemm_digits_kernel left out, added to the tiles by float64 FMAs.  A CTA
+// takes 16 x 32 outputs of a block with marks and its marked segments in order; the missing
+// outputs are dealt to the threads one by one, two each, or a few threads each
+// (along k) where there are few.  Bound by the float64 pipe (two FMAs a clock
+// and SM) where whole blocks are missing: two shared-memory reads an FMA, one
+// along the lanes and one broadcast, are a fifth of its time.  Where single
+// outputs are missing, by the latency of the loads, so two steps of 64 columns
+// are in flight; and blocks this small, taken from a list, spread what is missing
+// in a corner of a matrix over the SMs (exchange of 200 orbitals: 970 us with
+// blocks dealt by their place, 435 from the list).  Measured, whole calls with
+// every operand graded: 400 x 400 x 400 0.34 ms, 601 of 200 x 200 x 200 14.3 ms
+// (0.95 and 18.4 ms by gemm_f64_kernel alone).  Without marks 1.3 us.
+constexpr int FIX_THREADS = 256, FIX_ROWS = 16, FIX_COLS = 32, FIX_K = 64, FIX_LD = FIX_K + 1;
+constexpr int FIX_CTAS = 4;
+constexpr int FIX_OUT = FIX_ROWS * FIX_COLS / FIX_THREADS;
+constexpr int FIX_STAGE = (FIX_ROWS + FIX_COLS) * FIX_LD, FIX_SMEM = 2 * FIX_STAGE * (int)sizeof(double);
+
+__device__ __forceinline__ void copy8(double* dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+// rows [r0, r0 + nr) and columns [k0, k0 + kn) of an operand, row r at r FIX_LD
+template <int ROWS>
+__device__ __forceinline__ void fix_stage(double* dst, const DigOperand& o, int r0, int nr, int k0, int kn) {
+  for (int e = threadIdx.x; e < ROWS * FIX_K; e += FIX_THREADS) {
+    const int r = o.trans ? e % ROWS : e / FIX_K, k = o.trans ? e / ROWS : e % FIX_K;
+    if (r < nr && k < kn)
+      copy8(dst + r * FIX_LD + k,
+            o.src + (o.trans ? (size_t)(k0 + k) * o.ld + r0 + r : (size_t)(r0 + r) * o.ld + k0 + k));
+  }
+}
+
 __global__ void __launch_bounds__(FIX_THREADS, FIX_CTAS)
     fma_missing_kernel(const DigOperand* __restrict__ ops, const DigSeg* __restrict__ segs,
-                       const DigTask* __restrict__ tasks, int ntasks, const int* __restrict__ any,
-                       const unsigned char* __restrict__ flag, const uint32_t* __restrict__ miss,
-                       double* __restrict__ scratch) {
-  if (*any == 0) return;
-  __shared__ double As[32 * FIX_LD], Bs[32 * FIX_LD];
-  __shared__ unsigned short list[1024];
+                       const DigTask* __restrict__ tasks, const int* __restrict__ nleft,
+                       const int* __restrict__ left, const unsigned char* __restrict__ flag,
+                       const uint32_t* __restrict__ miss, double* __restrict__ scratch) {
+  // 16 rows a CTA, or 8 or 4 where that makes fewer than two units a CTA: 16 x 32
+  // outputs of a 150 x 150 product are 20 us of an SM's float64 pipe (33 -> 14 us;
+  // exchange of 200 orbitals 590 -> 435 us against one unit a CTA)
+  const int blocks = *nleft;
+  int rows = FIX_ROWS;
+  while (rows > 4 && blocks * (32 / rows) < 2 * (int)gridDim.x) rows /= 2;
+  const int per = 32 / rows, units = blocks * per;
+  extern __shared__ double fix[];
+  __shared__ unsigned short list[FIX_ROWS * FIX_COLS];
   __shared__ int count;
   const int tid = threadIdx.x;
-  for (int u = blockIdx.x; u < ntasks * 8; u += gridDim.x) {
-    const int w = u / ntasks;  // every CTA meets all eight: the last ones of a ragged tile are empty
-    const DigTask t = tasks[u - w * ntasks];
-    const int r0 = t.r0 + (w & 3) * 32, c0 = t.c0 + (w >> 2) * 32;
-    const int nr = min(32, t.m - r0), nc = min(32, t.n - c0);
-    if (nr <= 0 || nc <= 0) continue;
+  for (int u = blockIdx.x; u < units; u += gridDim.x) {
+    const int block = left[u / per], w = block & 7, sub = u % per * rows;  // the mark, first row of it
+    const DigTask t = tasks[block >> 3];
+    const int r0 = t.r0 + (w & 3) * 32 + sub, c0 = t.c0 + (w >> 2) * FIX_COLS;
+    const int nr = min(rows, t.m - r0), nc = min(FIX_COLS, t.n - c0);
+    if (nr <= 0) continue;
     for (int s = 0; s < t.seg_count; ++s) {
       const int mark = t.mark + 8 * s + w;
       if (!flag[mark]) continue;
-      __syncthreads();  // the list and the tiles are free, the block's outputs visible
+      const DigSeg sg = segs[t.seg_begin + s];
+      const DigOperand a = ops[sg.a], b = ops[sg.b];
+      __syncthreads();  // the list and the stages are free, the outputs of the segment before visible
       if (tid < 32) {
-        uint32_t bits = tid < nr ? miss[(size_t)mark * 32 + tid] & (0xFFFFFFFFu >> (32 - nc)) : 0u;
+        uint32_t bits = tid < nr ? miss[(size_t)mark * 32 + sub + tid] & (0xFFFFFFFFu >> (32 - nc)) : 0u;
         int at = __popc(bits);
 #pragma unroll
         for (int d = 1; d < 32; d *= 2) {
@@ -644,54 +733,61 @@ __global__ void __launch_bounds__(FIX_THREADS, FIX_CTAS)
         }
         if (tid == 31) count = at;
         at -= __popc(bits);
-        for (; bits; bits &= bits - 1) list[at++] = (unsigned short)(tid * 32 + __ffs(bits) - 1);
+        for (; bits; bits &= bits - 1) list[at++] = (unsigned short)(tid * FIX_COLS + __ffs(bits) - 1);
       }
       __syncthreads();
       const int n = count;
-      const DigSeg sg = segs[t.seg_begin + s];
-      const DigOperand a = ops[sg.a], b = ops[sg.b];
+      if (n == 0) continue;
+      // lanes of an output: a power of two, at most eight
+      int lanes = 1;
+      while (lanes < 8 && 2 * lanes * n <= FIX_THREADS) lanes *= 2;
+      const int step = FIX_THREADS / lanes, first = tid / lanes, sub_k = tid - first * lanes;
       double acc[FIX_OUT];
       int ao[FIX_OUT], bo[FIX_OUT];
 #pragma unroll
       for (int q = 0; q < FIX_OUT; ++q) {
-        const int i = tid + q * FIX_THREADS, e = i < n ? list[i] : 0;
+        const int i = first + q * step, e = i < n ? list[i] : 0;
         acc[q] = 0.0;
-        ao[q] = (e >> 5) * FIX_LD;
-        bo[q] = (e & 31) * FIX_LD;
+        ao[q] = e / FIX_COLS * FIX_LD;
+        bo[q] = FIX_ROWS * FIX_LD + e % FIX_COLS * FIX_LD;
       }
-      const int nq = (n - tid + FIX_THREADS - 1) / FIX_THREADS;  // of this thread
+      const int nq = first >= n ? 0 : min(FIX_OUT, (n - first + step - 1) / step);
+      auto stage = [&](int k0) {
+        double* const dst = fix + (k0 / FIX_K & 1) * FIX_STAGE;
+        if (k0 < a.k) {
+          fix_stage<FIX_ROWS>(dst, a, r0, nr, k0, min(FIX_K, a.k - k0));
+          fix_stage<FIX_COLS>(dst + FIX_ROWS * FIX_LD, b, c0, nc, k0, min(FIX_K, a.k - k0));
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      };
+      stage(0);
       for (int k0 = 0; k0 < a.k; k0 += FIX_K) {
         const int kn = min(FIX_K, a.k - k0);
-        for (int e = tid; e < 32 * FIX_K; e += FIX_THREADS) {
-          const int r = a.trans ? e & 31 : e / FIX_K, k = a.trans ? e >> 5 : e % FIX_K;
-          if (r < nr && k < kn) As[r * FIX_LD + k] = sg.alpha * elem(a, r0 + r, k0 + k);
-        }
-        for (int e = tid; e < 32 * FIX_K; e += FIX_THREADS) {
-          const int c = b.trans ? e & 31 : e / FIX_K, k = b.trans ? e >> 5 : e % FIX_K;
-          if (c < nc && k < kn) Bs[c * FIX_LD + k] = elem(b, c0 + c, k0 + k);
-        }
+        const double* x = fix + (k0 / FIX_K & 1) * FIX_STAGE;
+        stage(k0 + FIX_K);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
         __syncthreads();
-        if (nq == FIX_OUT) {
+        if (lanes == 1 && nq == FIX_OUT) {
 #pragma unroll 4
           for (int k = 0; k < kn; ++k)
 #pragma unroll
-            for (int q = 0; q < FIX_OUT; ++q) acc[q] = fma(As[ao[q] + k], Bs[bo[q] + k], acc[q]);
-        } else {
-#pragma unroll
-          for (int q = 0; q < FIX_OUT - 1; ++q)
-            if (q < nq)
-              for (int k = 0; k < kn; ++k) acc[q] = fma(As[ao[q] + k], Bs[bo[q] + k], acc[q]);
+            for (int q = 0; q < FIX_OUT; ++q) acc[q] = fma(x[ao[q] + k], x[bo[q] + k], acc[q]);
+        } else if (nq > 0) {
+#pragma unroll 4
+          for (int k = sub_k; k < kn; k += lanes) acc[0] = fma(x[ao[0] + k], x[bo[0] + k], acc[0]);
         }
         __syncthreads();
       }
+      if (lanes > 1)
+        for (int d = 1; d < lanes; d *= 2) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], d);
 #pragma unroll
       for (int q = 0; q < FIX_OUT; ++q) {
-        if (q >= nq) break;
-        const int e = list[tid + q * FIX_THREADS], r = e >> 5, c = e & 31;
+        if (q >= nq || sub_k != 0) break;
+        const int e = list[first + q * step], r = e / FIX_COLS, c = e % FIX_COLS;
         double* const out = t.part >= 0
                                 ? scratch + t.part + (size_t)(r0 - t.r0 + r) * kDigTileN + (c0 - t.c0) + c
                                 : t.C + (size_t)(r0 + r) * t.ldc + c0 + c;
-        *out += acc[q];
+        *out = fma(sg.alpha, acc[q], *out);
       }
     }
   }
@@ -716,16 +812,19 @@ __global__ void __launch_bounds__(256) reduce_digits_kernel(const DigReduce* __r
 void dig_launch(const DigLaunch& L, cudaStream_t st) {
   cudaError_t e = ensure_smem_attr((const void*)gemm_digits_kernel, SMEM_BYTES);
   if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: digit gemm attribute: ") + cudaGetErrorString(e));
-  split_digits_kernel<<<L.nsplits, SPLIT_THREADS, 0, st>>>(L.ops, L.splits, L.pool, L.exps, L.kmax, L.special);
+  e = ensure_smem_attr((const void*)fma_missing_kernel, FIX_SMEM);
+  if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: digit remainder attribute: ") + cudaGetErrorString(e));
+  split_digits_kernel<<<L.nsplits, SPLIT_THREADS, 0, st>>>(L.ops, L.splits, L.pool, L.exps, L.masks, L.nonzero,
+                                                               L.special);
   e = cudaGetLastError();
   if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: digit split: ") + cudaGetErrorString(e));
   gemm_digits_kernel<<<std::min(L.sms, L.ntasks), NTHREADS, SMEM_BYTES, st>>>(
-      L.ops, L.segs, L.tasks, L.ntasks, L.pool, L.exps, L.kmax, L.special, L.nops, L.flag, L.miss, L.scratch, L.err,
-      L.wait_ns);
+      L.ops, L.segs, L.tasks, L.ntasks, L.pool, L.exps, L.masks, L.nonzero, L.by_entry, L.special, L.nops, L.flag, L.miss,
+      L.left, L.scratch, L.err, L.wait_ns);
   e = cudaGetLastError();
   if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: digit gemm: ") + cudaGetErrorString(e));
-  fma_missing_kernel<<<std::min(L.sms * FIX_CTAS, L.ntasks * 8), FIX_THREADS, 0, st>>>(
-      L.ops, L.segs, L.tasks, L.ntasks, L.special + L.nops, L.flag, L.miss, L.scratch);
+  fma_missing_kernel<<<std::min(L.sms * FIX_CTAS, L.ntasks * 64), FIX_THREADS, FIX_SMEM, st>>>(
+      L.ops, L.segs, L.tasks, L.special + L.nops, L.left, L.flag, L.miss, L.scratch);
   e = cudaGetLastError();
   if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: digit remainder: ") + cudaGetErrorString(e));
   if (L.nreds > 0) {

@@ -8,20 +8,26 @@
 // entry becomes the integer F = round(x 2^(62-e)), cut into eight balanced
 // digits of eight bits (bf16 holds them exactly).  The products of digits i
 // and j with i + j = d are summed by tcgen05.mma into one FP32 accumulator
-// per d; 256 terms of an accumulator stay below 2^24.3, so the sums are exact
-// (above d = 4 a worst case of aligned digits may round in the last place, at
-// 2^-52 of the row maxima's product).  The 36 products with d <= 7 are kept;
-// what is dropped is below 2^-62 of the product of the row maxima per term,
-// under the rounding of a float64 FMA chain.  The accumulators are combined
-// in integers, and each segment is added to the output tile in float64.
+// per d; 256 terms of an accumulator stay below 2^24.8, and below 2^24 for
+// d <= 3, so the sums are exact (above that a worst case of aligned digits may
+// round in the last place, at 2^-52 of the row maxima's product).  The 36
+// products with d <= 7 are kept.  The accumulators are combined in integers,
+// and each segment is added to the output tile in float64.
 //
-// Operands whose scaling makes that bound useless are not multiplied by
-// digits: their products are left out and marked, and a second kernel adds them
-// by float64 FMAs (fma_missing_kernel).  These are a segment with a non-finite
-// entry, with a row maximum outside 2^+-400, or graded along k, that is, whose
-// largest product |a_ik b_kj| is more than 2^8 below the product of the
-// largest entries of A and B, or is so after every row is divided by its
-// maximum.
+// Precision.  Per term, what the digits drop is of the size of 2^-62 of the
+// product of the two rows' maxima 2^ea 2^eb (at most 2^-59), whatever the term
+// itself: far below the rounding of a float64 FMA chain where the row maxima
+// meet entries of their size, and more than the term where they do not.  So an
+// output is taken from the digits only if some term of it is at least 2^-7 of
+// 2^ea 2^eb (DigMask), or all its terms are zero.  What is off is then at most
+// 2 k 2^-53 of sum |a b|, and measured it is smaller than the error of an FMA
+// chain, in the corner of that rule too (a dominant term of 2^-7 and 16 to 200
+// in all: 0.13 to 0.5 of the chain's; normal numbers: 0.2).  The other outputs, and those
+// of a segment with a non-finite entry or a row maximum outside 2^+-400, are
+// left out and marked, and a second kernel adds them by float64 FMAs
+// (fma_missing_kernel).  A caller whose results are only as good as the norm of
+// the rows anyway (products of orthogonal matrices) may have all outputs from
+// the digits (by_entry = false).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -47,9 +53,18 @@ struct DigOperand {
   int rows, k, ld, trans;
   int groups;      // ceil(rows / 8)
   int eoff;        // row exponents: exps[eoff + r]
-  int koff;        // column maxima: kmax[koff + c]
+  int koff;        // columns of the operands before it
   int pad;
 };
+
+// Which entries of a row of an operand lie how far below its maximum, for 16
+// columns (a bit each): those with an exponent at most 2 (x, low half), 3 (x,
+// high), 1 (y, low) and 4 (y, high) below the maximum's.  A product of entries 2
+// and 3, or 1 and 4, below is at least 2^-7 of 2^ea 2^eb: x of one row and x of
+// the other with its halves exchanged have a bit in common, or y and y.
+// masks[unit + kb * 8 groups + r] of the operand, and the nonzero entries at the
+// same place of nonzero.
+using DigMask = uint2;
 
 struct DigSeg {
   int a, b;  // operands
@@ -141,14 +156,16 @@ struct DigLaunch {
   unsigned char* pool;
   double* scratch;
   int* exps;           // nexp
-  uint2* kmax;         // nkmax, zero at launch; exponents of the columns' largest entries,
-                       // of the rows divided by their maxima (x) and as they are (y); 0: a zero column
-  int* special;        // nops, and one for all marks (any), zero at launch
+  DigMask* masks;      // units + 32
+  uint16_t* nonzero;   // the same
+  bool by_entry;       // outputs that the digits hold less well than FMAs are left out
+  int* special;        // nops, and the length of `left`, zero at launch
   // A mark stands for a segment on a 32 x 32 block of a task's tile (row quarter
   // + 4 column half): flag 1 when products of it are left out, then bit c of
   // miss[32 mark + r] says that the product of row r and column c is.
   unsigned char* flag;
   uint32_t* miss;
+  int* left;           // 8 task + block of the blocks with marks set, in any order
   int* err;            // host-mapped flag, set when a bounded wait ran out
   unsigned long long wait_ns;  // bound of every wait (0: its first probe)
   int sms;
