@@ -3,15 +3,17 @@
 // Kernels:
 //   place_kernel        C += sum_s alpha_s op(S_s)            (HBM-bound block copies)
 //   gemm_f64_kernel     C += sum_s alpha_s op(A_s) op(B_s)    (FP64 on the FMA pipe: small blocks)
-//   gemm_digits_kernel (gemm_digits.cu)                        (FP64 as exact bf16 digit products on tcgen05)
+//   gemm_digits_kernel (gemm_digits.cu)                        (FP64 as exact bf16 digit products on tcgen05;
+//                       fma_missing_kernel adds what the digits hold less well than FMAs)
 //   gemm_tf32x3 (gemm_split.cu)                                (split-FP32 tensor-core path)
 //   dots/combine/axpby  vector algebra (FP64, deterministic two-stage reductions); davidson.cu has the
 //                       fused steps of an iteration
 //   eigh.cu             batched FP64 eigensolver: Jacobi for small matrices, tridiagonalisation on groups of
 //                       CTAs and divide and conquer for larger ones
-// All kernels are bounded loops over their inputs; the one wait on other CTAs,
-// the group barrier of the tridiagonalisation, gives up after the backend's
-// wait bound (2 s by default) and sets the error flag.
+// All kernels are bounded loops over their inputs.  What waits gives up after
+// the backend's wait bound (2 s by default) and sets an error flag: the CTA
+// groups of the tridiagonalisation for one another, the roles of a CTA of the
+// digit GEMM and (within its cluster) of the tcgen05 contraction.
 #include <cuda_runtime.h>
 
 #include <algorithm>

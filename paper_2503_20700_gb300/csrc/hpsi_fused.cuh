@@ -4,10 +4,11 @@
 //
 // with A_i a left-block operator sector block (m_a' x m_a, or the identity),
 // P_i the psi block (m_a x m_b) and B_i a right-block operator sector block
-// (m_b' x m_b, or the identity).  One CTA owns one 64 x 64 tile of one sigma
-// block and a chunk of its items; for every item and every 64-wide column
-// chunk of psi it forms X = alpha A P(:, chunk) on chip and accumulates
-// X B(:, chunk)^T, so the intermediate never reaches HBM.  Chunks of items of
+// (m_b' x m_b, or the identity).  One CTA owns one tile of one sigma block (64 x
+// 64; FP64: up to 1024 outputs, shaped to the block, in a last resort all rows of
+// a column tile) and a chunk of its items; for every item and every column chunk
+// of psi it forms X = alpha A P(:, chunk) on chip and accumulates X B(:, chunk)^T,
+// so the intermediate never reaches HBM.  Chunks of items of
 // the same tile are reduced by a second kernel in a fixed order
 // (deterministic, no atomics).
 #pragma once

@@ -1,6 +1,7 @@
 // Host planning of the batched tridiagonalisation (the density-matrix sectors
 // of a decimation): which matrices share a cooperative launch of one CTA per
-// SM, and how many CTAs each matrix gets.
+// SM, and how many CTAs each matrix gets.  (The names are those of the solver by
+// rotations that it planned for first.)
 #pragma once
 #include <algorithm>
 #include <stdexcept>
@@ -13,8 +14,8 @@ constexpr int kJacSmemN = 112;  // largest matrix that may stay on one CTA
 // Modelled time of an n x n matrix on g CTAs, in SM clocks: n steps of three
 // float64 FMAs per entry of the trailing matrix (n^2 / 3 entries on average,
 // two FMAs a clock), what every CTA repeats (about 4500 clocks) and, in a
-// group, a barrier (about 4000); the group sizes of a batch minimise the
-// slowest matrix.
+// group, the exchange (about 4000: the trip of a published value through L2 and
+// the waits around it); the group sizes of a batch minimise the slowest matrix.
 inline double jac_cost(int n, int g) {
   const double steps = std::max(1, n - 1);
   const double fma = 0.5 * (double)n * n;
