@@ -844,6 +844,7 @@ class CudaBackend : public Backend {
     L.nreds = (int)p.reds.size();
     L.nops = (int)p.ops.size();
     L.pool = (unsigned char*)ws;
+    L.last = L.pool + (size_t)p.units * kDigUnit;
     L.exps = (int*)(ws + ox);
     L.masks = (DigMask*)(ws + ok);
     L.nonzero = (uint16_t*)(ws + onz);

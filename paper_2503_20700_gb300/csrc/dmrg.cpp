@@ -1186,7 +1186,7 @@ void Engine::build_comp_from_normal(const Block& b, OpSet& dst, const std::vecto
         be_->memset0(Y, (size_t)M * N * sizeof(double));
         GemmBuilder gb;
         // the N dimension can be large: split into column panels (which also
-        // bounds the digit pool of one product, 16 B per element of K x panel)
+        // bounds the digit pool of one product, 18 B per element of K x panel)
         const size_t panel = 1 << 16;
         for (size_t c0 = 0; c0 < N; c0 += panel) {
           int nc = (int)std::min(panel, N - c0);

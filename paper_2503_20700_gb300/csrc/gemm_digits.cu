@@ -1,23 +1,23 @@
 // Float64 grouped GEMM by exact digit products on tcgen05 (gemm_digits.cuh).
 //
 // gemm_digits_kernel is persistent (one CTA per SM, tasks dealt longest
-// first).  A k-step of 16 brings the eight digits of 128 rows of op(A) and 64
-// columns of op(B) (48 KB, 16 bulk copies) into one of three stages; digit i
+// first).  A k-step of 16 brings the nine digits of 128 rows of op(A) and 64
+// columns of op(B) (54 KB, 18 bulk copies) into one of three stages; digit i
 // of A meets the digits 0..7-i of B, stacked along N, so one MMA of N = 256
 // covers four digits of B and its output columns are the accumulators
-// i..i+3: 12 MMAs and 1152 tensor clocks a k-step.  The eight accumulators
-// (128 x 64 FP32 each) fill TMEM.
+// i..i+3; digit 8-i of B comes on top of the last accumulator by an MMA of its
+// own (N = 64).  21 MMAs a k-step.  The eight accumulators (128 x 64 FP32 each)
+// fill TMEM.
 //
-// What bounds it: shared memory for long segments (a k-step's 12 MMAs read
-// 120 KB and its copies write 48 KB: 1500 clocks, 1152 on the tensor pipe
-// alone), the float64 pipe for short ones (three operations per output and
-// segment at two a clock and SM, 12300 clocks a tile).  The tile is 128 x 64
-// because eight accumulators of that size are all of TMEM; N = 64 alone would
-// read shared memory at 48 clocks per 32-clock MMA, which the stacked form
-// avoids.  Measured, 601 products of 200 x 200 x 200 (the rotation of 600
-// Cholesky vectors): 0.46 ms (0.52 ms where the right operand decays away from
-// its diagonal and its outputs take longer to test) and 0.16 ms for the split,
-// 15 TFLOP/s of float64; the FMA kernel needs 13 ms (0.74 TFLOP/s, 1.25 nominal
+// What bounds it: shared memory for long segments (a k-step's MMAs read 174 KB
+// and its copies write 54 KB), the float64 pipe for short ones (three operations
+// per output and segment at two a clock and SM, 12300 clocks a tile).  The tile
+// is 128 x 64 because eight accumulators of that size are all of TMEM; N = 64
+// alone would read shared memory at 48 clocks per 32-clock MMA, which the
+// stacked form avoids.  Measured, 152 tiles at once: 1.17 us a k-step (0.96 with
+// eight digits and 12 MMAs).  601 products of 200 x 200 x 200 (the rotation of
+// 600 Cholesky vectors): 0.6 ms (0.46) and 0.18 ms for the split (0.16), 12
+// TFLOP/s of float64; the FMA kernel needs 13 ms (0.74 TFLOP/s, 1.25 nominal
 // peak).
 #include <algorithm>
 #include <stdexcept>
@@ -34,10 +34,10 @@ constexpr int NSTAGE = 3;
 constexpr int A_SLICE = 16 * kDigUnit, B_SLICE = 8 * kDigUnit;  // 128 and 64 rows of one digit
 constexpr int A_BYTES = kDigSlices * A_SLICE, B_BYTES = kDigSlices * B_SLICE;
 constexpr int STAGE = A_BYTES + B_BYTES;
-// per epilogue warp: 32 x 32 outputs, turned from row-per-lane (TMEM) to
+// per epilogue warp: 16 x 32 outputs, turned from row-per-lane (TMEM) to
 // column-per-lane (coalesced C)
 constexpr int TURN_LD = 33;
-constexpr int OFF_TURN = NSTAGE * STAGE, TURN_BYTES = 32 * TURN_LD * 8;
+constexpr int OFF_TURN = NSTAGE * STAGE, TURN_BYTES = 16 * TURN_LD * 8;
 constexpr int SMEM_BYTES = OFF_TURN + 8 * TURN_BYTES + 1024;
 constexpr int CHUNK = 16;  // k-steps of 16 between drains: 256 exact terms
 constexpr int NTHREADS = 384;
@@ -152,16 +152,18 @@ __device__ __forceinline__ void tmem_ld4(uint32_t addr, uint32_t (&v)[4]) {
 __device__ __forceinline__ double elem(const DigOperand& o, int r, int c) {
   return o.trans ? __ldg(o.src + (size_t)c * o.ld + r) : __ldg(o.src + (size_t)r * o.ld + c);
 }
-// the eight bytes of u (digit + 128 each, digit 0 on top) as bf16 pairs: word
-// s of `w` gets digit s of this element in its half `half`
+// byte `byte` of word (digit s + 128) as the digit times 2^-8s
+template <int S>
 __device__ __forceinline__ float digit_float(uint32_t word, int byte) {
-  // 2^23 + byte, minus 2^23 + 128
-  return __uint_as_float(__byte_perm(word, 0x4B000000u, 0x7440 + byte)) - 8388736.0f;
+  // (2^23 + byte) 2^-8s, minus (2^23 + 128) 2^-8s
+  constexpr uint32_t one = 0x4B000000u - ((uint32_t)S << 26);
+  constexpr double weight = 1.0 / (double)(1ull << (8 * (S < 8 ? S : 7))) / (S < 8 ? 1.0 : 256.0);
+  return __uint_as_float(__byte_perm(word, one, 0x7440 + byte)) - (float)(8388736.0 * weight);
 }
 
 // 32 rows of one operand per CTA: row maxima, then the digits.  Bound by the
 // latency of its loads for the matrices of a sweep and by HBM and the integer
-// pipe together for large ones (8 B read twice, 16 B written, some forty
+// pipe together for large ones (8 B read twice, 18 B written, some fifty
 // integer operations per element), so a thread loads the eight columns of its
 // row before it uses the first.  Its eight 16-byte stores, one per digit, fill
 // 512 contiguous bytes each with those of its warp.
@@ -174,6 +176,7 @@ __device__ __forceinline__ void load8(const DigOperand& o, int r, int c0, double
 __global__ void __launch_bounds__(SPLIT_THREADS) split_digits_kernel(const DigOperand* __restrict__ ops,
                                                                      const DigSplit* __restrict__ splits,
                                                                      unsigned char* __restrict__ pool,
+                                                                     unsigned char* __restrict__ last,
                                                                      int* __restrict__ exps,
                                                                      DigMask* __restrict__ masks,
                                                                      uint16_t* __restrict__ nonzero,
@@ -212,7 +215,9 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_digits_kernel(const DigOp
   }
   const int g = (sp.r0 >> 3) + gl;
   const bool stored = g < o.groups;  // rows beyond the operand inside its last group are zero
-  unsigned char* const base = pool + (size_t)o.unit * kDigUnit + (size_t)g * kDigUnit + kc * 128 + (lane & 7) * 16;
+  const size_t at0 = (size_t)g * kDigUnit + kc * 128 + (lane & 7) * 16;
+  unsigned char* const base = pool + (size_t)o.unit * kDigUnit + at0;
+  unsigned char* const base_last = last + (size_t)o.unit / kDigSums * kDigUnit + at0;
   for (int kb = warp >> 1; kb < nkb; kb += KSTEP) {
     const int c0 = kb * 16 + kc * 8;
     double x[8];
@@ -228,23 +233,38 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_digits_kernel(const DigOp
         const unsigned long long bits = (unsigned long long)__double_as_longlong(x[i + q]);
         const int be = (int)((bits >> 52) & 0x7FF);
         unsigned long long m = (bits & 0xFFFFFFFFFFFFFull) | 1ull << 52;
-        const int sh = be - be_row + 9;  // at most 9
-        if (be == 0 || sh < -54) m = 0;
-        else if (sh >= 0) m <<= sh;
-        else m = (m + (1ull << (-sh - 1))) >> -sh;
-        const unsigned long long F = (long long)bits < 0 ? 0ull - m : m;
-        const unsigned long long u = F + 0x8080808080808080ull;
-        const uint32_t uh = (uint32_t)(u >> 32), ul = (uint32_t)u;
-#pragma unroll
-        for (int s = 0; s < 4; ++s) {
-          f[q][s] = digit_float(uh, 3 - s);
-          f[q][4 + s] = digit_float(ul, 3 - s);
+        // F of up to 71 bits: top 2^64 + m
+        const int sh = be - be_row + 17;  // at most 17
+        uint32_t top = 0u;
+        if (be == 0 || sh < -54) {
+          m = 0;
+        } else if (sh >= 0) {
+          top = sh > 11 ? (uint32_t)(m >> (64 - sh)) : 0u;
+          m <<= sh;
+        } else {
+          m = (m + (1ull << (-sh - 1))) >> -sh;
         }
+        if ((long long)bits < 0) {
+          m = 0ull - m;
+          top = ~top + (m == 0ull);
+        }
+        const unsigned long long u = m + 0x8080808080808080ull;  // every digit + 128
+        top += 0x80u + (u < 0x8080808080808080ull);
+        const uint32_t uh = (uint32_t)(u >> 32), ul = (uint32_t)u;
+        f[q][0] = digit_float<0>(top, 0);
+        f[q][1] = digit_float<1>(uh, 3);
+        f[q][2] = digit_float<2>(uh, 2);
+        f[q][3] = digit_float<3>(uh, 1);
+        f[q][4] = digit_float<4>(uh, 0);
+        f[q][5] = digit_float<5>(ul, 3);
+        f[q][6] = digit_float<6>(ul, 2);
+        f[q][7] = digit_float<7>(ul, 1);
+        f[q][8] = digit_float<8>(ul, 0);
         const int down = be_row - be;
-        mk.x |= be && down <= 2 ? 1u << (i + q) : 0u;
-        mk.x |= be && down <= 3 ? 0x10000u << (i + q) : 0u;
-        mk.y |= be && down <= 1 ? 1u << (i + q) : 0u;
-        mk.y |= be && down <= 4 ? 0x10000u << (i + q) : 0u;
+        mk.x |= be && down <= 5 ? 1u << (i + q) : 0u;
+        mk.x |= be && down <= 7 ? 0x10000u << (i + q) : 0u;
+        mk.y |= be && down <= 2 ? 1u << (i + q) : 0u;
+        mk.y |= be && down <= 10 ? 0x10000u << (i + q) : 0u;
         nz |= bits << 1 ? 1u << (i + q) : 0u;
       }
 #pragma unroll
@@ -253,9 +273,11 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_digits_kernel(const DigOp
     }
     if (stored) {
 #pragma unroll
-      for (int s = 0; s < kDigSlices; ++s)
-        *reinterpret_cast<uint4*>(base + ((size_t)kb * kDigSlices + s) * o.groups * kDigUnit) =
+      for (int s = 0; s < kDigSums; ++s)
+        *reinterpret_cast<uint4*>(base + ((size_t)kb * kDigSums + s) * o.groups * kDigUnit) =
             make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+      *reinterpret_cast<uint4*>(base_last + (size_t)kb * o.groups * kDigUnit) =
+          make_uint4(w[kDigSums][0], w[kDigSums][1], w[kDigSums][2], w[kDigSums][3]);
     }
     // the two halves of the 16 columns
     mk.x <<= 8 * kc;
@@ -274,7 +296,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_digits_kernel(const DigOp
 
 // ---------------------------------------------------------------- products
 // Bit c: the output of this lane's row and column c (of `ncol`) is to be left
-// out: no term of it is known to reach 2^-7 of 2^ea 2^eb, and not all are zero.
+// out: no term of it is known to reach 2^-14 of 2^ea 2^eb, and not all are zero.
 // ma, na: this lane's row (has_row: there is one), mb, nb: column 0, at k-block 0.
 // Two k-blocks at a time, for the latency of their loads; they settle a dense
 // operand, and 400 integer operations of a warp stand beside 3000 clocks of the
@@ -335,6 +357,7 @@ __device__ __forceinline__ uint32_t outputs_left(bool has_row, const DigMask* ma
 __global__ void __launch_bounds__(NTHREADS, 1)
     gemm_digits_kernel(const DigOperand* __restrict__ ops, const DigSeg* __restrict__ segs,
                        const DigTask* __restrict__ tasks, int ntasks, const unsigned char* __restrict__ pool,
+                       const unsigned char* __restrict__ last,
                        const int* __restrict__ exps, const DigMask* __restrict__ masks,
                        const uint16_t* __restrict__ nonzero, int by_entry,
                        int* __restrict__ special, int nops, unsigned char* __restrict__ flag,
@@ -385,10 +408,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
     if (warp == 0) {
       // ---------------------------------------------------------- producer
-      // lanes 0..7 copy digit `lane` of the A tile, lanes 8..15 of the B tile
+      // lanes 0..8 copy digit `lane` of the A tile, lanes 9..17 of the B tile
       int q = 0;
       bool ok = true;
-      const int s = lane & 7;
+      const int s = lane < kDigSlices ? lane : lane - kDigSlices;
       for (int t = blockIdx.x; ok && t < ntasks; t += gridDim.x) {
         const int r0 = tasks[t].r0, c0 = tasks[t].c0, sb = tasks[t].seg_begin, sc = tasks[t].seg_count;
         for (int k = sb; ok && k < sb + sc; ++k) {
@@ -396,11 +419,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           const int na = min(16, a.groups - (r0 >> 3)), nb = min(8, b.groups - (c0 >> 3));
           const uint32_t bslice = (uint32_t)((nb + 1) & ~1) * kDigUnit;  // 16-column steps
           const int nkb = (a.k + 15) >> 4;
-          const bool isb = lane >= 8;
+          const bool isb = lane >= kDigSlices, tail = s >= kDigSums;
           const int groups = isb ? b.groups : a.groups;
-          const unsigned char* src =
-              pool + ((isb ? b.unit : a.unit) + (size_t)s * groups + ((isb ? c0 : r0) >> 3)) * kDigUnit;
-          const size_t step = (size_t)kDigSlices * groups * kDigUnit;
+          const long long unit = isb ? b.unit : a.unit;
+          const int g0 = (isb ? c0 : r0) >> 3;
+          const unsigned char* src = tail ? last + ((size_t)unit / kDigSums + g0) * kDigUnit
+                                          : pool + ((size_t)unit + (size_t)s * groups + g0) * kDigUnit;
+          const size_t step = (size_t)(tail ? 1 : kDigSums) * groups * kDigUnit;
           const uint32_t bytes = (uint32_t)(isb ? nb : na) * kDigUnit;
           const uint32_t off = isb ? A_BYTES + s * bslice : s * A_SLICE;
           const uint32_t total = (uint32_t)(na + nb) * kDigSlices * kDigUnit;
@@ -411,7 +436,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             if (!ok) break;
             if (lane == 0) arrive_expect(&bar[B_FULL + st], total);
             __syncwarp();
-            if (lane < 16) bulk_load(sbase + st * STAGE + off, src, bytes, &bar[B_FULL + st]);
+            if (lane < 2 * kDigSlices) bulk_load(sbase + st * STAGE + off, src, bytes, &bar[B_FULL + st]);
             ++q;
           }
         }
@@ -447,17 +472,23 @@ __global__ void __launch_bounds__(NTHREADS, 1)
               for (int i = 0; i < kDigSlices; ++i) {
                 const uint64_t da = desc(sa + i * A_SLICE);
 #pragma unroll
-                for (int j = 0; j < kDigSlices - i; j += 4) {
-                  const int nj = kDigSlices - i - j < 4 ? kDigSlices - i - j : 4;
+                for (int j = 0; j < kDigSums - i; j += 4) {
+                  const int nj = kDigSums - i - j < 4 ? kDigSums - i - j : 4;
                   mma_bf16(tmem + kDigTileN * (i + j), da, desc(sB + j * B_SLICE), idesc(kDigTileN * nj),
                            (fresh && i == 0) ? 0u : 1u);
                 }
+                // d = 8, into the accumulator of d = 7
+                mma_bf16(tmem + kDigTileN * (kDigSums - 1), da, desc(sB + (kDigSums - i) * B_SLICE),
+                         idesc(kDigTileN), 1u);
               }
             } else {
-              for (int i = 0; i < kDigSlices; ++i)
-                for (int j = 0; j < kDigSlices - i; j += wide)
+              for (int i = 0; i < kDigSlices; ++i) {
+                for (int j = 0; j < kDigSums - i; j += wide)
                   mma_bf16(tmem + (uint32_t)(W * (i + j)), desc(sa + i * A_SLICE), desc(sB + j * bslice),
-                           idesc(W * min(wide, kDigSlices - i - j)), (fresh && i == 0) ? 0u : 1u);
+                           idesc(W * min(wide, kDigSums - i - j)), (fresh && i == 0) ? 0u : 1u);
+                mma_bf16(tmem + (uint32_t)(W * (kDigSums - 1)), desc(sa + i * A_SLICE),
+                         desc(sB + (kDigSums - i) * bslice), idesc(W), 1u);
+              }
             }
             commit(&bar[B_EMPTY + st]);
             ++q;
@@ -573,13 +604,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 #pragma unroll
           for (int c = 0; c < NC; c += 4) {
             if (!busy || half * NC + c >= W) break;
-            uint32_t v[kDigSlices][4];
+            uint32_t v[kDigSums][4];
 #pragma unroll
-            for (int d = 0; d < kDigSlices; ++d) tmem_ld4(lanes + (uint32_t)(W * d + half * NC + c), v[d]);
+            for (int d = 0; d < kDigSums; ++d) tmem_ld4(lanes + (uint32_t)(W * d + half * NC + c), v[d]);
             asm volatile("tcgen05.wait::ld.sync.aligned;");
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-              auto S = [&](int d) { return __float2int_rn(__uint_as_float(v[d][i])); };
+              // in units of their weights, 2^-8d
+              auto S = [&](int d) {
+                return __float2int_rn(__uint_as_float(v[d][i]) * __uint_as_float((uint32_t)(127 + 8 * d) << 23));
+              };
               long long lo = (long long)l[c + i] + S(7);
               lo = mad_wide(S(6), 1 << 8, lo);
               lo = mad_wide(S(5), 1 << 16, lo);
@@ -604,12 +638,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           arrive(&bar[B_ME + (q & 1)]);
           continue;
         }
+        double sum[NC];
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          if (c % 16 == 0 && half * NC + c >= W) break;
-          turn[lane * TURN_LD + c] = combined(h[c], l[c]);
-        }
-        __syncwarp();
+        for (int c = 0; c < NC; ++c) sum[c] = c < 16 || half * NC + 16 < W ? combined(h[c], l[c]) : 0.0;
         // bit r: this lane's column of row r is an output of the digits
         uint32_t live = nrow > 0 ? 0xFFFFFFFFu >> (32 - nrow) : 0u;
         if (some) {
@@ -623,15 +654,25 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const int m_rows = m.t.m;
         const int eb = m.eb[half * NC + lane];
 #pragma unroll
-        for (int r = 0; r < 32; ++r) {
-          if (r % 8 == 0 && gr0 + r >= m_rows) break;
-          // times 2^e: the value is zero or in [1, 2^84), |e| <= 872
-          const int e = eb + m.ea[(warp & 3) * 32 + r];
-          const double d = turn[r * TURN_LD + lane];
-          const int hi = __double2hiint(d);
-          if (live >> r & 1u) acc[r] = fma(alpha, __hiloint2double(hi ? hi + (e << 20) : 0, __double2loint(d)), acc[r]);
+        for (int p = 0; p < 2; ++p) {
+          // rows 16 p ... of the block
+          if (lane >> 4 == p) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) turn[(lane & 15) * TURN_LD + c] = sum[c];
+          }
+          __syncwarp();
+#pragma unroll
+          for (int r = 16 * p; r < 16 * p + 16; ++r) {
+            if (r % 8 == 0 && gr0 + r >= m_rows) break;
+            // times 2^e: the value is zero or in [1, 2^84), |e| <= 872
+            const int e = eb + m.ea[(warp & 3) * 32 + r];
+            const double d = turn[(r & 15) * TURN_LD + lane];
+            const int hi = __double2hiint(d);
+            if (live >> r & 1u)
+              acc[r] = fma(alpha, __hiloint2double(hi ? hi + (e << 20) : 0, __double2loint(d)), acc[r]);
+          }
+          __syncwarp();
         }
-        __syncwarp();
         arrive(&bar[B_ME + (q & 1)]);
       }
       if (!ok) break;
@@ -814,12 +855,12 @@ void dig_launch(const DigLaunch& L, cudaStream_t st) {
   if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: digit gemm attribute: ") + cudaGetErrorString(e));
   e = ensure_smem_attr((const void*)fma_missing_kernel, FIX_SMEM);
   if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: digit remainder attribute: ") + cudaGetErrorString(e));
-  split_digits_kernel<<<L.nsplits, SPLIT_THREADS, 0, st>>>(L.ops, L.splits, L.pool, L.exps, L.masks, L.nonzero,
+  split_digits_kernel<<<L.nsplits, SPLIT_THREADS, 0, st>>>(L.ops, L.splits, L.pool, L.last, L.exps, L.masks, L.nonzero,
                                                                L.special);
   e = cudaGetLastError();
   if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: digit split: ") + cudaGetErrorString(e));
   gemm_digits_kernel<<<std::min(L.sms, L.ntasks), NTHREADS, SMEM_BYTES, st>>>(
-      L.ops, L.segs, L.tasks, L.ntasks, L.pool, L.exps, L.masks, L.nonzero, L.by_entry, L.special, L.nops, L.flag, L.miss,
+      L.ops, L.segs, L.tasks, L.ntasks, L.pool, L.last, L.exps, L.masks, L.nonzero, L.by_entry, L.special, L.nops, L.flag, L.miss,
       L.left, L.scratch, L.err, L.wait_ns);
   e = cudaGetLastError();
   if (e != cudaSuccess) throw std::runtime_error(std::string("cuda: digit gemm: ") + cudaGetErrorString(e));

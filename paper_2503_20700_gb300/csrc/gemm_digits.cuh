@@ -5,29 +5,40 @@
 //   C += sum_s alpha_s op_s(A_s) op_s(B_s)
 //
 // Row i of op(A) (column j of op(B)) has one exponent e with |x| < 2^e; every
-// entry becomes the integer F = round(x 2^(62-e)), cut into eight balanced
-// digits of eight bits (bf16 holds them exactly).  The products of digits i
-// and j with i + j = d are summed by tcgen05.mma into one FP32 accumulator
-// per d; 256 terms of an accumulator stay below 2^24.8, and below 2^24 for
-// d <= 3, so the sums are exact (above that a worst case of aligned digits may
-// round in the last place, at 2^-52 of the row maxima's product).  The 36
-// products with d <= 7 are kept.  The accumulators are combined in integers,
-// and each segment is added to the output tile in float64.
+// entry becomes the integer F = round(x 2^(70-e)), cut into nine balanced
+// digits of eight bits, which are stored with their weights 2^-8i (bf16 holds
+// them exactly).  The 45 products of digits i and j with i + j = d <= 8 are
+// summed by tcgen05.mma into FP32 accumulators: one per d up to 6, and one for 7
+// and 8 together (eight are all of TMEM).  256 terms of an accumulator stay below
+// 2^24.6 of its unit, below 2^24 for d <= 3, so the sums up to d = 6 are exact
+// (a worst case of aligned digits may round in the last place above d = 3, at
+// 2^-52 of the row maxima's product and less); the last one carries d = 8 in the
+// bits that it has below its unit, 2^-68 of that product, and is rounded to it.
+// The accumulators are combined in integers, and each segment is added to the
+// output tile in float64.
 //
-// Precision.  Per term, what the digits drop is of the size of 2^-62 of the
-// product of the two rows' maxima 2^ea 2^eb (at most 2^-59), whatever the term
+// Precision.  Per term, what the digits drop is of the size of 2^-69 of the
+// product of the two rows' maxima 2^ea 2^eb (at most 2^-66), whatever the term
 // itself: far below the rounding of a float64 FMA chain where the row maxima
 // meet entries of their size, and more than the term where they do not.  So an
-// output is taken from the digits only if some term of it is at least 2^-7 of
+// output is taken from the digits only if some term of it is at least 2^-14 of
 // 2^ea 2^eb (DigMask), or all its terms are zero.  What is off is then at most
 // 2 k 2^-53 of sum |a b|, and measured it is smaller than the error of an FMA
-// chain, in the corner of that rule too (a dominant term of 2^-7 and 16 to 200
-// in all: 0.13 to 0.5 of the chain's; normal numbers: 0.2).  The other outputs, and those
-// of a segment with a non-finite entry or a row maximum outside 2^+-400, are
-// left out and marked, and a second kernel adds them by float64 FMAs
-// (fma_missing_kernel).  A caller whose results are only as good as the norm of
+// chain, in the corner of that rule too (a dominant term of 2^-14 and 16 to 200
+// in all: 0.1 to 0.4 of the chain's; normal numbers: 0.2).  The other outputs,
+// and those of a segment with a non-finite entry or a row maximum outside
+// 2^+-400, are left out and marked, and a second kernel adds them by float64
+// FMAs (fma_missing_kernel).  A caller whose results are only as good as the norm of
 // the rows anyway (products of orthogonal matrices) may have all outputs from
 // the digits (by_entry = false).
+//
+// Nine digits rather than eight (36 products, rule at 2^-7): a k-step takes a
+// fifth longer, but rotations near the identity and matrices that decay from
+// their diagonal, many of whose outputs eight digits hold less well than FMAs,
+// need the FMA pipe no more.  Measured, the rotation of 600 Cholesky vectors of
+// 200 orbitals by exp(-K), K = 0.01 N(0, 1): 16.4 ms with eight digits and that
+// rule, 1.8 ms with nine (26 ms by FMAs alone); its errors in units of
+// 2^-53 sum |a b| 0.11 (root mean square) against 1.09 by FMAs.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -40,13 +51,15 @@
 namespace dmrg {
 
 constexpr int kDigTileM = 128, kDigTileN = 64;  // output tile of a task
-constexpr int kDigSlices = 8;
+constexpr int kDigSlices = 9;
+constexpr int kDigSums = kDigSlices - 1;  // accumulators; digits laid out together
 constexpr int kDigUnit = 256;  // bytes: 8 rows x 16 columns of one digit
 
 // One operand: rows x k, element (r, c) = trans ? src[c ld + r] : src[r ld + c].
-// Digit s of rows [8g, 8g+8) x columns [16kb, 16kb+16) is unit
-// unit + (kb * 8 + s) * groups + g of the pool: two 8-row x 16-byte core
-// matrices (the canonical no-swizzle K-major layout), k fast.
+// Digit s < 8 of rows [8g, 8g+8) x columns [16kb, 16kb+16) is unit
+// unit + (kb * 8 + s) * groups + g of the pool, digit 8 unit
+// unit / 8 + kb * groups + g of the part behind the others: two 8-row x 16-byte
+// core matrices (the canonical no-swizzle K-major layout), k fast.
 struct DigOperand {
   const double* src;
   long long unit;  // first unit in the pool
@@ -58,9 +71,9 @@ struct DigOperand {
 };
 
 // Which entries of a row of an operand lie how far below its maximum, for 16
-// columns (a bit each): those with an exponent at most 2 (x, low half), 3 (x,
-// high), 1 (y, low) and 4 (y, high) below the maximum's.  A product of entries 2
-// and 3, or 1 and 4, below is at least 2^-7 of 2^ea 2^eb: x of one row and x of
+// columns (a bit each): those with an exponent at most 5 (x, low half), 7 (x,
+// high), 2 (y, low) and 10 (y, high) below the maximum's.  A product of entries 5
+// and 7, or 2 and 10, below is at least 2^-14 of 2^ea 2^eb: x of one row and x of
 // the other with its halves exchanged have a bit in common, or y and y.
 // masks[unit + kb * 8 groups + r] of the operand, and the nonzero entries at the
 // same place of nonzero.
@@ -103,7 +116,7 @@ struct DigPlan {
   long long scratch = 0;  // doubles of partial tiles
   int nexp = 0, nkmax = 0;
   int marks = 0;
-  size_t pool_bytes() const { return (size_t)units * kDigUnit; }
+  size_t pool_bytes() const { return (size_t)units / kDigSums * kDigSlices * kDigUnit; }
 };
 
 // Modelled SM clocks of one group by digit products and by the float64 FMA
@@ -154,6 +167,7 @@ struct DigLaunch {
   const DigReduce* reds;
   int nsplits, ntasks, nreds, nops;
   unsigned char* pool;
+  unsigned char* last;  // the part of the pool with the ninth digits
   double* scratch;
   int* exps;           // nexp
   DigMask* masks;      // units + 32

@@ -9,10 +9,10 @@ namespace dmrg {
 namespace {
 
 // Measured clocks of the kernel: a k-step of a 64-wide tile (bound by shared
-// memory: 12 MMAs read 120 KB, the copies write 48 KB), the epilogue of a
+// memory: 21 MMAs read 174 KB, the copies write 54 KB), the epilogue of a
 // segment behind the next one's k-steps (three float64 operations per output
 // at two a clock), and the drain that no k-step overlaps.
-constexpr double kStepClocks = 1500.0, kSegClocks = 15000.0, kDrainClocks = 5000.0;
+constexpr double kStepClocks = 2400.0, kSegClocks = 15000.0, kDrainClocks = 5000.0;
 // operands of one group beyond this (bytes of digits) stay on the FMA pipe
 constexpr double kMaxPool = 4e9;
 
@@ -33,7 +33,7 @@ DigCost dig_cost(const GemmGroup& g, const GemmSeg* segs) {
     elems += (double)k * (g.m + g.n);
     if (k > kDigMaxK) c.digits_tile = 1e300;
   }
-  if (16.0 * elems > kMaxPool) c.digits_tile = 1e300;
+  if (18.0 * elems > kMaxPool) c.digits_tile = 1e300;
   c.digits = c.digits_tile * ((g.m + kDigTileM - 1) / kDigTileM) * ((g.n + 15) / 16 * 0.25) + 0.6 * elems;
   c.fma = c.fma_tile * ((g.m + 63) / 64) * ((g.n + 63) / 64);
   return c;
@@ -61,7 +61,7 @@ int DigPlanner::operand(const double* p, int rows, int k, int ld, int trans) {
   o.unit = plan.units;
   o.eoff = plan.nexp;
   o.koff = plan.nkmax;
-  plan.units += (long long)((k + 15) / 16) * kDigSlices * o.groups;
+  plan.units += (long long)((k + 15) / 16) * kDigSums * o.groups;
   plan.nexp += rows;
   plan.nkmax += k;
   for (int r = 0; r < rows; r += 32) plan.splits.push_back({(int)plan.ops.size(), r});

@@ -3,14 +3,46 @@ rows: which outputs the digits may give (csrc/gemm_digits.cuh) and how far off
 an output can be.
 
 Bound of an output of k products: 2 k 2^-53 sum |a b| from the digits (what they
-drop is at most 2^-59 2^ea 2^eb a term, and a term of 2^-7 2^ea 2^eb is among
+drop is at most 2^-66 2^ea 2^eb a term, and a term of 2^-14 2^ea 2^eb is among
 them), k 2^-53 sum |a b| from FMAs, and two roundings of the result and of C."""
 from fractions import Fraction
 
 import numpy as np
 import pytest
 
-from test_digit_gemm import _chain, _exact, _product
+from test_digit_gemm import _chain, _exact
+
+
+def _digits(x):
+    """Row exponents e (|x| < 2^e) and the nine balanced digits of
+    F = round(x 2^(70-e)), as the split kernel forms them."""
+    big = np.abs(x).max(axis=1)
+    e = np.where(big > 0, np.frexp(big)[1], 0)
+    F = np.array([[int(abs(Fraction(float(v))) * Fraction(2) ** (70 - int(ei)) + Fraction(1, 2)) * (1 if v >= 0 else -1)
+                   for v in row] for row, ei in zip(x, e)], dtype=object)
+    d = np.zeros((9,) + x.shape, dtype=object)
+    for s in range(8, 0, -1):
+        d[s] = (F + 128) % 256 - 128
+        F = (F - d[s]) // 256
+    d[0] = F
+    return e, d
+
+
+def _product(a, b):
+    """op(A) op(B) by the kernel's arithmetic (a: m x k, b: n x k): the sums of
+    d = 7 and d = 8 share an accumulator and are rounded together."""
+    (ea, da), (eb, db) = _digits(a), _digits(b)
+    v = np.zeros((len(a), len(b)))
+    for i in range(len(a)):
+        for j in range(len(b)):
+            h = 0
+            for k0 in range(0, a.shape[1], 256):
+                s = [sum(int(x) * int(y) for p in range(d + 1)
+                         for x, y in zip(da[p][i, k0:k0 + 256], db[d - p][j, k0:k0 + 256])) for d in range(9)]
+                assert all(abs(x) < 2**25 for x in s)
+                h += round(Fraction(s[7] * 256 + s[8], 256)) + sum(s[d] << 8 * (7 - d) for d in range(7))
+            v[i, j] = np.ldexp(float(h), int(ea[i] + eb[j]) - 68)
+    return v
 
 
 def _from_digits(a, b):
@@ -20,7 +52,7 @@ def _from_digits(a, b):
         return e.max(axis=1, keepdims=True) - e
     da, db = down(a), down(b)
     hit = np.zeros((len(a), len(b)), bool)
-    for u, v in ((2, 3), (3, 2), (1, 4), (4, 1)):
+    for u, v in ((5, 7), (7, 5), (2, 10), (10, 2)):
         hit |= ((da <= u).astype(int) @ (db <= v).T.astype(int)) > 0
     return hit | (((a != 0).astype(int) @ (b != 0).T.astype(int)) == 0)
 
@@ -34,7 +66,7 @@ def _corner(rng, m, k, tail):
     """Row and column maxima meet zeros; one term at the edge of the rule."""
     a, b = (rng.standard_normal((m, k)) * 2.0**-tail for _ in range(2))
     a[:, 0], b[:, 0], a[:, 1], b[:, 1] = 1.9, 0.0, 0.0, 1.9
-    a[:, 2], b[:, 2] = rng.uniform(0.25, 0.26, m), rng.uniform(0.125, 0.13, m)
+    a[:, 2], b[:, 2] = 2.0**-5 * rng.uniform(1, 1.1, m), 2.0**-7 * rng.uniform(1, 1.1, m)
     return a, b
 
 
@@ -46,7 +78,7 @@ def _pairs(kind, rng, m, k):
     if kind == "spread":
         return tuple(rng.standard_normal((m, k)) * 10.0 ** (-6 * rng.random((m, k))) for _ in range(2))
     if kind == "corner":
-        return _corner(rng, m, k, int(rng.integers(4, 25)))
+        return _corner(rng, m, k, int(rng.integers(9, 30)))
     return tuple(rng.standard_normal((m, k)) * (rng.random((m, k)) < 0.1) for _ in range(2))  # sparse
 
 
@@ -133,7 +165,7 @@ def test_one_small_output_beside_large_ones(pkg):
     rng = np.random.default_rng(9)
     A, B = rng.standard_normal((m, k)), rng.standard_normal((k, n))
     A[77], B[:, 21] = 0.0, 0.0
-    A[77, :2], B[1, 21] = (1.0, 1.23e-12), 1.0
+    A[77, :2], B[1, 21] = (1.0, 1.23e-12), 1.0  # 2^-39 of the row's maximum
     C = np.zeros((m, n))
     pkg.ops.grouped_gemm(A.ravel(), B.ravel(), C, [(0, m, n, n, 0, 1)], [(0, 0, k, k, n, 0, 0, 1.0)])
     assert C[77, 21] == 1.23e-12
